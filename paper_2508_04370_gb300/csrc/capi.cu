@@ -111,8 +111,7 @@ struct ipm_ctx {
     int32_t *lperm = nullptr;    // pivoting mode: each front's interchanges (local index at each position)
     double *Ax = nullptr;
     double *theta = nullptr;  // owned copy for host entry points
-    double *vf = nullptr, *vx = nullptr, *vbest = nullptr, *vr = nullptr, *vad = nullptr, *vae = nullptr,
-           *vc = nullptr, *upd = nullptr;
+    double *vf = nullptr, *vx = nullptr, *vbest = nullptr, *vr = nullptr, *vad = nullptr, *vc = nullptr, *upd = nullptr;
     double *h_r7 = nullptr, *h_r1 = nullptr, *d_r7 = nullptr, *d_r1 = nullptr, *d_dx = nullptr, *d_dy = nullptr;
     int32_t *lvl_small = nullptr, *lvl_all = nullptr;
     int32_t *bwd_order = nullptr, *solve_sync = nullptr;
@@ -284,6 +283,17 @@ int dupload(ipm_ctx *c, T **p, const std::vector<T> &h) {
         if (e != cudaSuccess) return to_err(e);
     }
     return IPM_OK;
+}
+
+// The rows of a CSR pointer summed by a CTA each (more than kLongColumn
+// entries) and by a warp each (more than kWarpRow).
+template <typename V>
+void long_rows(const V &ptr, std::vector<int32_t> &lng, std::vector<int32_t> &mid) {
+    for (size_t i = 0; i + 1 < ptr.size(); i++) {
+        const int64_t len = ptr[i + 1] - ptr[i];
+        if (len > kLongColumn) lng.push_back((int32_t)i);
+        else if (len > kWarpRow) mid.push_back((int32_t)i);
+    }
 }
 
 // Items of the persistent level kernel for the large fronts of level l, in
@@ -1139,12 +1149,14 @@ int setup_device(ipm_ctx *c) {
         (rc = dalloc(c, &c->solve_sync, (size_t)3 * ns + 1)))
         return rc;
     c->slice_half_blocks = max_slice_blocks;
-    int32_t *d_sparent, *d_long;
+    int32_t *d_sparent, *d_long, *d_mid;
+    double *d_kval, *d_kabs;
     if ((rc = dupload(c, &d_sparent, P.sn_parent))) return rc;
-    std::vector<int32_t> long_cols;  // columns of K summed by a CTA each in the norm
-    for (int32_t i = 0; i < N; i++)
-        if (kp[i + 1] - kp[i] > kLongColumn) long_cols.push_back(i);
-    if ((rc = dupload(c, &d_long, long_cols))) return rc;
+    std::vector<int32_t> long_cols, mid_cols;  // rows of K summed by a CTA or a warp each
+    long_rows(kp, long_cols, mid_cols);
+    if ((rc = dupload(c, &d_long, long_cols)) || (rc = dupload(c, &d_mid, mid_cols)) ||
+        (rc = dalloc(c, &d_kval, (size_t)kp[N])) || (rc = dalloc(c, &d_kabs, (size_t)N)))
+        return rc;
     {
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
@@ -1196,6 +1208,10 @@ int setup_device(ipm_ctx *c) {
             (rc = dalloc(c, &d_ib, (size_t)P.batch_count)))
             return rc;
         dp.batch_count = P.batch_count;
+    dp.mid_cols = d_mid;
+    dp.nmid = (int32_t)mid_cols.size();
+    dp.kval = d_kval;
+    dp.kabs = d_kabs;
         dp.inst = d_inst;
         dp.inst_norm1 = d_in;
         dp.inst_b1 = d_ib;
@@ -1207,7 +1223,7 @@ int setup_device(ipm_ctx *c) {
         (rc = dalloc(c, &c->dyn, N)) || (rc = dalloc(c, &c->ctl, 1)) || (rc = dalloc(c, &c->Ax, nnzA)) ||
         (rc = dalloc(c, &c->theta, P.n)) ||
         (rc = dalloc(c, &c->vf, N)) || (rc = dalloc(c, &c->vx, N)) || (rc = dalloc(c, &c->vbest, N)) ||
-        (rc = dalloc(c, &c->vr, N)) || (rc = dalloc(c, &c->vad, N)) || (rc = dalloc(c, &c->vae, N)) ||
+        (rc = dalloc(c, &c->vr, N)) || (rc = dalloc(c, &c->vad, N)) ||
         (rc = dalloc(c, &c->vc, N)) || (rc = dalloc(c, &c->upd, (size_t)std::max<int64_t>(P.upd_total, 1))))
         return rc;
     if (c->opt.pivoting &&
@@ -1246,6 +1262,32 @@ int setup_device(ipm_ctx *c) {
         c->ne.Arp = d_arp;
         c->ne.Aci = d_aci;
         c->ne.Apos = d_apos;
+        {
+            // the long sums: entries of M, columns of A, rows of A (by their
+            // position in the factorisation order)
+            std::vector<int32_t> v[6];
+            long_rows(P.ne_tptr, v[0], v[1]);
+            long_rows(acp, v[2], v[3]);
+            long_rows(arp, v[4], v[5]);
+            for (int q = 4; q < 6; q++)
+                for (int32_t &i : v[q]) i = P.iperm[i];
+            int32_t *d[6];
+            for (int q = 0; q < 6; q++)
+                if ((rc = dupload(c, &d[q], v[q]))) return rc;
+            NeView &E = c->ne;
+            E.elong = d[0];
+            E.emid = d[1];
+            E.clong = d[2];
+            E.cmid = d[3];
+            E.rlong = d[4];
+            E.rmid = d[5];
+            E.nelong = (int32_t)v[0].size();
+            E.nemid = (int32_t)v[1].size();
+            E.nclong = (int32_t)v[2].size();
+            E.ncmid = (int32_t)v[3].size();
+            E.nrlong = (int32_t)v[4].size();
+            E.nrmid = (int32_t)v[5].size();
+        }
         c->ne.Acp = d_acp;
         c->ne.Ari = d_ari;
     }
@@ -1253,8 +1295,8 @@ int setup_device(ipm_ctx *c) {
     cudaMemset(c->fronts, 0, (size_t)std::max<int64_t>(P.front_doubles, 1) * sizeof(double));
     c->mixed_active = c->opt.precision != IPM_PREC_FP64;
     c->fallbacks = 0;
-    c->resid_w.flops = 6.0 * (double)kp[N];
-    c->resid_w.bytes = 20.0 * (double)kp[N] + 48.0 * N;
+    c->resid_w.flops = 4.0 * (double)kp[N];
+    c->resid_w.bytes = 12.0 * (double)kp[N] + 48.0 * N;
     c->dev_ready = true;
     return to_err(cudaGetLastError());
 }
@@ -1616,7 +1658,7 @@ int solve_inplace(ipm_ctx *c, double *x, cudaStream_t st, int *nl) {
 // (captured on a second stream) runs only when classical refinement ended
 // above the target; inside it every kernel tests the device-side flags of
 // GmDev, so cycles and Arnoldi steps that are not needed return at entry.
-int capture_gmres(ipm_ctx *c, const DevVals &V, cudaStream_t st) {
+int capture_gmres(ipm_ctx *c, cudaStream_t st) {
     const Plan &P = c->plan;
     const int64_t N = P.N;
     const int m = kGmresM;
@@ -1656,7 +1698,7 @@ int capture_gmres(ipm_ctx *c, const DevVals &V, cudaStream_t st) {
     launch_copy_if(c->vx, c->vbest, (int32_t)N, nullptr, 0, s2);
     for (int r = 0; r <= R; r++) {
         // r = f - K x and omega of the current x; keep it if it improved
-        launch_residual_omega(c->dp, V, c->vf, c->vx, c->vr, c->vad, c->vae, c->ctl, s2, &gm->stop);
+        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, s2, &gm->stop);
         launch_gm_cycle(c->ctl, gm, target, r, R, s2);
         launch_copy_if(c->vbest, c->vx, (int32_t)N, &gm->improved, 0, s2);
         if (r == R) break;
@@ -1670,7 +1712,7 @@ int capture_gmres(ipm_ctx *c, const DevVals &V, cudaStream_t st) {
                                       s2, &gm->skip_inner);
             launch_backward_persistent(c->sched, c->fronts, zj, c->solve_maxf, c->solve_grid, c->ctl, s2,
                                        &gm->skip_inner);
-            launch_residual_omega(c->dp, V, c->gm_zero, zj, c->gm_w, c->vad, c->vae, c->ctl, s2, &gm->skip_inner);
+            launch_residual_omega(c->dp, c->gm_zero, zj, c->gm_w, c->vad, c->ctl, s2, &gm->skip_inner);
             launch_scale_dev(vn, c->gm_w, gm, -1.0, N, &gm->skip_inner, s2);  // K z
             for (int pass = 0; pass < 2; pass++) {
                 launch_dots(vn, c->gm_V, N, j + 1, c->gm_part, gm->h, s2, &gm->skip_inner);
@@ -1706,22 +1748,16 @@ bool gmres_allowed(const ipm_ctx *c) {
 int solve_device_driven(ipm_ctx *c, const double *r7, const double *r1, double *dx, double *dy, cudaStream_t st) {
     const Plan &P = c->plan;
     const int32_t N = P.N;
-    DevVals V{};
-    V.Ax = c->Ax;
-    V.theta = c->theta;
-    V.rho = c->rho;
-    V.delta = c->delta;
     const int32_t *done = &c->ctl->done;
     const int32_t *improved = &c->ctl->improved;
     const double target = c->opt.omega_target;
     const int32_t rmax = c->opt.refine_max;
-    V.nev = c->ne.nev;
     if (P.form == 2) launch_ne_rhs(c->ne, c->dp.perm, c->Ax, r7, r1, c->vf, st);
     else launch_permute_in(c->dp, r7, r1, c->vf, st);
     launch_copy_if(c->vx, c->vf, N, nullptr, 0, st);
     launch_forward_persistent(c->sched, c->fronts, c->Dinv, c->vx, c->upd, c->solve_maxf, c->solve_grid, c->ctl, st);
     launch_backward_persistent(c->sched, c->fronts, c->vx, c->solve_maxf, c->solve_grid, c->ctl, st);
-    launch_residual_omega(c->dp, V, c->vf, c->vx, c->vr, c->vad, c->vae, c->ctl, st);
+    launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
     launch_refine_init(c->ctl, target, rmax, st);
     launch_copy_if(c->vbest, c->vx, N, nullptr, 0, st);
     for (int32_t step = 1; step <= rmax; step++) {
@@ -1730,12 +1766,12 @@ int solve_device_driven(ipm_ctx *c, const double *r7, const double *r1, double *
                                   done);
         launch_backward_persistent(c->sched, c->fronts, c->vc, c->solve_maxf, c->solve_grid, c->ctl, st, done);
         launch_axpy(c->vx, c->vc, N, st, done);
-        launch_residual_omega(c->dp, V, c->vf, c->vx, c->vr, c->vad, c->vae, c->ctl, st, done);
+        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st, done);
         launch_refine_step(c->ctl, target, step, rmax, st);
         launch_copy_if(c->vbest, c->vx, N, improved, 0, st);
     }
     if (c->gm_dev && gmres_allowed(c)) {
-        int rc = capture_gmres(c, V, st);
+        int rc = capture_gmres(c, st);
         if (rc) return rc;
     }
     launch_refine_finish(c->ctl, target, st);
@@ -2158,7 +2194,7 @@ static int gmres_alloc(ipm_ctx *c, cudaStream_t st) {
     return to_err(cudaGetLastError());
 }
 
-static int gmres_refine(ipm_ctx *c, const DevVals &V, cudaStream_t st, double &wbest, int *nl) {
+static int gmres_refine(ipm_ctx *c, cudaStream_t st, double &wbest, int *nl) {
     const Plan &P = c->plan;
     const int64_t N = P.N;
     const int m = kGmresRestart;
@@ -2174,7 +2210,7 @@ static int gmres_refine(ipm_ctx *c, const DevVals &V, cudaStream_t st, double &w
     cudaMemcpyAsync(c->vx, c->vbest, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
     for (int restart = 0; restart <= c->opt.gmres_restarts; restart++) {
         // r = f - K x and omega of the current x
-        launch_residual_omega(c->dp, V, c->vf, c->vx, c->vr, c->vad, c->vae, c->ctl, st);
+        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
         *nl += 2;
         DevCtl h{};
         if ((rc = read_ctl(c, st, &h))) return rc;
@@ -2203,7 +2239,7 @@ static int gmres_refine(ipm_ctx *c, const DevVals &V, cudaStream_t st, double &w
             double *vj = c->gm_V + (int64_t)j * N, *zj = c->gm_Z + (int64_t)j * N, *vn = vj + N;
             cudaMemcpyAsync(zj, vj, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
             if ((rc = solve_inplace(c, zj, st, nl))) return rc;
-            launch_residual_omega(c->dp, V, c->gm_zero, zj, c->gm_w, c->vad, c->vae, c->ctl, st);  // -K z
+            launch_residual_omega(c->dp, c->gm_zero, zj, c->gm_w, c->vad, c->ctl, st);  // -K z
             launch_scale(vn, c->gm_w, -1.0, N, st);
             *nl += 3;
             for (int pass = 0; pass < 2; pass++) {
@@ -2256,12 +2292,6 @@ static int solve_once(ipm_ctx *c, const double *r7, const double *r1, double *dx
     if ((P.n > 0 && (!r7 || !dx)) || (P.m > 0 && (!r1 || !dy))) return IPM_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     const int32_t N = P.N;
-    DevVals V{};
-    V.Ax = c->Ax;
-    V.theta = c->theta;
-    V.rho = c->rho;
-    V.delta = c->delta;
-    V.nev = c->ne.nev;
     int nl = 0;
     if (P.form == 2) launch_ne_rhs(c->ne, c->dp.perm, c->Ax, r7, r1, c->vf, st);  // r8 = r1 + A Theta~ r7
     else launch_permute_in(c->dp, r7, r1, c->vf, st);
@@ -2270,7 +2300,7 @@ static int solve_once(ipm_ctx *c, const double *r7, const double *r1, double *dx
     if ((rc = solve_inplace(c, c->vx, st, &nl))) return rc;
     {
         Prof pr(c, IPM_K_RESIDUAL, c->resid_w, st);
-        launch_residual_omega(c->dp, V, c->vf, c->vx, c->vr, c->vad, c->vae, c->ctl, st);
+        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
     }
     nl += 2;
     DevCtl h{};
@@ -2286,7 +2316,7 @@ static int solve_once(ipm_ctx *c, const double *r7, const double *r1, double *dx
         launch_axpy(c->vx, c->vc, N, st);
         {
             Prof pr(c, IPM_K_RESIDUAL, c->resid_w, st);
-            launch_residual_omega(c->dp, V, c->vf, c->vx, c->vr, c->vad, c->vae, c->ctl, st);
+            launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
         }
         nl += 3;
         if ((rc = read_ctl(c, st, &h))) return rc;
@@ -2304,7 +2334,7 @@ static int solve_once(ipm_ctx *c, const double *r7, const double *r1, double *dx
     // later iterations keep, rather than paying GMRES iterations every solve
     c->gmres_iters = 0;
     if (wbest > target && gmres_allowed(c) && !(h.status & kStatNonFinite)) {
-        if ((rc = gmres_refine(c, V, st, wbest, &nl))) return rc;
+        if ((rc = gmres_refine(c, st, wbest, &nl))) return rc;
         steps += c->gmres_iters;
     }
     launch_permute_out(c->dp, c->vbest, dx, dy, st);
@@ -2315,7 +2345,7 @@ static int solve_once(ipm_ctx *c, const double *r7, const double *r1, double *dx
     if (P.form == 2) {
         // dx = Theta~ (A^T dy - r7); the reported backward error is the one on K
         launch_ne_dx(c->ne, c->Ax, dy, r7, dx, st);
-        launch_residual_K(c->ne, c->Ax, c->theta, c->rho, c->delta, r7, r1, dx, dy, c->kf, c->kr, c->kad, c->kae,
+        launch_residual_K(c->ne, c->dp.perm, c->Ax, c->theta, c->rho, c->delta, r7, r1, dx, dy, c->kf, c->kr, c->kad, c->kae,
                           c->ctl, st);
         launch_omega_only(P.n + P.m, c->kr, c->kad, c->kae, c->kf, c->ctl, st);
         nl += 3;
@@ -2797,17 +2827,12 @@ int ipm_solve_noalloc(ipm_ctx *c, const double *r7, const double *r1, double *dx
     // every vector below is written before it is read within one call, so
     // nothing left by the previous call needs clearing
     double *vf = base, *vx = base + N, *vbest = base + 2 * N, *vr = base + 3 * N, *vad = base + 4 * N,
-           *vae = base + 5 * N, *vc = base + 6 * N, *upd = base + 7 * N;
+           *vc = base + 6 * N, *upd = base + 7 * N;
     cudaStream_t st = (cudaStream_t)stream;
-    DevVals V{};
-    V.Ax = c->Ax;
-    V.theta = c->theta;
-    V.rho = c->rho;
-    V.delta = c->delta;
     launch_permute_in(c->dp, r7, r1, vf, st);
     cudaMemcpyAsync(vx, vf, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
     if ((rc = noalloc_sweeps(c, vx, upd, st))) return rc;
-    launch_residual_omega(c->dp, V, vf, vx, vr, vad, vae, c->ctl, st);
+    launch_residual_omega(c->dp, vf, vx, vr, vad, c->ctl, st);
     DevCtl h{};
     if ((rc = read_ctl(c, st, &h))) return rc;
     double wbest = h.omega;
@@ -2819,7 +2844,7 @@ int ipm_solve_noalloc(ipm_ctx *c, const double *r7, const double *r1, double *dx
         cudaMemcpyAsync(vc, vr, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
         if ((rc = noalloc_sweeps(c, vc, upd, st))) return rc;
         launch_axpy(vx, vc, (int32_t)N, st);
-        launch_residual_omega(c->dp, V, vf, vx, vr, vad, vae, c->ctl, st);
+        launch_residual_omega(c->dp, vf, vx, vr, vad, c->ctl, st);
         if ((rc = read_ctl(c, st, &h))) return rc;
         steps++;
         if (steps < 16) c->omega_hist[steps] = h.omega;

@@ -79,10 +79,13 @@ struct DevPlan {
     const int64_t *kp;
     const int32_t *kj;
     const int64_t *ksrc;
-    // columns of K with more than kLongColumn stored entries (dense rows of A):
-    // summed by a whole CTA each in the norm
-    const int32_t *long_cols;
-    int32_t nlong;
+    // the entries' values and the row sums |K|e of the latest factorisation's
+    // matrix, written with its norm and read by every residual
+    double *kval, *kabs;
+    // rows of K with more than kLongColumn (a CTA each) and more than kWarpRow
+    // (a warp each) stored entries
+    const int32_t *long_cols, *mid_cols;
+    int32_t nlong, nmid;
     // batches of independent problems: instance of each unknown (factorisation
     // order) and, per instance, ||K_b||_1 and eps_piv ||K_b||_1; null otherwise
     int32_t batch_count;
@@ -129,6 +132,11 @@ struct NeView {
     const int32_t *Aci, *Apos;
     const int64_t *Acp;          // A by columns
     const int32_t *Ari;
+    // the sums over more than kLongColumn (a CTA each) and more than kWarpRow
+    // (a warp each) terms: entries of M by contributor pairs, columns of A,
+    // and rows of A (as positions in the factorisation order)
+    const int32_t *elong, *emid, *clong, *cmid, *rlong, *rmid;
+    int32_t nelong, nemid, nclong, ncmid, nrlong, nrmid;
 };
 
 // Dependency-driven solve schedule, built once per pattern.  A supernode
@@ -261,7 +269,8 @@ constexpr int kTrsmItemRowsHost = 32;  // rows of a triangular-solve item of the
 constexpr int kPanelWsHost = 32 * 33 + 32;
 void launch_large_update_strip(const DevPlan &P, double *fronts, const double *D, const TileItem *items,
                                int32_t count, int32_t w, cudaStream_t st);
-constexpr int64_t kLongColumn = 4096;
+constexpr int64_t kLongColumn = 2048;  // longer sums over a sparse row take a CTA each
+constexpr int64_t kWarpRow = 32;       // and longer than this a warp each (rows_common.cuh)
 // thin fronts (k <= nb, f <= kThinMaxF), one CTA per front: list[i] the front,
 // first_asm[i] its first assembly item (one per 32 columns, rows from the
 // block's first column), slots[i] its panel workspace slot
@@ -350,7 +359,7 @@ void launch_ne_form(const NeView &E, const double *Ax, const double *theta, doub
 void launch_ne_rhs(const NeView &E, const int32_t *perm, const double *Ax, const double *r7, const double *r1,
                    double *f, cudaStream_t st);
 void launch_ne_dx(const NeView &E, const double *Ax, const double *dy, const double *r7, double *dx, cudaStream_t st);
-void launch_residual_K(const NeView &E, const double *Ax, const double *theta, double rho, double delta,
+void launch_residual_K(const NeView &E, const int32_t *perm, const double *Ax, const double *theta, double rho, double delta,
                        const double *r7, const double *r1, const double *dx, const double *dy, double *f, double *r,
                        double *ad, double *ae, DevCtl *ctl, cudaStream_t st);
 // backward error from precomputed r, |K||d|, |K|e, f (ctl->dinf set)
@@ -361,8 +370,8 @@ const void *persistent_probe_kernel();
 void launch_permute_in(const DevPlan &P, const double *r7, const double *r1, double *f, cudaStream_t st);
 void launch_permute_out(const DevPlan &P, const double *x, double *dx, double *dy, cudaStream_t st);
 // skip != nullptr: the kernels return at entry while *skip != 0 (graph-captured refinement)
-void launch_residual_omega(const DevPlan &P, const DevVals &V, const double *f, const double *x, double *r,
-                           double *ad, double *ae, DevCtl *ctl, cudaStream_t st, const int32_t *skip = nullptr);
+void launch_residual_omega(const DevPlan &P, const double *f, const double *x, double *r, double *ad, DevCtl *ctl,
+                           cudaStream_t st, const int32_t *skip = nullptr);
 void launch_axpy(double *x, const double *c, int32_t N, cudaStream_t st, const int32_t *skip = nullptr);
 void launch_refine_init(DevCtl *ctl, double target, int32_t max_steps, cudaStream_t st);
 void launch_refine_step(DevCtl *ctl, double target, int32_t step, int32_t max_steps, cudaStream_t st);

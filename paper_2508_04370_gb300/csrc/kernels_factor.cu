@@ -29,6 +29,7 @@
 #include <cstdint>
 
 #include "ipm_dev.h"
+#include "rows_common.cuh"
 #include "sliced_common.cuh"
 
 namespace ipm {
@@ -1018,65 +1019,61 @@ __global__ void __launch_bounds__(kBodyThreads) k_large_level(DevPlan P, DevVals
     }
 }
 
-// ||K||_1 of the regularised augmented matrix (maximum absolute row sum of
-// the symmetric matrix, fixed summation order per row); also checks that
-// Theta is positive and finite.
-// |K_pi| of stored entry p of column i (with the static terms)
-__device__ __forceinline__ double kabs(const DevPlan &P, const DevVals &V, int i, int64_t p, bool &bad) {
+// The entries' values of the regularised matrix (the augmented K with its
+// static terms, or M + delta I), |K|e and ||K||_1 = max_i (|K|e)_i; also checks
+// that Theta is positive and finite.  The residuals of the refinement read the
+// values and the row sums from here instead of forming them again.
+__device__ __forceinline__ double k_entry(const DevPlan &P, const DevVals &V, int i, int64_t p, bool &bad) {
     const int64_t src = P.ksrc[p];
-    double val;
-    if (P.form == 2) val = V.nev[src] + (P.kj[p] == i ? V.delta : 0.0);
-    else if (src >= 0) val = V.Ax[src];
-    else if (src == kDualDiag) val = V.delta;
-    else {
-        const double th = V.theta[-1 - src];
-        if (!(th > 0.0) || !isfinite(th)) bad = true;
-        val = 1.0 / th + V.rho;
-    }
-    return fabs(val);
+    if (P.form == 2) return V.nev[src] + (P.kj[p] == i ? V.delta : 0.0);
+    if (src >= 0) return V.Ax[src];
+    if (src == kDualDiag) return V.delta;
+    const double th = V.theta[-1 - src];
+    if (!(th > 0.0) || !isfinite(th)) bad = true;
+    return -(1.0 / th + V.rho);
 }
 
-// ||K||_1: column sums in entry order, one thread per column; columns longer
-// than kLongColumn are left to k_norm1_long (a thread alone on a dense row of
-// A would take milliseconds)
-__global__ void k_norm1(DevPlan P, DevVals V, DevCtl *ctl) {
+__global__ void __launch_bounds__(rows::kThreads) k_norm1(DevPlan P, DevVals V, DevCtl *ctl) {
+    __shared__ double sh[rows::kThreads / 32][1];
+    const rows::Part w = rows::part(P.nmid, P.nlong);
+    const int lane = threadIdx.x & 31;
     double mx = 0.0;
     bool bad = false;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.N; i += gridDim.x * blockDim.x) {
-        if (P.kp[i + 1] - P.kp[i] > kLongColumn) continue;
-        double sum = 0.0;
-        for (int64_t p = P.kp[i]; p < P.kp[i + 1]; p++) sum += kabs(P, V, i, p, bad);
+    auto put = [&](int i, double sum) {
+        P.kabs[i] = sum;
         mx = fmax(mx, sum);
-        if (P.inst) atomicMax((unsigned long long *)&P.inst_norm1[P.inst[i]], (unsigned long long)__double_as_longlong(sum));
+        if (P.inst)
+            atomicMax((unsigned long long *)&P.inst_norm1[P.inst[i]], (unsigned long long)__double_as_longlong(sum));
+    };
+    auto strided = [&](int i, int t, int nt) {
+        double sum = 0.0;
+        const int64_t p1 = P.kp[i + 1];
+#pragma unroll 4
+        for (int64_t p = P.kp[i] + t; p < p1; p += nt) {
+            const double v = k_entry(P, V, i, p, bad);
+            P.kval[p] = v;
+            sum += fabs(v);
+        }
+        return sum;
+    };
+    if (w.cta >= 0) {
+        const int i = P.long_cols[w.cta];
+        double a[1] = {strided(i, threadIdx.x, rows::kThreads)};
+        rows::cta_add(a, sh);
+        if (threadIdx.x == 0) put(i, a[0]);
+    } else if (w.mid >= 0) {
+        if (w.mid < P.nmid) {
+            const int i = P.mid_cols[w.mid];
+            double a[1] = {strided(i, lane, 32)};
+            rows::warp_add(a);
+            if (lane == 0) put(i, a[0]);
+        }
+    } else {
+        for (int i = w.first; i < P.N; i += w.stride)
+            if (P.kp[i + 1] - P.kp[i] <= kWarpRow) put(i, strided(i, 0, 1));
     }
     mx = warp_max(mx);
-    if ((threadIdx.x & 31) == 0) atomicMax((unsigned long long *)&ctl->norm1, (unsigned long long)__double_as_longlong(mx));
-    if (bad) atomicOr(&ctl->status, kStatNonFinite);
-}
-
-// One long column per CTA: thread t sums the t-th of 256 contiguous runs in
-// entry order, then the runs' sums are added pairwise in a fixed tree (a
-// deterministic order, not the sequential one).
-__global__ void __launch_bounds__(256) k_norm1_long(DevPlan P, DevVals V, DevCtl *ctl) {
-    __shared__ double part[256];
-    const int i = P.long_cols[blockIdx.x];
-    const int64_t p0 = P.kp[i], n = P.kp[i + 1] - p0;
-    const int64_t run = (n + 255) / 256;
-    const int64_t a = p0 + run * threadIdx.x, b = min(a + run, p0 + n);
-    bool bad = false;
-    double sum = 0.0;
-    for (int64_t p = a; p < b; p++) sum += kabs(P, V, i, p, bad);
-    part[threadIdx.x] = sum;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) part[threadIdx.x] += part[threadIdx.x + h];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        atomicMax((unsigned long long *)&ctl->norm1, (unsigned long long)__double_as_longlong(part[0]));
-        if (P.inst)
-            atomicMax((unsigned long long *)&P.inst_norm1[P.inst[i]], (unsigned long long)__double_as_longlong(part[0]));
-    }
+    if (lane == 0) atomicMax((unsigned long long *)&ctl->norm1, (unsigned long long)__double_as_longlong(mx));
     if (bad) atomicOr(&ctl->status, kStatNonFinite);
 }
 
@@ -1482,10 +1479,8 @@ void launch_test_recip(const double *x, double *rcp, double *quo, int64_t n, cud
 }
 
 void launch_norm1(const DevPlan &P, const DevVals &V, DevCtl *ctl, double eps_piv, cudaStream_t st) {
-    const int grid = (P.N + 255) / 256 < 608 ? (P.N + 255) / 256 : 608;
     if (P.inst) cudaMemsetAsync(P.inst_norm1, 0, sizeof(double) * P.batch_count, st);
-    k_norm1<<<grid > 0 ? grid : 1, 256, 0, st>>>(P, V, ctl);
-    if (P.nlong > 0) k_norm1_long<<<P.nlong, 256, 0, st>>>(P, V, ctl);
+    k_norm1<<<rows::grid(P.N, P.nmid, P.nlong), rows::kThreads, 0, st>>>(P, V, ctl);
     k_set_b1<<<P.inst ? (P.batch_count + 255) / 256 : 1, 256, 0, st>>>(P, ctl, eps_piv);
 }
 

@@ -13,6 +13,7 @@
 #include <cstdint>
 
 #include "ipm_dev.h"
+#include "rows_common.cuh"
 
 namespace ipm {
 
@@ -917,86 +918,60 @@ __global__ void k_permute_out(const int32_t *__restrict__ perm, int N, int n, co
     }
 }
 
-// r = f - K x, ad = |K||x|, ae = |K|e in the factorisation order; also the
-// running max of |x| (ctl->dinf, as ordered bits of a non-negative double).
-__global__ void k_residual(DevPlan P, DevVals V, const double *__restrict__ f, const double *__restrict__ x,
-                           double *__restrict__ r, double *__restrict__ ad, double *__restrict__ ae, DevCtl *ctl,
-                           const int32_t *skip) {
+// r = f - K x and ad = |K||x| in the factorisation order, from the entries'
+// values that the factorisation's norm stored (12 bytes per entry, and no
+// division by Theta); also the running max of |x| (ctl->dinf, as ordered bits
+// of a non-negative double).  Two FP64 instructions per entry.
+__global__ void __launch_bounds__(rows::kThreads) k_residual(DevPlan P, const double *__restrict__ f,
+                                                             const double *__restrict__ x, double *__restrict__ r,
+                                                             double *__restrict__ ad, DevCtl *ctl,
+                                                             const int32_t *skip) {
     if (skip && *skip) return;
+    __shared__ double sh[rows::kThreads / 32][2];
+    const rows::Part w = rows::part(P.nmid, P.nlong);
+    const int lane = threadIdx.x & 31;
     double xm = 0.0;
     bool bad = false;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < P.N; i += gridDim.x * blockDim.x) {
-        xm = fmax(xm, fabs(x[i]));
-        if (P.kp[i + 1] - P.kp[i] > kLongColumn) continue;  // k_residual_long
-        double s = 0.0, sa = 0.0, se = 0.0;
-        for (int64_t p = P.kp[i]; p < P.kp[i + 1]; p++) {
-            const int64_t src = P.ksrc[p];
-            double val;
-            if (P.form == 2) val = V.nev[src] + (P.kj[p] == i ? V.delta : 0.0);
-            else if (src >= 0) val = V.Ax[src];
-            else if (src == kDualDiag) val = V.delta;
-            else val = -(1.0 / V.theta[-1 - src] + V.rho);
-            const double xj = x[P.kj[p]];
-            s += val * xj;
-            sa += fabs(val) * fabs(xj);
-            se += fabs(val);
+    auto strided = [&](int i, int t, int nt, double (&a)[2]) {
+        a[0] = a[1] = 0.0;
+        const int64_t p1 = P.kp[i + 1];
+#pragma unroll 4
+        for (int64_t p = P.kp[i] + t; p < p1; p += nt) {
+            const double v = P.kval[p], xj = x[P.kj[p]];
+            a[0] += v * xj;
+            a[1] += fabs(v) * fabs(xj);
         }
-        const double ri = f[i] - s;
+    };
+    auto put = [&](int i, const double (&a)[2]) {
+        const double ri = f[i] - a[0];
         if (!isfinite(ri)) bad = true;
         r[i] = ri;
-        ad[i] = sa;
-        ae[i] = se;
+        ad[i] = a[1];
+        xm = fmax(xm, fabs(x[i]));
+    };
+    double a[2];
+    if (w.cta >= 0) {
+        const int i = P.long_cols[w.cta];
+        strided(i, threadIdx.x, rows::kThreads, a);
+        rows::cta_add(a, sh);
+        if (threadIdx.x == 0) put(i, a);
+    } else if (w.mid >= 0) {
+        if (w.mid < P.nmid) {
+            const int i = P.mid_cols[w.mid];
+            strided(i, lane, 32, a);
+            rows::warp_add(a);
+            if (lane == 0) put(i, a);
+        }
+    } else {
+        for (int i = w.first; i < P.N; i += w.stride) {
+            if (P.kp[i + 1] - P.kp[i] > kWarpRow) continue;
+            strided(i, 0, 1, a);
+            put(i, a);
+        }
     }
     xm = warp_max(xm);
-    if ((threadIdx.x & 31) == 0) atomicMax((unsigned long long *)&ctl->dinf, (unsigned long long)__double_as_longlong(xm));
+    if (lane == 0) atomicMax((unsigned long long *)&ctl->dinf, (unsigned long long)__double_as_longlong(xm));
     if (bad) atomicOr(&ctl->status, kStatNonFinite);
-}
-
-// The rows of K longer than kLongColumn (dense rows of A), one CTA each:
-// thread t sums the t-th of 256 contiguous runs of the row in entry order,
-// the runs' sums are added pairwise in a fixed tree.
-__global__ void __launch_bounds__(256) k_residual_long(DevPlan P, DevVals V, const double *__restrict__ f,
-                                                       const double *__restrict__ x, double *__restrict__ r,
-                                                       double *__restrict__ ad, double *__restrict__ ae, DevCtl *ctl,
-                                                       const int32_t *skip) {
-    if (skip && *skip) return;
-    __shared__ double ps[256], pa[256], pe[256];
-    const int i = P.long_cols[blockIdx.x];
-    const int64_t p0 = P.kp[i], n = P.kp[i + 1] - p0;
-    const int64_t run = (n + 255) / 256;
-    const int64_t a = p0 + run * threadIdx.x, b = min(a + run, p0 + n);
-    double s = 0.0, sa = 0.0, se = 0.0;
-    for (int64_t p = a; p < b; p++) {
-        const int64_t src = P.ksrc[p];
-        double val;
-        if (P.form == 2) val = V.nev[src] + (P.kj[p] == i ? V.delta : 0.0);
-        else if (src >= 0) val = V.Ax[src];
-        else if (src == kDualDiag) val = V.delta;
-        else val = -(1.0 / V.theta[-1 - src] + V.rho);
-        const double xj = x[P.kj[p]];
-        s += val * xj;
-        sa += fabs(val) * fabs(xj);
-        se += fabs(val);
-    }
-    ps[threadIdx.x] = s;
-    pa[threadIdx.x] = sa;
-    pe[threadIdx.x] = se;
-    __syncthreads();
-    for (int h = 128; h > 0; h >>= 1) {
-        if ((int)threadIdx.x < h) {
-            ps[threadIdx.x] += ps[threadIdx.x + h];
-            pa[threadIdx.x] += pa[threadIdx.x + h];
-            pe[threadIdx.x] += pe[threadIdx.x + h];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        const double ri = f[i] - ps[0];
-        if (!isfinite(ri)) atomicOr(&ctl->status, kStatNonFinite);
-        r[i] = ri;
-        ad[i] = pa[0];
-        ae[i] = pe[0];
-    }
 }
 
 // omega = max_i |r_i| / den_i, den_i = (|K||x| + |f|)_i, replaced by
@@ -1154,8 +1129,8 @@ void launch_permute_out(const DevPlan &P, const double *x, double *dx, double *d
     k_permute_out<<<(P.N + 255) / 256, 256, 0, st>>>(P.perm, P.N, P.n, x, dx, dy, P.form);
 }
 
-void launch_residual_omega(const DevPlan &P, const DevVals &V, const double *f, const double *x, double *r,
-                           double *ad, double *ae, DevCtl *ctl, cudaStream_t st, const int32_t *skip) {
+void launch_residual_omega(const DevPlan &P, const double *f, const double *x, double *r, double *ad, DevCtl *ctl,
+                           cudaStream_t st, const int32_t *skip) {
     const int grid = (P.N + 255) / 256 < 608 ? (P.N + 255) / 256 : 608;
     if (!skip) {
         cudaMemsetAsync(&ctl->dinf, 0, sizeof(double), st);
@@ -1163,9 +1138,8 @@ void launch_residual_omega(const DevPlan &P, const DevVals &V, const double *f, 
     } else {
         k_clear_norms<<<1, 1, 0, st>>>(ctl, skip);
     }
-    k_residual<<<grid, 256, 0, st>>>(P, V, f, x, r, ad, ae, ctl, skip);
-    if (P.nlong > 0) k_residual_long<<<P.nlong, 256, 0, st>>>(P, V, f, x, r, ad, ae, ctl, skip);
-    k_omega<<<grid, 256, 0, st>>>(P.N, r, ad, ae, f, ctl, skip);
+    k_residual<<<rows::grid(P.N, P.nmid, P.nlong), rows::kThreads, 0, st>>>(P, f, x, r, ad, ctl, skip);
+    k_omega<<<grid, 256, 0, st>>>(P.N, r, ad, P.kabs, f, ctl, skip);
 }
 
 void launch_omega_only(int32_t N, const double *r, const double *ad, const double *ae, const double *f, DevCtl *ctl,
