@@ -520,6 +520,8 @@ int build_solve_schedule(ipm_ctx *c, const std::vector<int32_t> &fwd_order, cons
     const Plan &P = c->plan;
     const int32_t ns = P.nsuper;
     std::vector<SolveNode> nodes(ns);
+    int64_t nrpart = 0;
+    int32_t single_maxf = 32;  // the widest front that is one forward item
     for (int32_t s = 0; s < ns; s++) {
         SolveNode &nd = nodes[s];
         nd.off = P.sn_off[s];
@@ -535,6 +537,10 @@ int build_solve_schedule(ipm_ctx *c, const std::vector<int32_t> &fwd_order, cons
         nd.nblk = (nd.k + 31) / 32;
         nd.nrect = (nd.f > nd.k && (rect >= kRectSplit || nd.nblk > 1)) ? (nd.f - nd.k + kRectRows - 1) / kRectRows : 0;
         nd.inv = -1;
+        nd.nback = nd.f - nd.k > kBackSplit ? (nd.f - nd.k + kBackRows - 1) / kBackRows : 0;
+        nd.part = nrpart;
+        nrpart += (int64_t)nd.nblk * nd.nback * 32;
+        if (nd.nblk == 1 && nd.nrect == 0) single_maxf = std::max(single_maxf, nd.f);
     }
     // Supernodes whose diagonal blocks the sweeps apply through explicit
     // inverses (computed once per factorisation): every block of a supernode
@@ -621,7 +627,10 @@ int build_solve_schedule(ipm_ctx *c, const std::vector<int32_t> &fwd_order, cons
             if (bleaf.size() % 8 == 0) bwd.push_back({(int32_t)(bleaf.size() / 8 - 1), kLeafGroup});
             continue;
         }
-        for (int32_t b = nodes[s].nblk - 1; b >= 0; b--) bwd.push_back({s, -1 - b});
+        for (int32_t b = nodes[s].nblk - 1; b >= 0; b--) {
+            for (int32_t r = 0; r < nodes[s].nback; r++) bwd.push_back({s, b * nodes[s].nback + r});
+            bwd.push_back({s, -1 - b});
+        }
     }
     if (bleaf.size() % 8) {
         bwd.push_back({(int32_t)(bleaf.size() / 8), kLeafGroup});
@@ -630,11 +639,12 @@ int build_solve_schedule(ipm_ctx *c, const std::vector<int32_t> &fwd_order, cons
     SolveNode *d_nodes;
     int64_t *d_grp, *d_gsrc;
     SolveItem *d_fwd, *d_bwd;
-    double *d_yv;
+    double *d_yv, *d_rpart;
     int32_t *d_fleaf, *d_bleaf;
     int rc;
     if ((rc = dupload(c, &d_nodes, nodes)) || (rc = dupload(c, &d_grp, grp)) || (rc = dupload(c, &d_gsrc, gsrc)) ||
         (rc = dupload(c, &d_fwd, fwd)) || (rc = dupload(c, &d_bwd, bwd)) || (rc = dalloc(c, &d_yv, (size_t)P.N)) ||
+        (rc = dalloc(c, &d_rpart, (size_t)nrpart)) ||
         (rc = dupload(c, &d_fleaf, fleaf)) || (rc = dupload(c, &d_bleaf, bleaf)) ||
         (rc = dupload(c, &c->inv_items, inv_items)) || (rc = dupload(c, &c->pair_items, pair_items)) ||
         (rc = dalloc(c, &c->linv, (size_t)ninv)))
@@ -655,9 +665,13 @@ int build_solve_schedule(ipm_ctx *c, const std::vector<int32_t> &fwd_order, cons
     S.sync = c->solve_sync;
     S.yv = d_yv;
     S.nyv = P.N;
+    S.rpart = d_rpart;
+    S.nrpart = nrpart;
     S.fwd_leaf = d_fleaf;
     S.bwd_leaf = d_bleaf;
     S.Linv = c->linv;
+    c->solve_maxf = single_maxf;
+    c->solve_grid = std::max(1, std::min(std::max(S.nfwd, S.nbwd), c->sms * solve_ctas_per_sm(single_maxf)));
     return IPM_OK;
 }
 
@@ -1118,7 +1132,6 @@ int setup_device(ipm_ctx *c) {
     c->nfronts_thin = (int32_t)thin_list.size();
     std::vector<int64_t> upd_off(P.upd_off.begin(), P.upd_off.end());
     std::vector<int32_t> bwd_order(lvl_all.rbegin(), lvl_all.rend());
-    c->solve_maxf = P.max_f;
     int rc = 0;
     int32_t *d_c0, *d_k, *d_f, *d_ld, *d_rows, *d_cptr, *d_clist, *d_relmap, *d_odst, *d_perm, *d_kj;
     int64_t *d_off, *d_rptr, *d_moff, *d_optr, *d_osrc, *d_uoff, *d_kp, *d_ksrc;
@@ -1158,12 +1171,9 @@ int setup_device(ipm_ctx *c) {
         (rc = dalloc(c, &d_kval, (size_t)kp[N])) || (rc = dalloc(c, &d_kabs, (size_t)N)))
         return rc;
     {
-        int dev = 0, sms = 0, per_sm = 0;
+        int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persistent_probe_kernel(), 256,
-                                                      (size_t)std::max(P.max_f, kRectRows) * sizeof(double));
-        c->solve_grid = std::max(1, std::min(ns, sms * std::max(1, per_sm)));
         int lvl_per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lvl_per_sm, large_level_kernel(), 256, 0);
         c->lvl_grid = sms * std::max(1, lvl_per_sm);
@@ -1198,6 +1208,10 @@ int setup_device(ipm_ctx *c) {
     dp.ksrc = d_ksrc;
     dp.long_cols = d_long;
     dp.nlong = (int32_t)long_cols.size();
+    dp.mid_cols = d_mid;
+    dp.nmid = (int32_t)mid_cols.size();
+    dp.kval = d_kval;
+    dp.kabs = d_kabs;
     dp.batch_count = 0;
     dp.inst = nullptr;
     dp.inst_norm1 = dp.inst_b1 = nullptr;
@@ -1208,10 +1222,6 @@ int setup_device(ipm_ctx *c) {
             (rc = dalloc(c, &d_ib, (size_t)P.batch_count)))
             return rc;
         dp.batch_count = P.batch_count;
-    dp.mid_cols = d_mid;
-    dp.nmid = (int32_t)mid_cols.size();
-    dp.kval = d_kval;
-    dp.kabs = d_kabs;
         dp.inst = d_inst;
         dp.inst_norm1 = d_in;
         dp.inst_b1 = d_ib;
@@ -1252,16 +1262,6 @@ int setup_device(ipm_ctx *c) {
             (rc = dalloc(c, &c->kr, (size_t)n + m)) || (rc = dalloc(c, &c->kad, (size_t)n + m)) ||
             (rc = dalloc(c, &c->kae, (size_t)n + m)))
             return rc;
-        c->ne.n = n;
-        c->ne.m = m;
-        c->ne.nnz = P.ne_cp[N];
-        c->ne.tptr = d_tptr;
-        c->ne.ta = d_ta;
-        c->ne.tb = d_tb;
-        c->ne.tj = d_tj;
-        c->ne.Arp = d_arp;
-        c->ne.Aci = d_aci;
-        c->ne.Apos = d_apos;
         {
             // the long sums: entries of M, columns of A, rows of A (by their
             // position in the factorisation order)
@@ -1288,6 +1288,16 @@ int setup_device(ipm_ctx *c) {
             E.nrlong = (int32_t)v[4].size();
             E.nrmid = (int32_t)v[5].size();
         }
+        c->ne.n = n;
+        c->ne.m = m;
+        c->ne.nnz = P.ne_cp[N];
+        c->ne.tptr = d_tptr;
+        c->ne.ta = d_ta;
+        c->ne.tb = d_tb;
+        c->ne.tj = d_tj;
+        c->ne.Arp = d_arp;
+        c->ne.Aci = d_aci;
+        c->ne.Apos = d_apos;
         c->ne.Acp = d_acp;
         c->ne.Ari = d_ari;
     }
@@ -1648,7 +1658,7 @@ int solve_inplace(ipm_ctx *c, double *x, cudaStream_t st, int *nl) {
     }
     {
         Prof pr(c, IPM_K_BACKWARD, bw, st);
-        launch_backward_persistent(c->sched, c->fronts, x, c->solve_maxf, c->solve_grid, c->ctl, st);
+        launch_backward_persistent(c->sched, c->fronts, x, c->solve_grid, c->ctl, st);
     }
     *nl += 4;  // per sweep: the reset of its counters and chain values, then the sweep
     return to_err(cudaGetLastError());
@@ -1710,7 +1720,7 @@ int capture_gmres(ipm_ctx *c, cudaStream_t st) {
             launch_copy_if(zj, vj, (int32_t)N, &gm->skip_inner, 1, s2);
             launch_forward_persistent(c->sched, c->fronts, c->Dinv, zj, c->upd, c->solve_maxf, c->solve_grid, c->ctl,
                                       s2, &gm->skip_inner);
-            launch_backward_persistent(c->sched, c->fronts, zj, c->solve_maxf, c->solve_grid, c->ctl, s2,
+            launch_backward_persistent(c->sched, c->fronts, zj, c->solve_grid, c->ctl, s2,
                                        &gm->skip_inner);
             launch_residual_omega(c->dp, c->gm_zero, zj, c->gm_w, c->vad, c->ctl, s2, &gm->skip_inner);
             launch_scale_dev(vn, c->gm_w, gm, -1.0, N, &gm->skip_inner, s2);  // K z
@@ -1756,7 +1766,7 @@ int solve_device_driven(ipm_ctx *c, const double *r7, const double *r1, double *
     else launch_permute_in(c->dp, r7, r1, c->vf, st);
     launch_copy_if(c->vx, c->vf, N, nullptr, 0, st);
     launch_forward_persistent(c->sched, c->fronts, c->Dinv, c->vx, c->upd, c->solve_maxf, c->solve_grid, c->ctl, st);
-    launch_backward_persistent(c->sched, c->fronts, c->vx, c->solve_maxf, c->solve_grid, c->ctl, st);
+    launch_backward_persistent(c->sched, c->fronts, c->vx, c->solve_grid, c->ctl, st);
     launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
     launch_refine_init(c->ctl, target, rmax, st);
     launch_copy_if(c->vbest, c->vx, N, nullptr, 0, st);
@@ -1764,7 +1774,7 @@ int solve_device_driven(ipm_ctx *c, const double *r7, const double *r1, double *
         launch_copy_if(c->vc, c->vr, N, done, 1, st);
         launch_forward_persistent(c->sched, c->fronts, c->Dinv, c->vc, c->upd, c->solve_maxf, c->solve_grid, c->ctl, st,
                                   done);
-        launch_backward_persistent(c->sched, c->fronts, c->vc, c->solve_maxf, c->solve_grid, c->ctl, st, done);
+        launch_backward_persistent(c->sched, c->fronts, c->vc, c->solve_grid, c->ctl, st, done);
         launch_axpy(c->vx, c->vc, N, st, done);
         launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st, done);
         launch_refine_step(c->ctl, target, step, rmax, st);

@@ -148,11 +148,15 @@ struct SolveNode {
     int64_t upd;    // offset of its contribution vector
     int64_t rptr;   // first entry in sn_rows and gat_rp
     int64_t inv;    // inverses of its diagonal blocks in SolveSched::Linv, -1: none (layout: block_slot)
+    int64_t part;   // its row chunks' sums in SolveSched::rpart (32 per block and chunk)
     int32_t f, k, ld, c0;
     int32_t parent, nchild, nrect, nblk;  // nblk: items of L11 (32-column blocks; 1 when unsplit)
+    int32_t nback;  // row chunks of L21 in the backward sweep (0: the blocks take all rows themselves)
 };
 struct SolveItem {
-    int32_t s, r;  // r < 0: block -1-r of L11; else row chunk r of L21
+    // r < 0: block -1-r of L11; else forward: row chunk r of L21, backward: row
+    // chunk r % nback of L21 for the columns of block r / nback
+    int32_t s, r;
 };
 struct SolveSched {
     const SolveNode *node;
@@ -167,6 +171,8 @@ struct SolveSched {
     double *yv;              // the values split supernodes' blocks pass along their chain (y forward,
                              // z backward), reset to an unset pattern before each sweep
     int32_t nyv;
+    double *rpart;           // backward sweep: the row chunks' sums, reset like yv
+    int64_t nrpart;
     const int32_t *fwd_leaf, *bwd_leaf;  // leaf groups: 8 childless single-item supernodes with f <= 32
                                          // per ticket (-1 pads), one warp each
     const double *Linv;                  // inverse unit-lower diagonal blocks, column-major 32 x 32
@@ -180,6 +186,11 @@ struct InvItem {
 constexpr int32_t kLeafGroup = INT32_MIN;  // SolveItem.r of a leaf group (s = group index)
 constexpr int kRectRows = 32;
 constexpr int64_t kRectSplit = 8192;  // split when k (f - k) reaches this
+// Backward sweep: a block of 32 columns with more than kBackSplit rows below
+// leaves them to items of kBackRows rows.  A block's 1,400 rows are 45,000 FMAs, 11 us
+// of one SM's FP64 rate on the path from the root; chunks of 256 rows are 2 us.
+constexpr int kBackRows = 256;
+constexpr int kBackSplit = 384;
 
 // Work item of the large-front path.
 struct PanelItem {
@@ -314,8 +325,8 @@ void launch_diag_inverse(const SolveSched &S, const double *fronts, double *Linv
 void launch_forward_persistent(const SolveSched &S, const double *fronts, const double *Dinv, double *x, double *upd,
                                int32_t maxf, int32_t grid, DevCtl *ctl, cudaStream_t st,
                                const int32_t *skip = nullptr);
-void launch_backward_persistent(const SolveSched &S, const double *fronts, double *x, int32_t maxf, int32_t grid,
-                                DevCtl *ctl, cudaStream_t st, const int32_t *skip = nullptr);
+void launch_backward_persistent(const SolveSched &S, const double *fronts, double *x, int32_t grid, DevCtl *ctl,
+                                cudaStream_t st, const int32_t *skip = nullptr);
 // GMRES refinement vectors (kernels_krylov.cu)
 constexpr int kMaxDots = 16;  // vectors per dot-product launch (restart length + 1 at most)
 constexpr int kGmresM = 8;    // GMRES restart length
@@ -365,8 +376,8 @@ void launch_residual_K(const NeView &E, const int32_t *perm, const double *Ax, c
 // backward error from precomputed r, |K||d|, |K|e, f (ctl->dinf set)
 void launch_omega_only(int32_t N, const double *r, const double *ad, const double *ae, const double *f, DevCtl *ctl,
                        cudaStream_t st);
-// kernel used to size the persistent sweeps' grid (occupancy query)
-const void *persistent_probe_kernel();
+// CTAs per SM of the persistent sweeps (maxf: the widest front that is one forward item)
+int32_t solve_ctas_per_sm(int32_t maxf);
 void launch_permute_in(const DevPlan &P, const double *r7, const double *r1, double *f, cudaStream_t st);
 void launch_permute_out(const DevPlan &P, const double *x, double *dx, double *dy, cudaStream_t st);
 // skip != nullptr: the kernels return at entry while *skip != 0 (graph-captured refinement)

@@ -786,12 +786,63 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
     }
 }
 
+// Up to this many rows below, a lane takes a column and a warp an eighth of
+// the rows (at most 128 contiguous bytes per lane): the same FMAs as
+// rect_columns without its reduction, on the chains of the small fronts (64 x 64
+// grid, fronts of about 60 rows: a refined solve 1.28 ms, 1.31 with it).
+constexpr int kBackLanes = 128;
+
+// A w-column block of L (rows contiguous) on its way into L2 while the item
+// still waits for the values it multiplies.
+__device__ __forceinline__ void prefetch_rect(const double *Lr, int ld, int w, int nr) {
+    const int nl = (nr + 15) / 16;  // 128-byte lines per column
+    for (int q = threadIdx.x; q < w * nl; q += kSolveThreads) {
+        const int c = q / nl, t = 16 * (q - c * nl);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(Lr + (int64_t)c * ld + t));
+    }
+}
+
+// Sums over the rows below a block for its w columns: a warp takes four
+// columns (lanes over the rows, so every load is a coalesced 256 bytes, where
+// a lane per column touched 32 lines per load) and the warps that are left
+// over when w <= 16 split the rows.  out[rs][q] receives slice rs of column q
+// (the caller's barrier follows); returns the number of slices.  Bound by the
+// FP64 rate (2 FMAs per clock and SM).  With the chunks of kBackRows rows one
+// IPM iteration of a 10-period staircase (six backward sweeps of 1.67 ms) takes
+// 29.5 ms instead of 36.5.
+__device__ __forceinline__ int rect_columns(const double *Lr, int ld, int w, int nr, const double *zr,
+                                            double (*out)[33]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cgs = w > 16 ? 8 : w > 8 ? 4 : w > 4 ? 2 : 1, nrs = 8 / cgs;
+    const int cg = warp & (cgs - 1), rs = warp / cgs;
+    const double *Lc = Lr + (int64_t)4 * cg * ld;
+    const int wc = w - 4 * cg;
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
+    for (int t = 32 * rs + lane; t < nr; t += 32 * nrs) {
+        const double zt = zr[t];
+#pragma unroll
+        for (int c = 0; c < 4; c++) a[c] += (c < wc ? Lc[(int64_t)c * ld + t] : 0.0) * zt;
+    }
+    // 4 sums over 32 lanes: halving the columns with the lanes takes six adds
+    const bool h = lane & 16;
+    double b0 = h ? a[2] : a[0], b1 = h ? a[3] : a[1];
+    b0 += __shfl_xor_sync(0xffffffffu, h ? a[0] : a[2], 16);
+    b1 += __shfl_xor_sync(0xffffffffu, h ? a[1] : a[3], 16);
+    const bool g = lane & 8;
+    double v = (g ? b1 : b0) + __shfl_xor_sync(0xffffffffu, g ? b0 : b1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 7) == 0) out[rs][4 * cg + (h ? 2 : 0) + (g ? 1 : 0)] = v;
+    return nrs;
+}
+
 __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveSched S, const double *__restrict__ fronts,
                                                                         double *x, DevCtl *ctl, const int32_t *skip) {
-    extern __shared__ double z[];  // [0, 32): the block; [32, 32 + f - k): x of the rows below
+    extern __shared__ double z[];  // [0, 32): the block; [32, 32 + kBackSplit): x of the rows below
     __shared__ double Lb[32 * 33];
     __shared__ double Wb[32 * 33];  // V_b of a multi-block supernode
-    __shared__ double part[8][33];
+    __shared__ double part[8][33], rect[8][33];
     __shared__ double zs[2][32];
     __shared__ SolveItem sh_it;
     __shared__ SolveNode sh_nd;
@@ -811,8 +862,28 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
         const int f = nd.f, k = nd.k, ld = nd.ld, c0 = nd.c0;
         const double *L = fronts + nd.off;
         const int32_t *rows = S.sn_rows + nd.rptr;
-        const int b = -1 - it.r, b0 = 32 * b, w = min(32, k - b0);
         const int nrr = f - k;  // rows below the supernode's columns
+        if (it.r >= 0) {
+            // rows [t0, t1) below for the columns of one block: sum_t L_tq x_t
+            const int b = it.r / nd.nback, t0 = (it.r % nd.nback) * kBackRows, t1 = min(t0 + kBackRows, nrr);
+            const int w = min(32, k - 32 * b);
+            const double *Lr = L + (int64_t)32 * b * ld + k + t0;
+            prefetch_rect(Lr, ld, w, t1 - t0);
+            if (tid == 0) wait_count(&flag[nd.parent], 1, ctl, S.spin_limit);
+            __syncthreads();
+            if (tid < t1 - t0) z[32 + tid] = __ldcg(x + rows[k + t0 + tid]);
+            __syncthreads();
+            const int nrs = rect_columns(Lr, ld, w, t1 - t0, z + 32, rect);
+            __syncthreads();
+            if (warp == 0 && lane < w) {
+                double sum = rect[0][lane];
+                for (int q = 1; q < nrs; q++) sum += rect[q][lane];
+                publish_value(S.rpart + nd.part + 32 * (int64_t)it.r + lane, sum);
+            }
+            __syncthreads();
+            continue;
+        }
+        const int b = -1 - it.r, b0 = 32 * b, w = min(32, k - b0);
         // independent of other items: the diagonal block (or its inverse) and
         // this block's values after the forward sweep
         const bool inv = nd.inv >= 0;
@@ -821,18 +892,31 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
         else stage_diag(Lb, L, ld, b0, w);
         if (pair) stage_inverse(Wb, S.Linv + block_slot(nd, b) + 2048, 32);
         const double xb = (tid < w) ? __ldcg(x + c0 + b0 + tid) : 0.0;
-        if (tid == 0 && nrr > 0) wait_count(&flag[nd.parent], 1, ctl, S.spin_limit);
-        __syncthreads();
-        for (int t = tid; t < nrr; t += kSolveThreads) z[32 + t] = __ldcg(x + rows[k + t]);
-        __syncthreads();
         // z_q = x_q - sum_{i >= k} L_iq x_rows[i] - sum_{later blocks} L_iq z_i:
-        // lane = column q of the block, warp g takes a slice of the rows below
-        // and rows 4g..4g+3 of every later block
+        // the rows below from their chunks' sums (warp g polls chunks g,
+        // g + 8, ...) or here, then lane = column q, warp g rows 4g..4g+3 of
+        // every later block
+        int nrs = 0;
         double acc = 0.0;
-        if (lane < w && nrr > 0) {
-            const int chunk = (nrr + 7) / 8, t0 = warp * chunk, t1 = min(nrr, t0 + chunk);
-            const double *Lc = L + (int64_t)(b0 + lane) * ld + k;
-            for (int t = t0; t < t1; t++) acc += Lc[t] * z[32 + t];
+        if (nd.nback > 0) {
+            double sum = 0.0;
+            for (int q = warp; q < nd.nback; q += kSolveThreads / 32)
+                sum += poll_block(S.rpart + nd.part + 32 * ((int64_t)b * nd.nback + q), w, ctl, S.spin_limit);
+            rect[warp][lane] = sum;
+            nrs = min(nd.nback, kSolveThreads / 32);
+        } else if (nrr > 0) {
+            const double *Lr = L + (int64_t)b0 * ld + k;
+            if (nrr > kBackLanes) prefetch_rect(Lr, ld, w, nrr);
+            if (tid == 0) wait_count(&flag[nd.parent], 1, ctl, S.spin_limit);
+            __syncthreads();
+            for (int t = tid; t < nrr; t += kSolveThreads) z[32 + t] = __ldcg(x + rows[k + t]);
+            __syncthreads();
+            if (nrr > kBackLanes) {
+                nrs = rect_columns(Lr, ld, w, nrr, z + 32, rect);
+            } else if (lane < w) {
+                const int chunk = (nrr + 7) / 8, t0 = warp * chunk, t1 = min(nrr, t0 + chunk);
+                for (int t = t0; t < t1; t++) acc += Lr[(int64_t)lane * ld + t] * z[32 + t];
+            }
         }
         for (int bp = nd.nblk - 1; bp > b + (pair ? 1 : 0); bp--) {
             const int wp = min(32, k - 32 * bp);
@@ -854,6 +938,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
             double sum = part[0][lane];
 #pragma unroll
             for (int q = 1; q < kSolveThreads / 32; q++) sum += part[q][lane];
+            for (int q = 0; q < nrs; q++) sum += rect[q][lane];
             z[lane] = xb - sum;
         }
         __syncthreads();
@@ -884,6 +969,9 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
             }
             if (b == 0) {
                 wait_count(&tcnt[s], nd.nblk - 1, ctl, S.spin_limit);
+                // (with row chunks only their items acquired the parent's flag: take
+                // it here, so that the children see every ancestor's x)
+                if (nd.nback > 0) wait_count(&flag[nd.parent], 1, ctl, S.spin_limit);
                 __threadfence();
                 atomicExch(&flag[s], 1);
             }
@@ -892,11 +980,14 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
 }
 
 // Before a persistent sweep: the ticket and the counters to zero, the block
-// values of the chains to the unset pattern.
-__global__ void k_sweep_reset(int32_t *__restrict__ sync, int32_t ncnt, double *__restrict__ yv, int32_t nyv) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ncnt || i < nyv; i += gridDim.x * blockDim.x) {
+// values of the chains and the row chunks' sums to the unset pattern.
+__global__ void k_sweep_reset(int32_t *__restrict__ sync, int32_t ncnt, double *__restrict__ yv, int32_t nyv,
+                              double *__restrict__ rpart, int64_t nrpart) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncnt || i < nyv || i < nrpart;
+         i += (int64_t)gridDim.x * blockDim.x) {
         if (i < ncnt) sync[i] = 0;
         if (i < nyv) yv[i] = __longlong_as_double((long long)kUnset);
+        if (i < nrpart) rpart[i] = __longlong_as_double((long long)kUnset);
     }
 }
 
@@ -1067,7 +1158,16 @@ void launch_backward(const DevPlan &P, const double *fronts, double *x, const in
     k_backward<<<count, kSolveThreads, (size_t)maxf * sizeof(double), st>>>(P, fronts, x, list);
 }
 
-const void *persistent_probe_kernel() { return (const void *)k_forward_persistent; }
+constexpr size_t kBackSmem = (32 + kBackSplit) * sizeof(double);
+
+int32_t solve_ctas_per_sm(int32_t maxf) {
+    int f = 0, b = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f, k_forward_persistent, kSolveThreads,
+                                                  (size_t)(maxf > kRectRows ? maxf : kRectRows) * sizeof(double));
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_backward_persistent, kSolveThreads, kBackSmem);
+    const int n = f < b ? f : b;
+    return n > 1 ? n : 1;
+}
 
 void launch_diag_inverse(const SolveSched &S, const double *fronts, double *Linv, const InvItem *items,
                          int32_t count, const InvItem *pairs, int32_t npairs, cudaStream_t st) {
@@ -1095,30 +1195,27 @@ void launch_backward_bk(const DevPlan &P, const double *fronts, const int32_t *l
     k_backward_bk<<<count, kSolveThreads, (size_t)maxf * sizeof(double), st>>>(P, fronts, lperm, x, list);
 }
 
-void launch_sweep_reset(const SolveSched &S, int32_t ncnt, cudaStream_t st) {
-    const int grid = (S.nyv + 255) / 256 < 304 ? (S.nyv + 255) / 256 : 304;
-    k_sweep_reset<<<grid > 0 ? grid : 1, 256, 0, st>>>(S.sync, ncnt, S.yv, S.nyv);
+void launch_sweep_reset(const SolveSched &S, int32_t ncnt, int64_t nrpart, cudaStream_t st) {
+    const int64_t n = S.nyv > nrpart ? S.nyv : nrpart, grid = (n + 255) / 256 < 304 ? (n + 255) / 256 : 304;
+    k_sweep_reset<<<grid > 0 ? (int)grid : 1, 256, 0, st>>>(S.sync, ncnt, S.yv, S.nyv, S.rpart, nrpart);
 }
 
 void launch_forward_persistent(const SolveSched &S, const double *fronts, const double *Dinv, double *x, double *upd,
                                int32_t maxf, int32_t grid, DevCtl *ctl, cudaStream_t st, const int32_t *skip) {
     static uint64_t attr = 0;
-    if (first_on_device(attr)) {
+    if (first_on_device(attr))
         cudaFuncSetAttribute(k_forward_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmemLimit);
-        cudaFuncSetAttribute(k_backward_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmemLimit);
-    }
     // sync[0] = ticket; then per supernode: finished children, finished items
-    launch_sweep_reset(S, 2 * S.nsuper + 1, st);
+    launch_sweep_reset(S, 2 * S.nsuper + 1, 0, st);
     const size_t smem = (size_t)(maxf > kRectRows ? maxf : kRectRows) * sizeof(double);
     k_forward_persistent<<<grid, kSolveThreads, smem, st>>>(S, fronts, Dinv, x, upd, ctl, skip);
 }
 
-void launch_backward_persistent(const SolveSched &S, const double *fronts, double *x, int32_t maxf, int32_t grid,
-                                DevCtl *ctl, cudaStream_t st, const int32_t *skip) {
+void launch_backward_persistent(const SolveSched &S, const double *fronts, double *x, int32_t grid, DevCtl *ctl,
+                                cudaStream_t st, const int32_t *skip) {
     // sync[0] = ticket; then per supernode: done flag, finished blocks
-    launch_sweep_reset(S, 2 * S.nsuper + 1, st);
-    const size_t smem = (size_t)(maxf + 32) * sizeof(double);
-    k_backward_persistent<<<grid, kSolveThreads, smem, st>>>(S, fronts, x, ctl, skip);
+    launch_sweep_reset(S, 2 * S.nsuper + 1, S.nrpart, st);
+    k_backward_persistent<<<grid, kSolveThreads, kBackSmem, st>>>(S, fronts, x, ctl, skip);
 }
 
 void launch_permute_in(const DevPlan &P, const double *r7, const double *r1, double *f, cudaStream_t st) {
