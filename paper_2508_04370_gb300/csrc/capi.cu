@@ -117,9 +117,8 @@ struct ipm_ctx {
     int32_t *bwd_order = nullptr, *solve_sync = nullptr;
     SolveSched sched{};  // dependency-driven solve schedule (device pointers)
     int32_t solve_maxf = 0, solve_grid = 0;
-    PanelItem *asm_items = nullptr, *panel_items = nullptr, *trsm_items = nullptr;
-    AsmItem *asm_info = nullptr;
-    int32_t *asm_cr = nullptr;
+    PanelItem *panel_items = nullptr, *trsm_items = nullptr;
+    AsmLists al{};  // assembly items of the large fronts and their terms
     int32_t *trsm_slots = nullptr;
     int32_t *trsm_sbase = nullptr;     // sliced path: first slice block of each TRSM item's front (-1: none)
     int32_t *thin_list = nullptr, *thin_asm = nullptr, *thin_slot = nullptr;  // thin fronts by level
@@ -341,8 +340,8 @@ void build_level_items(const Plan &P, int32_t l, LevelWork &W, const std::vector
     int64_t ai = W.asm_off;
     for (int32_t q = t0; q < t1; q++) {
         const int32_t s = P.lvl_large[q];
-        for (int32_t cl = 0; cl < P.sn_f[s]; cl += B) {
-            FactorItem it = item(kItemAssemble, s, 0, cl, std::min(cl + B, P.sn_f[s]), (int32_t)ai++);
+        for (int32_t u = 0; u < asm_tiles(P.sn_f[s]); u++) {
+            FactorItem it = item(kItemAssemble, s, 0, 0, 0, (int32_t)ai++);
             it.sig = cbase[s];
             it.add = 1;
             items.push_back(it);
@@ -415,7 +414,7 @@ void build_level_items(const Plan &P, int32_t l, LevelWork &W, const std::vector
                 FactorItem it = item(kItemDiag, s, t, 0, 0, slot_of[s]);
                 if (t == 0) {
                     it.wait0 = cbase[s];
-                    it.need0 = (P.sn_f[s] + B - 1) / B;
+                    it.need0 = asm_tiles(P.sn_f[s]);
                 } else {
                     it.wait0 = tidx(s, t, t);
                     it.need0 = 8 * t;
@@ -751,9 +750,12 @@ int setup_device(ipm_ctx *c) {
     }
     // per-level lists
     std::vector<int32_t> lvl_all, small_lists;
-    std::vector<PanelItem> asm_items, panel_items, trsm_items;
-    std::vector<AsmItem> asm_info;
-    std::vector<int32_t> asm_cr;
+    std::vector<PanelItem> panel_items, trsm_items;
+    std::vector<AsmItem> asm_items;
+    std::vector<AsmChild> asm_child;
+    std::vector<int32_t> seg_dst, asm_rt;
+    std::vector<int64_t> seg_ptr(1, 0), seg_src;
+    std::vector<int64_t> first_item(P.nsuper, -1);  // a front's assembly items in asm_items
     std::vector<int32_t> trsm_slots, trsm_sbase, slot_of(P.nsuper, -1);
     std::vector<int32_t> thin_list, thin_asm, thin_slot;
     int32_t nslots = 0;
@@ -781,28 +783,82 @@ int setup_device(ipm_ctx *c) {
         }
         return fr;
     };
-    // One assembly item: columns [cl, ce), rows [rlo, rhi) of large front s;
-    // its original entries (those of the columns) and, per child, the
-    // contribution-block columns and rows that land in it.
-    auto add_asm = [&](int32_t s, int32_t cl, int32_t ce, int32_t rlo, int32_t rhi) {
-        const int32_t ld = P.sn_ld[s];
-        asm_items.push_back({s, cl, ce, 0});
-        const int32_t *d0 = P.orig_dst.data() + P.orig_ptr[s], *d1 = P.orig_dst.data() + P.orig_ptr[s + 1];
-        AsmItem ai;
-        ai.o0 = std::lower_bound(d0, d1, (int64_t)cl * ld) - P.orig_dst.data();
-        ai.o1 = std::lower_bound(d0, d1, (int64_t)ce * ld) - P.orig_dst.data();
-        ai.cr = (int64_t)(asm_cr.size() / 4);
-        ai.r_lo = rlo;
-        ai.r_hi = rhi;
-        for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
-            const int32_t ch = P.child_list[q];
-            const int32_t *m0 = P.relmap.data() + P.map_off[ch], *m1 = m0 + (P.sn_f[ch] - P.sn_k[ch]);
-            asm_cr.push_back((int32_t)(std::lower_bound(m0, m1, cl) - m0));
-            asm_cr.push_back((int32_t)(std::lower_bound(m0, m1, ce) - m0));
-            asm_cr.push_back((int32_t)(std::lower_bound(m0, m1, rlo) - m0));
-            asm_cr.push_back((int32_t)(std::lower_bound(m0, m1, rhi) - m0));
+    // The assembly items of large front s, one per 32 columns x kAsmRows rows of
+    // its lower part, appended to asm_items (the terms' lists are built once
+    // per front; a front's items may be appended again).
+    std::vector<std::vector<std::pair<int32_t, int64_t>>> points;  // per item: destination, arena position
+    std::vector<std::vector<AsmChild>> block_child;                // per column block
+    auto add_asm = [&](int32_t s) {
+        const int32_t ld = P.sn_ld[s], f = P.sn_f[s], ntile = asm_tiles(f), nblk = (f + 31) / 32;
+        if (first_item[s] >= 0) {
+            for (int32_t t = 0; t < ntile; t++) {
+                const AsmItem ai = asm_items[first_item[s] + t];
+                asm_items.push_back(ai);
+            }
+            return;
         }
-        asm_info.push_back(ai);
+        first_item[s] = (int64_t)asm_items.size();
+        if ((int32_t)points.size() < ntile) points.resize(ntile);
+        if ((int32_t)block_child.size() < nblk) block_child.resize(nblk);
+        std::vector<int32_t> first_tile(nblk);  // item of the block's first rows
+        for (int32_t cb = 0, t = 0; cb < nblk; cb++) {
+            first_tile[cb] = t;
+            t += (f + kAsmRows - 1) / kAsmRows - 32 * cb / kAsmRows;
+        }
+        for (int32_t t = 0; t < ntile; t++) points[t].clear();
+        for (int32_t cb = 0; cb < nblk; cb++) block_child[cb].clear();
+        for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
+            const int32_t ch = P.child_list[q], kc = P.sn_k[ch], cc = P.sn_f[ch] - kc, ldc = P.sn_ld[ch];
+            const int32_t *m = P.relmap.data() + P.map_off[ch];
+            const int64_t cb0 = P.sn_off[ch] + (int64_t)kc * ldc + kc;
+            if (cc <= kPointRows) {
+                for (int32_t jj = 0; jj < cc; jj++)
+                    for (int32_t ii = jj; ii < cc; ii++) {
+                        const int32_t cb = m[jj] / 32, t = first_tile[cb] + m[ii] / kAsmRows - 32 * cb / kAsmRows;
+                        points[t].push_back({kAsmRows * (m[jj] % 32) + m[ii] % kAsmRows, cb0 + (int64_t)jj * ldc + ii});
+                    }
+                continue;
+            }
+            const int32_t rt = (int32_t)asm_rt.size();
+            for (int32_t r = 0; r < f + kAsmRows; r += kAsmRows)
+                asm_rt.push_back((int32_t)(std::lower_bound(m, m + cc, r) - m));
+            for (int32_t a = 0, b; a < cc; a = b) {
+                const int32_t cb = m[a] / 32;
+                for (b = a; b < cc && m[b] / 32 == cb; b++) {}
+                block_child[cb].push_back({cb0, P.map_off[ch], ldc, a, b, rt});
+            }
+        }
+        const int32_t *d0 = P.orig_dst.data() + P.orig_ptr[s], *d1 = P.orig_dst.data() + P.orig_ptr[s + 1];
+        for (int32_t cb = 0, t = 0; cb < nblk; cb++) {
+            AsmItem ai;
+            ai.s = s;
+            ai.c_lo = 32 * cb;
+            ai.c_hi = std::min(32 * cb + 32, f);
+            ai.o0 = std::lower_bound(d0, d1, (int64_t)ai.c_lo * ld) - P.orig_dst.data();
+            ai.o1 = std::lower_bound(d0, d1, (int64_t)ai.c_hi * ld) - P.orig_dst.data();
+            ai.ch0 = (int32_t)asm_child.size();
+            asm_child.insert(asm_child.end(), block_child[cb].begin(), block_child[cb].end());
+            ai.ch1 = (int32_t)asm_child.size();
+            for (int32_t rb = 32 * cb / kAsmRows; rb * kAsmRows < f; rb++, t++) {
+                ai.r_lo = std::max(rb * kAsmRows, ai.c_lo);
+                ai.r_hi = std::min((rb + 1) * kAsmRows, f);
+                std::vector<std::pair<int32_t, int64_t>> &pt = points[t];
+                std::stable_sort(pt.begin(), pt.end(), [](const std::pair<int32_t, int64_t> &x, const std::pair<int32_t, int64_t> &y) {
+                    return x.first < y.first;
+                });
+                ai.seg0 = (int64_t)seg_dst.size();
+                for (size_t u = 0; u < pt.size(); u++) {
+                    if (u == 0 || pt[u].first != pt[u - 1].first) {
+                        if (u > 0) seg_ptr.push_back((int64_t)seg_src.size());
+                        seg_dst.push_back(pt[u].first);
+                    }
+                    seg_src.push_back(pt[u].second);
+                }
+                if (!pt.empty()) seg_ptr.push_back((int64_t)seg_src.size());
+                ai.seg1 = (int64_t)seg_dst.size();
+                asm_items.push_back(ai);
+            }
+        }
     };
     // One step of the large-front path: for each (front s, panel start p0)
     // of fp, the diagonal block of the panel, the triangular solve of the rows
@@ -979,12 +1035,11 @@ int setup_device(ipm_ctx *c) {
         W.asm_off = (int64_t)asm_items.size();
         int32_t maxsteps = 0;
         std::vector<int32_t> main_fronts;
-        std::vector<int64_t> main_first;
         W.thin_off = (int64_t)thin_list.size();
         for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++) {
             const int32_t s = P.lvl_large[t];
             const int64_t first = (int64_t)asm_items.size();
-            for (int32_t cl = 0; cl < P.sn_f[s]; cl += 32) add_asm(s, cl, std::min(cl + 32, P.sn_f[s]), cl, P.sn_f[s]);
+            add_asm(s);
             const bool thin = P.sn_k[s] <= c->opt.nb && P.sn_f[s] <= kThinMaxF &&
                               !(c->opt.precision != IPM_PREC_FP64 && P.sn_f[s] >= c->opt.mixed_min_front);
             if (thin) {
@@ -996,7 +1051,6 @@ int setup_device(ipm_ctx *c) {
                 W.thin_w.bytes += fr.bytes;
             } else {
                 main_fronts.push_back(s);
-                main_first.push_back(first);
                 maxsteps = std::max(maxsteps, (P.sn_k[s] + c->opt.nb - 1) / c->opt.nb);
             }
         }
@@ -1006,12 +1060,7 @@ int setup_device(ipm_ctx *c) {
             // the per-step assembly launch takes the other fronts' items (copies)
             W.asm_off2 = (int64_t)asm_items.size();
             for (size_t q = 0; q < main_fronts.size(); q++)
-                for (int64_t a = main_first[q]; a < main_first[q] + (P.sn_f[main_fronts[q]] + 31) / 32; a++) {
-                    const PanelItem pi = asm_items[a];
-                    const AsmItem ai = asm_info[a];
-                    asm_items.push_back(pi);
-                    asm_info.push_back(ai);
-                }
+                add_asm(main_fronts[q]);
             W.asm_cnt2 = (int32_t)((int64_t)asm_items.size() - W.asm_off2);
         } else {
             W.asm_off2 = W.asm_off;
@@ -1106,11 +1155,7 @@ int setup_device(ipm_ctx *c) {
                 Work aw;
                 int32_t swait = -1;
                 for (int32_t s : starting[g]) {
-                    // one item per 32 columns (splitting the rows too made more,
-                    // shorter CTAs that slowed the trailing tiles beside them more
-                    // than they sped up the assembly)
-                    const int32_t f = P.sn_f[s];
-                    for (int32_t cl = 0; cl < f; cl += 32) add_asm(s, cl, std::min(cl + 32, f), cl, f);
+                    add_asm(s);
                     aw.bytes += front_work(s).bytes;
                     swait = std::max(swait, nsmall_child[s]);
                     active.push_back(s);
@@ -1131,6 +1176,14 @@ int setup_device(ipm_ctx *c) {
     c->steps_levels = steps_levels;
     c->nfronts_thin = (int32_t)thin_list.size();
     std::vector<int64_t> upd_off(P.upd_off.begin(), P.upd_off.end());
+    // children in the order their entries are summed: those the large fronts'
+    // assembly takes as point lists first (the pivoting mode, without that
+    // path, keeps the plain ascending order)
+    std::vector<int32_t> child_order(P.child_list);
+    if (!c->opt.pivoting)
+        for (int32_t s = 0; s < ns; s++)
+            std::stable_partition(child_order.begin() + P.child_ptr[s], child_order.begin() + P.child_ptr[s + 1],
+                                  [&](int32_t ch) { return P.sn_f[ch] - P.sn_k[ch] <= kPointRows; });
     std::vector<int32_t> bwd_order(lvl_all.rbegin(), lvl_all.rend());
     int rc = 0;
     int32_t *d_c0, *d_k, *d_f, *d_ld, *d_rows, *d_cptr, *d_clist, *d_relmap, *d_odst, *d_perm, *d_kj;
@@ -1140,15 +1193,17 @@ int setup_device(ipm_ctx *c) {
     if ((rc = dupload(c, &d_c0, c0)) || (rc = dupload(c, &d_k, P.sn_k)) || (rc = dupload(c, &d_f, P.sn_f)) ||
         (rc = dupload(c, &d_ld, P.sn_ld)) || (rc = dupload(c, &d_off, P.sn_off)) ||
         (rc = dupload(c, &d_rptr, P.sn_rptr)) || (rc = dupload(c, &d_rows, P.sn_rows)) ||
-        (rc = dupload(c, &d_cptr, P.child_ptr)) || (rc = dupload(c, &d_clist, P.child_list)) ||
+        (rc = dupload(c, &d_cptr, P.child_ptr)) || (rc = dupload(c, &d_clist, child_order)) ||
         (rc = dupload(c, &d_moff, P.map_off)) || (rc = dupload(c, &d_relmap, P.relmap)) ||
         (rc = dupload(c, &d_optr, P.orig_ptr)) || (rc = dupload(c, &d_odst, P.orig_dst)) ||
         (rc = dupload(c, &d_osrc, P.orig_src)) || (rc = dupload(c, &d_sign, sign)) ||
         (rc = dupload(c, &d_perm, P.perm)) || (rc = dupload(c, &d_uoff, upd_off)) || (rc = dupload(c, &d_kp, kp)) ||
         (rc = dupload(c, &d_kj, kj)) || (rc = dupload(c, &d_ksrc, ksrc)) ||
         (rc = dupload(c, &c->lvl_small, small_lists)) || (rc = dupload(c, &c->lvl_all, lvl_all)) ||
-        (rc = dupload(c, &c->asm_items, asm_items)) || (rc = dupload(c, &c->asm_info, asm_info)) ||
-        (rc = dupload(c, &c->asm_cr, asm_cr)) || (rc = dupload(c, &c->panel_items, panel_items)) ||
+        (rc = dupload(c, (AsmItem **)&c->al.items, asm_items)) || (rc = dupload(c, (int32_t **)&c->al.seg_dst, seg_dst)) ||
+        (rc = dupload(c, (int64_t **)&c->al.seg_ptr, seg_ptr)) || (rc = dupload(c, (int64_t **)&c->al.src, seg_src)) ||
+        (rc = dupload(c, (AsmChild **)&c->al.child, asm_child)) || (rc = dupload(c, (int32_t **)&c->al.rt, asm_rt)) ||
+        (rc = dupload(c, &c->panel_items, panel_items)) ||
         (rc = dupload(c, &c->trsm_items, trsm_items)) || (rc = dupload(c, &c->trsm_slots, trsm_slots)) ||
         (rc = dalloc(c, &c->panel_ws, (size_t)std::max(nslots, 1) * kPanelWsHost)) ||
         (rc = dupload(c, &c->tile_items, tile_items)) || (rc = dupload(c, &c->tc_items, tc_items)) ||
@@ -1545,8 +1600,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             if (S.small_wait >= 0) cudaStreamWaitEvent(sd, c->dep_ev[4 + 5 * S.small_wait], 0);
             if (S.asm_cnt > 0) {
                 Prof pr(c, IPM_K_LARGE_ASSEMBLE, S.asm_w, sd);
-                launch_large_assemble(c->dp, V, c->fronts, c->asm_items + S.asm_off, c->asm_info + S.asm_off,
-                                      c->asm_cr, S.asm_cnt, sd);
+                launch_large_assemble(c->dp, V, c->fronts, c->al, S.asm_off, S.asm_cnt, sd);
                 nl++;
             }
             emit_step(S);
@@ -1578,7 +1632,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
                 {
                     Prof pr(c, IPM_K_LARGE_PANEL, W.lvl_w, sd);
                     launch_large_level(c->dp, V, c->fronts, c->D, c->Dinv, c->dyn, c->ctl, c->lvl_items + W.lvl_off,
-                                       W.lvl_cnt, c->lvl_sync, W.lvl_ncnt, c->asm_info, c->asm_cr, c->panel_ws,
+                                       W.lvl_cnt, c->lvl_sync, W.lvl_ncnt, c->al, c->panel_ws,
                                        c->opt.nb, level_grid(c),
                                        c->opt.spin_limit_log2 < 0 ? 0 : (1ll << c->opt.spin_limit_log2), sd);
                 }
@@ -1589,14 +1643,13 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             }
             if (W.asm_cnt2 > 0) {
                 Prof pr(c, IPM_K_LARGE_ASSEMBLE, W.asm_w, sd);
-                launch_large_assemble(c->dp, V, c->fronts, c->asm_items + W.asm_off2, c->asm_info + W.asm_off2,
-                                      c->asm_cr, W.asm_cnt2, sd);
+                launch_large_assemble(c->dp, V, c->fronts, c->al, W.asm_off2, W.asm_cnt2, sd);
                 nl++;
             }
             if (W.thin_cnt > 0) {
                 Prof pr(c, IPM_K_LARGE_PANEL, W.thin_w, sd);
                 launch_thin_fronts(c->dp, V, c->fronts, c->D, c->Dinv, c->dyn, c->ctl, c->thin_list + W.thin_off,
-                                   c->thin_asm + W.thin_off, c->thin_slot + W.thin_off, c->asm_info, c->asm_cr,
+                                   c->thin_asm + W.thin_off, c->thin_slot + W.thin_off, c->al,
                                    c->panel_ws, W.thin_cnt, c->opt.nb, sd);
                 nl++;
             }

@@ -198,14 +198,37 @@ struct PanelItem {
     int32_t r0, r1;  // row range (local) handled by this block
     int32_t p0;      // first column of the item's panel (diagonal blocks, triangular solves)
 };
-// Precomputed ranges of an assembly item (front columns [r0, r1) of a large
-// front, rows [r_lo, r_hi)): its original entries [o0, o1) (those of the
-// columns; the item keeps the ones in its rows) and, at acr[4 * cr ...], per
-// child (children ascending) the range [a, b) of contribution-block columns
-// and the range [ilo, ihi) of contribution-block rows that land in the item.
+// An assembly item: columns [c_lo, c_hi) (a block of 32), rows [r_lo, r_hi) (a
+// block of kAsmRows, from the columns' first: the upper part is never read) of
+// large front s.  Its terms, in the order they are added: the original entries
+// among [o0, o1) (those of the columns) that lie in its rows; the entries of
+// the small children (contribution blocks of up to kPointRows rows) as one list
+// of arena positions per destination, [seg0, seg1) of AsmLists; the large
+// children [ch0, ch1).  Device child lists hold the small children before the
+// large ones, so every path adds in this order.
+constexpr int kAsmRows = 64;
+constexpr int kPointRows = 64;
 struct AsmItem {
-    int64_t o0, o1, cr;
-    int32_t r_lo, r_hi;  // front rows [r_lo, r_hi) handled (rows below the columns' first: the upper part is never read)
+    int64_t o0, o1, seg0, seg1;
+    int32_t ch0, ch1, s, c_lo, c_hi, r_lo, r_hi;
+};
+__host__ __device__ inline int32_t asm_tiles(int32_t f) {  // items of a front of f rows
+    const int32_t nc = (f + 31) / 32, nr = (f + kAsmRows - 1) / kAsmRows;
+    return nc * nr - (nc - 1) * (nc - 1) / 4;  // block column i starts at block row i / 2
+}
+// A large child's part in a block of columns: its columns [a, b) land there;
+// rt + i is where its rows of the front's i-th block of kAsmRows rows begin.
+struct AsmChild {
+    int64_t cb, map;  // its contribution block in the arena, its row map
+    int32_t ldc, a, b, rt;
+};
+struct AsmLists {
+    const AsmItem *items;
+    const int32_t *seg_dst;  // destination within the item: 64 (column - c_lo) + row % 64
+    const int64_t *seg_ptr;  // its arena positions, children ascending
+    const int64_t *src;
+    const AsmChild *child;
+    const int32_t *rt;
 };
 struct TileItem {
     int32_t s;
@@ -249,7 +272,7 @@ enum : int32_t { kItemAssemble = 0, kItemDiag = 1, kItemTrsm = 2, kItemStrip = 3
 struct FactorItem {
     int32_t kind;
     int32_t s, t;  // front, pivot block (panel) index
-    int32_t a, b;  // assemble: columns [a, b); trsm: rows [a, b); strip / tile: first row, first column
+    int32_t a, b;  // trsm: rows [a, b); strip / tile: first row, first column
     int32_t aux;   // assemble: AsmItem index; diag / trsm: panel workspace slot
     int32_t wait0, need0, wait1, need1;
     int32_t sig, add;
@@ -261,8 +284,8 @@ void launch_norm1(const DevPlan &P, const DevVals &V, DevCtl *ctl, double eps_pi
 void launch_small_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                          DevCtl *ctl, const int32_t *list, int32_t count, int32_t nb, int32_t maxf, int32_t threads,
                          cudaStream_t st);
-void launch_large_assemble(const DevPlan &P, const DevVals &V, double *fronts, const PanelItem *items,
-                           const AsmItem *ainfo, const int32_t *acr, int32_t count, cudaStream_t st);
+void launch_large_assemble(const DevPlan &P, const DevVals &V, double *fronts, const AsmLists &A, int64_t first,
+                           int32_t count, cudaStream_t st);
 // panel step 1 (diagonal block of the panel [item.p0, item.p0 + nb), one item
 // per front; item.r1 = workspace slot)
 void launch_panel_diag(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
@@ -283,17 +306,15 @@ void launch_large_update_strip(const DevPlan &P, double *fronts, const double *D
 constexpr int64_t kLongColumn = 2048;  // longer sums over a sparse row take a CTA each
 constexpr int64_t kWarpRow = 32;       // and longer than this a warp each (rows_common.cuh)
 // thin fronts (k <= nb, f <= kThinMaxF), one CTA per front: list[i] the front,
-// first_asm[i] its first assembly item (one per 32 columns, rows from the
-// block's first column), slots[i] its panel workspace slot
+// first_asm[i] its first assembly item, slots[i] its panel workspace slot
 constexpr int kThinMaxF = 512;
 void launch_thin_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                         DevCtl *ctl, const int32_t *list, const int32_t *first_asm, const int32_t *slots,
-                        const AsmItem *ainfo, const int32_t *acr, double *pws, int32_t count, int32_t nb,
-                        cudaStream_t st);
+                        const AsmLists &A, double *pws, int32_t count, int32_t nb, cudaStream_t st);
 void launch_large_level(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                         DevCtl *ctl, const FactorItem *items, int32_t count, int32_t *sync, int32_t ncounters,
-                        const AsmItem *ainfo, const int32_t *acr, double *pws, int32_t nb, int32_t grid,
-                        long long spin_limit, cudaStream_t st);
+                        const AsmLists &A, double *pws, int32_t nb, int32_t grid, long long spin_limit,
+                        cudaStream_t st);
 const void *large_level_kernel();
 void launch_large_update(const DevPlan &P, double *fronts, const double *D, const TileItem *items, int32_t count,
                          int32_t w, cudaStream_t st);

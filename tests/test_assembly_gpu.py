@@ -1,0 +1,58 @@
+"""Assembly of large fronts: children of up to 64 contribution rows go in as
+lists of positions per destination, larger ones by columns and row blocks.
+Children at the edges of the two classes and of the 32-column and 64-row
+blocks, in the level kernel, the per-step launches and the dependency order:
+the factor against the oracle, and the three equal bit for bit."""
+import numpy as np
+import pytest
+
+import synth
+from synth.lp import _from_coo
+from test_parity_gpu import check_pair, run_pair
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2508_04370_gb300.build import build
+
+    build()
+    import paper_2508_04370_gb300 as p
+
+    return p
+
+
+def lp_with_columns(m, lengths, seed):
+    """Column j holds lengths[j] entries; eliminated first (natural order), it is
+    a front with that many contribution rows, and the dense rows are one front
+    of about m rows."""
+    rng = np.random.default_rng(seed)
+    rows = np.concatenate([np.sort(rng.choice(m, size=k, replace=False)) for k in lengths])
+    cols = np.repeat(np.arange(len(lengths)), lengths)
+    return _from_coo(m, len(lengths), rows, cols, rng.standard_normal(rows.size), "columns")
+
+
+@pytest.mark.parametrize("m,lengths", [
+    (130, [63, 64, 65, 66, 31, 32, 33, 130, 1, 2] * 3 + [128, 129, 130]),
+    (192, [64, 65, 100, 191, 192] + [6] * 120),
+    (257, [257, 64, 65, 127, 129] + [1, 5, 33] * 90),
+])
+def test_children_at_class_and_block_edges(pkg, m, lengths):
+    lp = lp_with_columns(m, lengths, m)
+    theta = synth.theta_loguniform(lp.n, 5, -3.0, 3.0)
+    r7, r1 = synth.rhs_normal(lp.n, 6), synth.rhs_normal(lp.m, 7)
+    base = None
+    for opts in (dict(), dict(level_kernel=0), dict(schedule=pkg.IPM_SCHED_DEPENDENCY)):
+        r = run_pair(pkg, lp, theta, r7, r1, ordering=pkg.IPM_ORD_NATURAL, **opts)
+        assert r["info"]["nfronts_large"] > 0
+        check_pair(r, lp)
+        if base is None:
+            base = r
+        else:
+            assert np.array_equal(base["D"], r["D"]) and np.array_equal(base["L"], r["L"])
+        r["s"].close()
