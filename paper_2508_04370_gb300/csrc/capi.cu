@@ -41,7 +41,7 @@ struct StepWork {
     int64_t alt_off;  // FP64 tiles of the same fronts, used after a precision fallback
     int32_t alt_cnt;
     int32_t alt_cnt1;  // lookahead tiles among them
-    int64_t st_off;   // sliced path: 128 x 32 output tiles; the first st_cnt1 cover the next panel's
+    int64_t st_off;   // sliced path: segments of output tiles (a CTA each); the first st_cnt1 cover the next panel's
     int32_t st_cnt;   // columns (critical path), the rest run beside the next panel
     int32_t st_cnt1;
     Work panel_w, trsm_w, tile_w, tile_w1, tc_w, alt_w, alt_w1, st_w1, st_w2, asm_w;
@@ -124,10 +124,11 @@ struct ipm_ctx {
     int32_t *thin_list = nullptr, *thin_asm = nullptr, *thin_slot = nullptr;  // thin fronts by level
     double *panel_ws = nullptr;
     TileItem *tile_items = nullptr, *tc_items = nullptr, *alt_items = nullptr;
-    SlicedTile *sliced_tiles = nullptr;  // sliced tensor-core path: output tiles per step
-    uint8_t *slice_ws = nullptr;       // digit images of a step: two halves, used by alternate steps
-    int32_t *slice_exp = nullptr;      // their row scales (two halves)
-    int64_t slice_half_blocks = 0;     // slice blocks per half
+    SlicedRun *sliced_runs = nullptr;  // sliced tensor-core path: runs of output tiles
+    SlicedSeg *sliced_segs = nullptr;  // and the CTAs' segments of them per step
+    uint8_t *slice_ws = nullptr;       // digit images of a step: three parts, used in turn
+    int32_t *slice_exp = nullptr;      // their row scales (three parts)
+    int64_t slice_part_blocks = 0;     // slice blocks per part
     FactorItem *lvl_items = nullptr;  // persistent level kernel: items of all levels
     InvItem *inv_items = nullptr;     // diagonal blocks inverted after each factorisation
     InvItem *pair_items = nullptr;    // blocks of multi-block supernodes (neighbour products)
@@ -179,6 +180,8 @@ struct ipm_ctx {
     cudaStream_t cap_stream = nullptr;  // private stream used only for capturing
     cudaStream_t side = nullptr;        // large fronts of a level run here, beside the small fronts
     cudaStream_t side2 = nullptr;       // trailing updates beside the next panel (lookahead)
+    cudaStream_t side3 = nullptr;       // those of the sliced path, beside the next two panels
+    cudaStream_t side4 = nullptr;       // dependency order: assembly beside the step before
     cudaStream_t cls[2] = {nullptr, nullptr};  // the 2nd and 3rd small-front size classes of a level
     std::vector<cudaEvent_t> dep_ev;    // level-to-level dependencies between the streams
     std::vector<cudaEvent_t> step_ev;   // per-step fork/join of the trailing updates
@@ -482,6 +485,10 @@ void free_device(ipm_ctx *c) {
     c->side = nullptr;
     if (c->side2) cudaStreamDestroy(c->side2);
     c->side2 = nullptr;
+    if (c->side3) cudaStreamDestroy(c->side3);
+    c->side3 = nullptr;
+    if (c->side4) cudaStreamDestroy(c->side4);
+    c->side4 = nullptr;
     for (cudaStream_t &q : c->cls) {
         if (q) cudaStreamDestroy(q);
         q = nullptr;
@@ -681,6 +688,11 @@ int setup_device(ipm_ctx *c) {
         cudaGetLastError();
         return IPM_ERR_NO_DEVICE;
     }
+    {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->opt.device);
+        c->sms = std::max(1, sms);
+    }
     const int32_t ns = P.nsuper, N = P.N;
     std::vector<int32_t> c0(ns);
     for (int32_t s = 0; s < ns; s++) c0[s] = P.sn_start[s];
@@ -762,7 +774,8 @@ int setup_device(ipm_ctx *c) {
     for (int32_t s = 0; s < P.nsuper; s++)
         if (P.sn_large[s]) slot_of[s] = nslots++;
     std::vector<TileItem> tile_items, tc_items, alt_items;
-    std::vector<SlicedTile> sliced_tiles;
+    std::vector<SlicedRun> sliced_runs;
+    std::vector<SlicedSeg> sliced_segs;
     int64_t max_slice_blocks = 0;
     const bool sliced = c->opt.precision == IPM_PREC_SLICED;
     std::vector<FactorItem> lvl_items;
@@ -871,9 +884,9 @@ int setup_device(ipm_ctx *c) {
         S.tile_off = (int64_t)tile_items.size();
         S.tc_off = (int64_t)tc_items.size();
         S.alt_off = (int64_t)alt_items.size();
-        S.st_off = (int64_t)sliced_tiles.size();
+        S.st_off = (int64_t)sliced_segs.size();
         int32_t nblk = 0;  // slice blocks of this step
-        std::vector<SlicedTile> t1, t2;  // sliced tiles: next panel's columns / the rest
+        std::vector<SlicedRun> t1, t2;  // sliced runs: next panel's columns / the rest (whole rows, cut below)
         std::vector<TileItem> u1, u2, a1, a2;  // lookahead / remaining tiles of this step
         Work w1, w2, wa1, wa2;
         // lower entries of a kUpdTile tile times 2 w flops (and its bytes)
@@ -917,21 +930,26 @@ int setup_device(ipm_ctx *c) {
                 const double wk = pair_second ? w + c->opt.nb : w;  // columns of the product
                 const int32_t jend = pair_first ? p1 + kSliceCols : f;
                 nblk += (f - p1 + kSliceRows - 1) / kSliceRows;
-                for (int32_t j0 = p1; j0 < jend; j0 += kSliceCols)
-                    for (int32_t b = (j0 - p1) / kSliceRows; p1 + b * kSliceRows < f; b++) {
-                        const int32_t i0 = p1 + b * kSliceRows;
-                        const bool la = next_panel && j0 == p1;
-                        (la ? t1 : t2).push_back({s, i0, j0, base + b, base + (j0 - p1) / kSliceRows,
-                                                  (j0 - p1) % kSliceRows, kc});
+                // the columns on the critical path end here: the next panel's; after a
+                // pair's second panel those of the next two, so that the rest of the
+                // pair's update has two steps to run beside
+                const int32_t ahead = pair_second ? 2 * kSliceCols : kSliceCols;
+                const int32_t jla = next_panel ? std::min(std::min(p1 + ahead, jend), p1 + (k - p1 + 31) / 32 * 32) : p1;
+                for (int32_t i0 = p1; i0 < f; i0 += kSliceRows) {
+                    const int32_t jrow = std::min(jend, std::min(f, i0 + kSliceRows));  // this row block's columns
+                    if (jla > p1) t1.push_back({s, i0, p1, (std::min(jla, jrow) - p1 + kSliceCols - 1) / kSliceCols, base, p1, kc});
+                    if (jrow > jla) t2.push_back({s, i0, jla, (jrow - jla + kSliceCols - 1) / kSliceCols, base, p1, kc});
+                    for (int32_t j0 = p1; j0 < jrow; j0 += kSliceCols) {
                         // lower entries of the tile times 2 wk flops; its C read and write
                         double e = 0.0;
                         for (int32_t j = j0; j < std::min(j0 + kSliceCols, f); j++)
                             e += std::max(0, std::min(i0 + kSliceRows, f) - std::max(i0, j));
-                        Work &tw = la ? S.st_w1 : S.st_w2;
+                        Work &tw = j0 < jla ? S.st_w1 : S.st_w2;
                         tw.flops += 2.0 * wk * e;
                         // C read and written; the digit images of its 128 A rows and 32 B rows (bf16)
                         tw.bytes += 16.0 * e + 2.0 * kSlices * wk * (kSliceRows + kSliceCols);
                     }
+                }
                 S.trsm_w.bytes += 2.0 * kSlices * 2.0 * rest * wk;  // the slices the solve writes
                 if (pair_second) S.trsm_w.bytes += 8.0 * rest * c->opt.nb;  // the first panel's rows it re-reads
             } else if (tc) {
@@ -977,10 +995,34 @@ int setup_device(ipm_ctx *c) {
         S.tile_cnt = (int32_t)(tile_items.size() - S.tile_off);
         S.tc_cnt = (int32_t)(tc_items.size() - S.tc_off);
         S.alt_cnt = (int32_t)(alt_items.size() - S.alt_off);
-        sliced_tiles.insert(sliced_tiles.end(), t1.begin(), t1.end());
-        sliced_tiles.insert(sliced_tiles.end(), t2.begin(), t2.end());
-        S.st_cnt = (int32_t)(sliced_tiles.size() - S.st_off);
-        S.st_cnt1 = (int32_t)t1.size();
+        // one CTA per SM, each with an equal share of the tiles in row order; the
+        // rest leaves kSliceFreeSms SMs to the next panels' kernels
+        auto cut = [&](const std::vector<SlicedRun> &rows, int32_t most) {
+            int64_t total = 0;
+            for (const SlicedRun &r : rows) total += r.nt;
+            const int64_t ctas = std::min<int64_t>(total, most);
+            int64_t done = 0, cta = 0;  // tiles placed, segments finished
+            int32_t first = (int32_t)sliced_runs.size();
+            for (const SlicedRun &r : rows)
+                for (int32_t t = 0; t < r.nt;) {
+                    const int64_t share = total * (cta + 1) / ctas - done;  // left in this segment
+                    SlicedRun u = r;
+                    u.j0 = r.j0 + t * kSliceCols;
+                    u.nt = (int32_t)std::min<int64_t>(r.nt - t, share);
+                    sliced_runs.push_back(u);
+                    t += u.nt;
+                    done += u.nt;
+                    if (u.nt == share) {
+                        sliced_segs.push_back({first, (int32_t)sliced_runs.size()});
+                        first = (int32_t)sliced_runs.size();
+                        cta++;
+                    }
+                }
+        };
+        cut(t1, c->sms);
+        S.st_cnt1 = (int32_t)(sliced_segs.size() - S.st_off);
+        cut(t2, std::max(1, c->sms - kSliceFreeSms));
+        S.st_cnt = (int32_t)(sliced_segs.size() - S.st_off);
         max_slice_blocks = std::max<int64_t>(max_slice_blocks, nblk);
         return S;
     };
@@ -1208,15 +1250,15 @@ int setup_device(ipm_ctx *c) {
         (rc = dalloc(c, &c->panel_ws, (size_t)std::max(nslots, 1) * kPanelWsHost)) ||
         (rc = dupload(c, &c->tile_items, tile_items)) || (rc = dupload(c, &c->tc_items, tc_items)) ||
         (rc = dupload(c, &c->alt_items, alt_items)) || (rc = dupload(c, &c->bwd_order, bwd_order)) ||
-        (rc = dupload(c, &c->trsm_sbase, trsm_sbase)) || (rc = dupload(c, &c->sliced_tiles, sliced_tiles)) ||
+        (rc = dupload(c, &c->trsm_sbase, trsm_sbase)) || (rc = dupload(c, &c->sliced_runs, sliced_runs)) || (rc = dupload(c, &c->sliced_segs, sliced_segs)) ||
         (rc = dupload(c, &c->thin_list, thin_list)) || (rc = dupload(c, &c->thin_asm, thin_asm)) ||
         (rc = dupload(c, &c->thin_slot, thin_slot)) ||
-        (rc = dalloc(c, &c->slice_ws, 2 * (size_t)max_slice_blocks * (size_t)kSliceBlockBytes)) ||
-        (rc = dalloc(c, &c->slice_exp, 2 * (size_t)std::max<int64_t>(max_slice_blocks, 1) * kSliceRows * 2)) ||
+        (rc = dalloc(c, &c->slice_ws, 3 * (size_t)max_slice_blocks * (size_t)kSliceBlockBytes)) ||
+        (rc = dalloc(c, &c->slice_exp, 3 * (size_t)std::max<int64_t>(max_slice_blocks, 1) * kSliceRows * 2)) ||
         (rc = dupload(c, &c->lvl_items, lvl_items)) || (rc = dalloc(c, &c->lvl_sync, (size_t)max_ncnt + 1)) ||
         (rc = dalloc(c, &c->solve_sync, (size_t)3 * ns + 1)))
         return rc;
-    c->slice_half_blocks = max_slice_blocks;
+    c->slice_part_blocks = max_slice_blocks;
     int32_t *d_sparent, *d_long, *d_mid;
     double *d_kval, *d_kabs;
     if ((rc = dupload(c, &d_sparent, P.sn_parent))) return rc;
@@ -1226,13 +1268,9 @@ int setup_device(ipm_ctx *c) {
         (rc = dalloc(c, &d_kval, (size_t)kp[N])) || (rc = dalloc(c, &d_kabs, (size_t)N)))
         return rc;
     {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         int lvl_per_sm = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&lvl_per_sm, large_level_kernel(), 256, 0);
-        c->lvl_grid = sms * std::max(1, lvl_per_sm);
-        c->sms = std::max(1, sms);
+        c->lvl_grid = c->sms * std::max(1, lvl_per_sm);
     }
     DevPlan &dp = c->dp;
     dp.N = N;
@@ -1417,18 +1455,20 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
     // two instead of their sum.  Level l's small fronts wait for the large
     // fronts of level l-1 and vice versa (events; a captured graph keeps them
     // as edges).
-    if (!c->side) {
+    if (!c->side || !c->side4) {
         // the large fronts' per-step chain (diagonal block, triangular solve,
         // lookahead update) is the factorisation's critical path: its stream
         // gets the highest priority, so its CTAs go first when the trailing
-        // updates running beside it on side2 release SMs
+        // updates running beside it on side2 release SMs; so does the assembly
+        // of the fronts the chain takes up next
         int prio_lo = 0, prio_hi = 0;
         cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
-        if (cudaStreamCreateWithPriority(&c->side, cudaStreamNonBlocking, prio_hi) != cudaSuccess) {
-            cudaGetLastError();
-            c->side = nullptr;
-            return IPM_ERR_CUDA;
-        }
+        for (cudaStream_t *q : {&c->side, &c->side4})
+            if (!*q && cudaStreamCreateWithPriority(q, cudaStreamNonBlocking, prio_hi) != cudaSuccess) {
+                cudaGetLastError();
+                *q = nullptr;
+                return IPM_ERR_CUDA;
+            }
     }
     const size_t nev = 5 * (size_t)P.nlevels + 2;  // per level: fork, two joins, small done, large done
     while (c->dep_ev.size() < nev) {
@@ -1439,7 +1479,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         }
         c->dep_ev.push_back(e);
     }
-    for (cudaStream_t *q : {&c->side2, &c->cls[0], &c->cls[1]}) {
+    for (cudaStream_t *q : {&c->side2, &c->side3, &c->cls[0], &c->cls[1]}) {
         if (!*q && cudaStreamCreateWithFlags(q, cudaStreamNonBlocking) != cudaSuccess) {
             cudaGetLastError();
             *q = nullptr;
@@ -1448,7 +1488,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
     }
     size_t nsteps = c->dsteps.size();
     for (const LevelWork &W : c->levels) nsteps += W.steps.size();
-    while (c->step_ev.size() < 2 * nsteps) {
+    while (c->step_ev.size() < 3 * nsteps) {
         cudaEvent_t e;
         if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
@@ -1456,7 +1496,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         }
         c->step_ev.push_back(e);
     }
-    while (c->done_ev.size() < c->dsteps.size() + 1) {
+    while (c->done_ev.size() < 2 * c->dsteps.size() + 1) {
         cudaEvent_t e;
         if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
@@ -1464,7 +1504,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         }
         c->done_ev.push_back(e);
     }
-    cudaStream_t sd = c->side, sd2 = c->side2;
+    cudaStream_t sd = c->side, sd2 = c->side2, sd3 = c->side3;
     size_t sidx = 0;
     cudaEventRecord(c->dep_ev[0], st);
     cudaStreamWaitEvent(sd, c->dep_ev[0], 0);
@@ -1497,8 +1537,21 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
     // stay on the critical path; the remaining trailing tiles run on a third
     // stream beside the next step's diagonal blocks.  Every entry still
     // receives the panels' updates in panel order: the lookahead tiles of
-    // step s wait for the remaining tiles of step s-1.
+    // step s wait for the remaining tiles of step s-1.  On the sliced path the
+    // lookahead after a pair of panels covers the next two panels' columns, so
+    // the lookahead of step s waits only for the sliced rest of step s-2.
     cudaEvent_t prev_rest = nullptr;
+    // ends of each step's remaining tiles: FP64, sliced (each on one stream, so
+    // a later end implies the earlier ones)
+    std::vector<cudaEvent_t> fp64_rest(nsteps, nullptr), sliced_rest(nsteps, nullptr);
+    auto wait_rest = [&](cudaStream_t q, size_t steps) {  // those of the first `steps` steps
+        for (const std::vector<cudaEvent_t> *v : {&fp64_rest, &sliced_rest})
+            for (size_t g = std::min(steps, v->size()); g > 0; g--)
+                if ((*v)[g - 1]) {
+                    cudaStreamWaitEvent(q, (*v)[g - 1], 0);
+                    break;
+                }
+    };
     auto emit_step = [&](const StepWork &S) {
         {
             Prof pr(c, IPM_K_PIVOT_BLOCK, S.panel_w, sd);
@@ -1508,12 +1561,11 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         nl++;
         const bool use_tc = (S.tc_cnt > 0 || S.st_cnt > 0) && c->mixed_active;
         const bool use_sliced = use_tc && S.st_cnt > 0;
-        // sliced path: the digit images of this step (alternate halves of the
-        // work space: the rest of step s-1 may still read its half while
-        // step s slices; step s+1 slices only after step s's lookahead,
-        // which waits for the rest of step s-1)
-        uint8_t *ws = c->slice_ws + (sidx & 1) * c->slice_half_blocks * kSliceBlockBytes;
-        int32_t *wexp = c->slice_exp + (sidx & 1) * c->slice_half_blocks * kSliceRows * 2;
+        // sliced path: the digit images of this step, in one of three parts of
+        // the work space (the rest of step s is waited for by the lookahead of
+        // step s+2, so step s+3 may write where step s did)
+        uint8_t *ws = c->slice_ws + (sidx % 3) * c->slice_part_blocks * kSliceBlockBytes;
+        int32_t *wexp = c->slice_exp + (sidx % 3) * c->slice_part_blocks * kSliceRows * 2;
         if (S.trsm_cnt > 0) {
             // on the sliced path the solve also writes the slices of the rows it finishes
             Prof pr(c, IPM_K_LARGE_PANEL, S.trsm_w, sd);
@@ -1525,10 +1577,9 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         const int32_t rest_tiles = S.tile_cnt - S.tile_cnt1;
         const int32_t rest_alt = ((S.tc_cnt > 0 || S.st_cnt > 0) && !c->mixed_active) ? S.alt_cnt - S.alt_cnt1 : 0;
         const int32_t rest_sliced = use_sliced ? S.st_cnt - S.st_cnt1 : 0;
-        cudaEvent_t this_rest = nullptr;
-        if (rest_tiles > 0 || rest_alt > 0 || rest_sliced > 0) {
-            cudaEvent_t ev_in = c->step_ev[2 * sidx], ev_out = c->step_ev[2 * sidx + 1];
-            cudaEventRecord(ev_in, sd);
+        cudaEvent_t this_rest = nullptr, ev_in = c->step_ev[3 * sidx];
+        if (rest_tiles > 0 || rest_alt > 0 || rest_sliced > 0) cudaEventRecord(ev_in, sd);
+        if (rest_tiles > 0 || rest_alt > 0) {
             cudaStreamWaitEvent(sd2, ev_in, 0);
             if (rest_tiles > 0) {
                 Prof pr(c, IPM_K_LARGE_UPDATE, S.tile_w, sd2);
@@ -1542,17 +1593,24 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
                                     c->opt.nb, sd2);
                 nl++;
             }
-            if (rest_sliced > 0) {
-                Prof pr(c, IPM_K_LARGE_UPDATE_TC, S.st_w2, sd2);
-                launch_update_sliced(c->dp, c->fronts, c->sliced_tiles + S.st_off + S.st_cnt1, rest_sliced, ws, wexp,
-                                     c->ctl, sd2);
+            this_rest = c->step_ev[3 * sidx + 1];
+            cudaEventRecord(this_rest, sd2);
+            fp64_rest[sidx] = this_rest;
+        }
+        if (rest_sliced > 0) {
+            cudaStreamWaitEvent(sd3, ev_in, 0);
+            {
+                Prof pr(c, IPM_K_LARGE_UPDATE_TC, S.st_w2, sd3);
+                launch_update_sliced(c->dp, c->fronts, c->sliced_runs, c->sliced_segs + S.st_off + S.st_cnt1,
+                                     rest_sliced, ws, wexp, c->ctl, sd3);
                 nl++;
             }
-            cudaEventRecord(ev_out, sd2);
-            this_rest = ev_out;
+            cudaEventRecord(c->step_ev[3 * sidx + 2], sd3);
+            sliced_rest[sidx] = c->step_ev[3 * sidx + 2];
         }
         sidx++;
         if (prev_rest) cudaStreamWaitEvent(sd, prev_rest, 0);
+        if (sidx >= 3 && sliced_rest[sidx - 3]) cudaStreamWaitEvent(sd, sliced_rest[sidx - 3], 0);
         if (S.tile_cnt1 > 0) {
             Prof pr(c, IPM_K_LARGE_UPDATE, S.tile_w1, sd);
             launch_large_update_strip(c->dp, c->fronts, c->D, c->tile_items + S.tile_off, S.tile_cnt1, c->opt.nb,
@@ -1566,7 +1624,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         } else if (use_sliced) {
             if (S.st_cnt1 > 0) {
                 Prof pr(c, IPM_K_LARGE_UPDATE_TC, S.st_w1, sd);
-                launch_update_sliced(c->dp, c->fronts, c->sliced_tiles + S.st_off, S.st_cnt1, ws, wexp, c->ctl, sd);
+                launch_update_sliced(c->dp, c->fronts, c->sliced_runs, c->sliced_segs + S.st_off, S.st_cnt1, ws, wexp, c->ctl, sd);
                 nl++;
             }
         } else if (use_tc) {
@@ -1588,7 +1646,10 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         auto issue_small = [&](int32_t g) {
             while (next < P.nlevels && c->small_dep[next] < g) {
                 if (!c->levels[next].small.empty()) {
-                    if (c->small_dep[next] >= 0) cudaStreamWaitEvent(st, c->done_ev[c->small_dep[next]], 0);
+                    if (c->small_dep[next] >= 0) {
+                        cudaStreamWaitEvent(st, c->done_ev[c->small_dep[next]], 0);
+                        wait_rest(st, c->small_dep[next]);
+                    }
                     emit_small(next);
                 }
                 next++;
@@ -1597,16 +1658,30 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         for (int32_t g = 0; g < T; g++) {
             issue_small(g);
             const StepWork &S = c->dsteps[g];
-            if (S.small_wait >= 0) cudaStreamWaitEvent(sd, c->dep_ev[4 + 5 * S.small_wait], 0);
             if (S.asm_cnt > 0) {
-                Prof pr(c, IPM_K_LARGE_ASSEMBLE, S.asm_w, sd);
-                launch_large_assemble(c->dp, V, c->fronts, c->al, S.asm_off, S.asm_cnt, sd);
+                // the starting fronts' children were done two steps ago: their
+                // assembly runs beside the step before this one (on the critical
+                // stream it kept the other fronts' chains waiting)
+                cudaStream_t sa = c->side4;
+                if (g >= 2) {
+                    cudaStreamWaitEvent(sa, c->done_ev[g - 2], 0);
+                    wait_rest(sa, g - 1);
+                } else {
+                    cudaStreamWaitEvent(sa, c->dep_ev[0], 0);
+                }
+                if (S.small_wait >= 0) cudaStreamWaitEvent(sa, c->dep_ev[4 + 5 * S.small_wait], 0);
+                {
+                    Prof pr(c, IPM_K_LARGE_ASSEMBLE, S.asm_w, sa);
+                    launch_large_assemble(c->dp, V, c->fronts, c->al, S.asm_off, S.asm_cnt, sa);
+                }
                 nl++;
+                cudaEventRecord(c->done_ev[T + 1 + g], sa);
+                cudaStreamWaitEvent(sd, c->done_ev[T + 1 + g], 0);
             }
             emit_step(S);
             cudaEventRecord(c->done_ev[g], sd);
         }
-        if (prev_rest) cudaStreamWaitEvent(sd, prev_rest, 0);
+        wait_rest(sd, nsteps);
         cudaEventRecord(c->done_ev[T], sd);
         issue_small(INT32_MAX);
     } else {
@@ -1655,7 +1730,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             }
             prev_rest = nullptr;
             for (const StepWork &S : W.steps) emit_step(S);
-            if (prev_rest) cudaStreamWaitEvent(sd, prev_rest, 0);
+            wait_rest(sd, sidx);
             last_large = c->dep_ev[5 + 5 * l];
             cudaEventRecord(last_large, sd);
         }

@@ -254,14 +254,22 @@ constexpr int64_t kSliceOperandBytes = 4 * kSlicePairBytes;
 constexpr int64_t kSliceChunkBytes = 2 * kSliceOperandBytes;  // operand A (L), then operand B (L d)
 constexpr int64_t kSliceBlockBytes = kSliceChunks * kSliceChunkBytes;
 
-struct SlicedTile {
+// A run of output tiles: rows i0 .. i0+127 (one slice block), nt tiles of 32
+// columns from j0 (lower part only).  A CTA works through the runs
+// [first, last) of its segment.
+struct SlicedRun {
     int32_t s;
-    int32_t i0, j0;     // output rows i0 .. i0+127, columns j0 .. j0+31 (lower part only)
-    int32_t blk_a;      // slice block of rows i0 ..
-    int32_t blk_b;      // slice block holding columns j0 .. j0+31 as rows,
-    int32_t roff_b;     // at row offset roff_b (a multiple of 32) inside it
-    int32_t kc;         // chunks of the product: 1 (one panel, K <= 32) or 2 (a pair of panels, K <= 64)
+    int32_t i0, j0, nt;
+    int32_t base, p1;  // slice block of rows p1 ..
+    int32_t kc;        // chunks of the product: 1 (one panel, K <= 32) or 2 (a pair of panels, K <= 64)
 };
+struct SlicedSeg {
+    int32_t first, last;
+};
+// SMs the launch of a pair's trailing update leaves to the next panels' kernels
+// (50-period staircase, factorisation: 61.1 ms with 0, 60.3 with 8, 60.6 with 16,
+// 66.8 with 48).
+constexpr int kSliceFreeSms = 8;
 
 // One item of the persistent level kernel (large fronts of one tree level):
 // it waits until counter wait0 >= need0 and counter wait1 >= need1 (-1: no
@@ -320,7 +328,7 @@ void launch_large_update(const DevPlan &P, double *fronts, const double *D, cons
                          int32_t w, cudaStream_t st);
 void launch_large_update_tc(const DevPlan &P, double *fronts, const double *D, const TileItem *items, int32_t count,
                             int32_t w, DevCtl *ctl, cudaStream_t st);
-void launch_update_sliced(const DevPlan &P, double *fronts, const SlicedTile *items, int32_t count,
+void launch_update_sliced(const DevPlan &P, double *fronts, const SlicedRun *runs, const SlicedSeg *segs, int32_t count,
                           const uint8_t *ws, const int32_t *ws_exp, DevCtl *ctl, cudaStream_t st);
 int measure_fp64_peaks(double *out, int blocks, int iters, int reps, cudaStream_t st, double *dfma_tflops,
                        double *dmma_tflops);

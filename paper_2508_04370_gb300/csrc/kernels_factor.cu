@@ -695,50 +695,63 @@ __device__ __forceinline__ void body_trsm(const DevPlan &P, double *__restrict__
         }
     }
     __syncthreads();
-    if (warp < nr) {
-        // rows warp, warp + 8, ... : RW independent chains share L_11 in registers
+    if constexpr (RW == 4) {
+        // rows warp, warp + 8, warp + 16 and warp + 24, eight lanes each: lane e of
+        // a row holds columns e, e + 8, e + 16 and e + 24, so that a finished u is
+        // applied to the columns after its block of eight only (79 FMAs per warp;
+        // a lane per column and a row after the other takes 124, half of them on
+        // columns that are finished)
+        const int e = lane & 7, rr = warp + kTrsmRows * (lane >> 3);
+        if (warp < nr) {
+            double t[4];
+#pragma unroll
+            for (int b = 0; b < 4; b++) t[b] = T[8 * b + e][rr];
+#pragma unroll
+            for (int c = 0; c < 31; c++) {
+                const double u = __shfl_sync(0xffffffffu, t[c >> 3], (lane & 24) | (c & 7));
+#pragma unroll
+                for (int b = c >> 3; b < 4; b++)
+                    if (8 * b + e > c) t[b] -= u * Wd[(8 * b + e) * 33 + c];
+            }
+#pragma unroll
+            for (int b = 0; b < 4; b++) T[8 * b + e][rr] = t[b] * Wd[32 * 33 + 8 * b + e];
+        }
+        __syncwarp();
+    } else if (warp < nr) {
+        // row warp, one lane per column
         double Lr[32];
 #pragma unroll
         for (int c = 0; c < 32; c++) Lr[c] = Wd[lane * 33 + c];
-        double t[RW];
-#pragma unroll
-        for (int j = 0; j < RW; j++) t[j] = T[lane][warp + kTrsmRows * j];
+        double t = T[lane][warp];
 #pragma unroll
         for (int c = 0; c < 31; c++) {
-#pragma unroll
-            for (int j = 0; j < RW; j++) {
-                const double u = __shfl_sync(0xffffffffu, t[j], c);
-                if (lane > c) t[j] -= u * Lr[c];
-            }
+            const double u = __shfl_sync(0xffffffffu, t, c);
+            if (lane > c) t -= u * Lr[c];
         }
-        const double dinv = Wd[32 * 33 + lane];
-#pragma unroll
-        for (int j = 0; j < RW; j++) {
-            const int rr = warp + kTrsmRows * j;
-            if (rr >= nr) break;  // uniform over the warp
-            const double lv = t[j] * dinv;
-            T[lane][rr] = lv;
-            if (so.ws) {
-                // the finished row, sliced for the tensor-core update
-                const int row = r0 + rr;
-                const int c0 = P.sn_c0[s];
-                const double dq = lane < w ? so.D[c0 + p0 + lane] : 0.0;
-                const double lq = lane < w ? lv : 0.0;
-                const int blk = so.base + (row - so.p1) / kSliceRows;
-                uint8_t *bp = so.ws + (int64_t)blk * kSliceBlockBytes;
-                int32_t *ep = so.exps + (int64_t)blk * kSliceRows * 2;
-                bool bad;
-                if (so.pair) {
-                    // the previous panel (always 32 columns) as chunk 0, this one as chunk 1
-                    const double l2[2] = {__ldcg(F + (int64_t)(p0 - 32 + lane) * ld + row), lq};
-                    const double d2[2] = {so.D[c0 + p0 - 32 + lane], dq};
-                    bad = sliced::slice_row_warp<2>(l2, d2, bp, ep, (row - so.p1) % kSliceRows);
-                } else {
-                    const double l1[1] = {lq}, d1[1] = {dq};
-                    bad = sliced::slice_row_warp<1>(l1, d1, bp, ep, (row - so.p1) % kSliceRows);
-                }
-                if (bad && lane == 0) atomicOr(&so.ctl->status, kStatNonFinite);
+        T[lane][warp] = t * Wd[32 * 33 + lane];
+        __syncwarp();
+    }
+    if (so.ws) {
+        // the finished rows, sliced for the tensor-core update
+        const int c0 = P.sn_c0[s];
+        const double dq = lane < w ? so.D[c0 + p0 + lane] : 0.0;
+        for (int rr = warp; rr < nr; rr += kTrsmRows) {
+            const int row = r0 + rr;
+            const double lq = lane < w ? T[lane][rr] : 0.0;
+            const int blk = so.base + (row - so.p1) / kSliceRows;
+            uint8_t *bp = so.ws + (int64_t)blk * kSliceBlockBytes;
+            int32_t *ep = so.exps + (int64_t)blk * kSliceRows * 2;
+            bool bad;
+            if (so.pair) {
+                // the previous panel (always 32 columns) as chunk 0, this one as chunk 1
+                const double l2[2] = {__ldcg(F + (int64_t)(p0 - 32 + lane) * ld + row), lq};
+                const double d2[2] = {so.D[c0 + p0 - 32 + lane], dq};
+                bad = sliced::slice_row_warp<2>(l2, d2, bp, ep, (row - so.p1) % kSliceRows);
+            } else {
+                const double l1[1] = {lq}, d1[1] = {dq};
+                bad = sliced::slice_row_warp<1>(l1, d1, bp, ep, (row - so.p1) % kSliceRows);
             }
+            if (bad && lane == 0) atomicOr(&so.ctl->status, kStatNonFinite);
         }
     }
     __syncthreads();
@@ -873,7 +886,7 @@ __device__ __forceinline__ void body_strip(const DevPlan &P, double *__restrict_
 // One launch per step: one item per CTA.
 __global__ void __launch_bounds__(kBodyThreads) k_large_assemble(DevPlan P, DevVals V, double *__restrict__ fronts,
                                                                   AsmLists A, int64_t first) {
-    __shared__ double pool[kPoolDoubles];
+    __shared__ double pool[32 * kAsmRows];
     const AsmItem ai = A.items[first + blockIdx.x];
     body_assemble(P, V, fronts, A, ai, pool);
 }

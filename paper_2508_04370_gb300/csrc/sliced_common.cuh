@@ -22,6 +22,15 @@ __device__ __forceinline__ uint32_t swz_chunk(int r, int c) {
     return (uint32_t)r * 128u + ((((uint32_t)c) ^ ((uint32_t)r & 7u)) << 4);
 }
 
+// Operand B of a chunk: per group of 32 rows the eight slices' 32 rows one after
+// the other (256 rows of 64 bytes, 64-byte swizzle), so that one MMA takes the
+// slices 0 .. 7 - t of the tile's columns as its N dimension.
+constexpr int kGroupBytes = kSlices * 32 * 64;
+__device__ __forceinline__ uint32_t swz_b(int r, int t, int c) {
+    return (uint32_t)(r >> 5) * (uint32_t)kGroupBytes + (uint32_t)(t * 32 + (r & 31)) * 64u +
+           (((uint32_t)c ^ (((uint32_t)r >> 1) & 3u)) << 4);
+}
+
 // Biased exponent field of a double given as bits.
 __device__ __forceinline__ int biased_exp(long long b) { return (int)((b >> 52) & 0x7ff); }
 
@@ -124,9 +133,10 @@ __device__ __forceinline__ bool slice_row_warp(const double (&l)[NC], const doub
                 const uint32_t w2 = __shfl_down_sync(0xffffffffu, pair, 4);
                 const uint32_t w3 = __shfl_down_sync(0xffffffffu, pair, 6);
                 if ((lane & 7) == 0) {
-                    const int chunk = (t & 1) * 4 + (lane >> 3);
-                    *(uint4 *)(img + (t >> 1) * kSlicePairBytes + swz_chunk(rr, chunk)) =
-                        make_uint4(pair, w1, w2, w3);
+                    const uint32_t at = op == 0 ? (t >> 1) * (uint32_t)kSlicePairBytes +
+                                                      swz_chunk(rr, (t & 1) * 4 + (lane >> 3))
+                                                : swz_b(rr, t, lane >> 3);
+                    *(uint4 *)(img + at) = make_uint4(pair, w1, w2, w3);
                 }
             }
         }
