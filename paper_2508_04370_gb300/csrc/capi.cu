@@ -1078,16 +1078,21 @@ int setup_device(ipm_ctx *c) {
         int32_t maxsteps = 0;
         std::vector<int32_t> main_fronts;
         W.thin_off = (int64_t)thin_list.size();
+        auto is_thin = [&](int32_t s) {
+            return P.sn_k[s] <= c->opt.nb && P.sn_f[s] <= kThinMaxF &&
+                   !(c->opt.precision != IPM_PREC_FP64 && P.sn_f[s] >= c->opt.mixed_min_front);
+        };
+        int32_t inner = 0;  // thin fronts with children
         for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++) {
             const int32_t s = P.lvl_large[t];
-            const int64_t first = (int64_t)asm_items.size();
+            inner += is_thin(s) && P.child_ptr[s] < P.child_ptr[s + 1];
+        }
+        std::vector<std::pair<double, int32_t>> thin;  // work, front
+        for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++) {
+            const int32_t s = P.lvl_large[t];
             add_asm(s);
-            const bool thin = P.sn_k[s] <= c->opt.nb && P.sn_f[s] <= kThinMaxF &&
-                              !(c->opt.precision != IPM_PREC_FP64 && P.sn_f[s] >= c->opt.mixed_min_front);
-            if (thin) {
-                thin_list.push_back(s);
-                thin_asm.push_back((int32_t)first);
-                thin_slot.push_back(slot_of[s]);
+            if (is_thin(s) && (P.child_ptr[s] == P.child_ptr[s + 1] || inner >= kThinInner)) {
+                thin.push_back({(double)P.sn_k[s] * P.sn_f[s] * P.sn_f[s], s});
                 const Work fr = front_work(s);
                 W.thin_w.flops += fr.flops;
                 W.thin_w.bytes += fr.bytes;
@@ -1095,6 +1100,15 @@ int setup_device(ipm_ctx *c) {
                 main_fronts.push_back(s);
                 maxsteps = std::max(maxsteps, (P.sn_k[s] + c->opt.nb - 1) / c->opt.nb);
             }
+        }
+        // the longest first, so that none starts when the others are done
+        std::stable_sort(thin.begin(), thin.end(), [](const std::pair<double, int32_t> &x, const std::pair<double, int32_t> &y) {
+            return x.first > y.first;
+        });
+        for (const auto &e : thin) {
+            thin_list.push_back(e.second);
+            thin_asm.push_back((int32_t)first_item[e.second]);
+            thin_slot.push_back(slot_of[e.second]);
         }
         W.asm_cnt = (int32_t)(asm_items.size() - W.asm_off);
         W.thin_cnt = (int32_t)((int64_t)thin_list.size() - W.thin_off);

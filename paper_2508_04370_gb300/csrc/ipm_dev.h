@@ -316,6 +316,12 @@ constexpr int64_t kWarpRow = 32;       // and longer than this a warp each (rows
 // thin fronts (k <= nb, f <= kThinMaxF), one CTA per front: list[i] the front,
 // first_asm[i] its first assembly item, slots[i] its panel workspace slot
 constexpr int kThinMaxF = 512;
+// Thin fronts with children take that path only where a level has this many:
+// one CTA assembles its front block by block (0.5 to 2 ms with ten to a hundred
+// children of 300 rows), where the per-step launches spread the blocks over the
+// chip (40 block-angular blocks with 300 dense rows, three levels of 10 to 200
+// such fronts: 5.9 ms as thin fronts, 1.2 through the steps).
+constexpr int kThinInner = 1024;
 void launch_thin_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                         DevCtl *ctl, const int32_t *list, const int32_t *first_asm, const int32_t *slots,
                         const AsmLists &A, double *pws, int32_t count, int32_t nb, cudaStream_t st);

@@ -314,13 +314,13 @@ constexpr int kPoolDoubles = 2 * 32 * 33 + 32;  // a 32 x 32 update tile's two o
 // children's order without CTA barriers, the next child's maps fetched
 // while this one's entries arrive.  50-period staircase: the assembly launches
 // of a factorisation take 5.6 ms instead of 23.7 (10.8 GB).
-__device__ __forceinline__ void body_assemble(const DevPlan &P, const DevVals &V, double *__restrict__ fronts,
-                                              const AsmLists &A, const AsmItem &ai, double *pool) {
+template <class Out>  // out(r, c, v): stores the assembled value v of front entry (r, c)
+__device__ __forceinline__ void assemble_block(const DevPlan &P, const DevVals &V, const double *fronts,
+                                               const AsmLists &A, const AsmItem &ai, double *pool, Out out) {
     constexpr int NT = kBodyThreads, R = kAsmRows;
     static_assert(32 * R <= kPoolDoubles && NT / 32 == 8, "the block fits the pool, four columns per warp");
     double *T = pool;  // column c, row r at T[R (c - c_lo) + r % R]
-    const int s = ai.s, ld = P.sn_ld[s];
-    double *F = fronts + P.sn_off[s];
+    const int ld = P.sn_ld[ai.s];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c_lo = ai.c_lo, r_lo = ai.r_lo, r_hi = ai.r_hi, rbase = r_lo & ~(R - 1);
 #pragma unroll
@@ -398,8 +398,15 @@ __device__ __forceinline__ void body_assemble(const DevPlan &P, const DevVals &V
     __syncthreads();
     for (int t = tid; t < 32 * R; t += NT) {
         const int c = c_lo + t / R, r = rbase + t % R;
-        if (c < ai.c_hi && r >= r_lo && r < r_hi) F[(int64_t)c * ld + r] = T[t];
+        if (c < ai.c_hi && r >= r_lo && r < r_hi) out(r, c, T[t]);
     }
+}
+
+__device__ __forceinline__ void body_assemble(const DevPlan &P, const DevVals &V, double *__restrict__ fronts,
+                                              const AsmLists &A, const AsmItem &ai, double *pool) {
+    const int ld = P.sn_ld[ai.s];
+    double *F = fronts + P.sn_off[ai.s];
+    assemble_block(P, V, fronts, A, ai, pool, [&](int r, int c, double v) { F[(int64_t)c * ld + r] = v; });
 }
 
 // The nb x nb diagonal block of panel [p0, p0 + nb) of front s as a
@@ -934,12 +941,20 @@ __global__ void __launch_bounds__(kBodyThreads) k_large_update_strip(DevPlan P, 
     body_strip(P, fronts, Dg, it.s, it.i0, it.j0, it.p0, w, pool);
 }
 
-// A thin front (one pivot block, k <= nb, f <= kThinMaxF) whole in one CTA:
-// the same bodies as the one-launch-per-step kernels, called in sequence
-// (assembly by 32-column blocks, the diagonal block, the triangular solve in
-// 32-row items, the trailing 32 x 32 tiles), so the front's values are
-// those of the per-step path bit for bit; a level of many such fronts costs
-// one launch instead of one per body and item.
+// A thin front (one pivot block, k <= nb, f <= kThinMaxF) whole in one CTA.
+// Every entry gets the operations of the per-step path in its order, so the
+// front's values are those of that path bit for bit; what differs is what
+// moves: the rows of L and L d are kept in shared memory, the contribution
+// block is formed and written in one pass (0 minus the products where the front
+// has no children, assembled and updated block by block in shared memory
+// otherwise), and up to kThinCols pivot columns a thread solves a row by
+// itself.  With the per-step bodies in sequence a leaf of one column and 302
+// rows took about 0.9 ms of a CTA's time in barriers and round trips; now its
+// 46,000 products bound it (FP64, two per clock and SM).  40 block-angular
+// blocks with 300 dense rows: the launch of 8,317 leaves takes 3.4 ms (1.1 at the
+// FP64 rate), 17 ms with all thin fronts in the per-step bodies' sequence.
+constexpr int kThinCols = 4;
+constexpr int kThinPanel = 6144;  // doubles of L kept (three CTAs per SM fit)
 __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevVals V, double *__restrict__ fronts,
                                                                double *__restrict__ Dg, double *__restrict__ Dig,
                                                                double *__restrict__ dyng, DevCtl *ctl,
@@ -947,29 +962,113 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
                                                                const int32_t *__restrict__ first_asm,
                                                                const int32_t *__restrict__ slots,
                                                                AsmLists A, double *__restrict__ pws, int nb) {
+    extern __shared__ double panel[];
     __shared__ double pool[kPoolDoubles];
+    __shared__ double Bt[32][33];  // L(c, q) d_q of a block's columns
     const int s = list[blockIdx.x];
-    const int f = P.sn_f[s], k = P.sn_k[s];
+    const int f = P.sn_f[s], k = P.sn_k[s], ld = P.sn_ld[s], c0 = P.sn_c0[s];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    double *F = fronts + P.sn_off[s];
     const int64_t a0 = first_asm[blockIdx.x];
-    for (int a = 0, na = asm_tiles(f); a < na; a++) {
-        const AsmItem ai = A.items[a0 + a];
-        body_assemble(P, V, fronts, A, ai, pool);
+    const bool leaf = P.child_ptr[s] == P.child_ptr[s + 1];
+    const int nr = (f + kAsmRows - 1) / kAsmRows;  // the first column block's items
+    if (leaf) {
+        // originals lie in the pivot columns
+        for (int c = warp; c < k; c += kBodyThreads / 32)
+            for (int r = c + lane; r < f; r += 32) F[(int64_t)c * ld + r] = 0.0;
         __syncthreads();
+        for (int64_t q = P.orig_ptr[s] + tid; q < P.orig_ptr[s + 1]; q += kBodyThreads)
+            F[P.orig_dst[q]] = orig_value(P, V, P.orig_src[q]);
+        __syncthreads();
+    } else {
+        for (int a = 0; a < nr; a++) {
+            const AsmItem ai = A.items[a0 + a];
+            body_assemble(P, V, fronts, A, ai, pool);
+            __syncthreads();
+        }
     }
     double *ws = pws + (int64_t)slots[blockIdx.x] * kPanelWs;
     body_diag(P, V, fronts, Dg, Dig, dyng, ctl, s, 0, nb, ws, pool);
     __syncthreads();
-    // (one row per warp: the light variant keeps three CTAs per SM; these
-    // fronts' solves are short, k <= 32 columns)
-    for (int r0 = k; r0 < f; r0 += kTrsmRows) {
-        body_trsm<1>(P, fronts, s, r0, min(r0 + kTrsmRows, f), 0, nb, ws, pool);
+    if (k <= kThinCols) {
+        // u_q = F_iq - sum_{q' < q} u_q' L_qq', l_q = u_q / d_q
+        for (int i = k + tid; i < f; i += kBodyThreads) {
+            double u[kThinCols];
+#pragma unroll
+            for (int q = 0; q < kThinCols; q++) {
+                u[q] = q < k ? F[(int64_t)q * ld + i] : 0.0;
+#pragma unroll
+                for (int c = 0; c < q; c++)
+                    if (q < k) u[q] -= u[c] * ws[q * 33 + c];
+            }
+#pragma unroll
+            for (int q = 0; q < kThinCols; q++)
+                if (q < k) F[(int64_t)q * ld + i] = u[q] * ws[32 * 33 + q];
+        }
         __syncthreads();
-    }
-    for (int j0 = k; j0 < f; j0 += kUpdTile)
-        for (int i0 = j0; i0 < f; i0 += kUpdTile) {
-            body_tile(P, fronts, Dg, s, i0, j0, 0, nb, pool);
+    } else {
+        for (int r0 = k; r0 < f; r0 += kTrsmRows) {
+            body_trsm<1>(P, fronts, s, r0, min(r0 + kTrsmRows, f), 0, nb, ws, pool);
             __syncthreads();
         }
+    }
+    // the rows of L: in shared memory where they fit
+    const bool kept = k * f <= kThinPanel;
+    const double *Lp = kept ? panel : F;
+    const int ls = kept ? f : ld;
+    if (kept) {
+        for (int q = 0; q < k; q++)
+            for (int i = k + tid; i < f; i += kBodyThreads) panel[q * f + i] = F[(int64_t)q * ld + i];
+        __syncthreads();
+    }
+    // columns of the contribution block with nothing assembled beside them: all
+    // of a leaf's, else those of the first block (whose values are in the slab)
+    const int c_end = leaf ? f : min(32, f);
+    const double dq = lane < k ? Dg[c0 + lane] : 0.0;
+    for (int j = k + warp; j < c_end; j += kBodyThreads / 32) {
+        const double b = lane < k ? Lp[lane * ls + j] * dq : 0.0;
+        constexpr int U = 4;  // rows a lane carries together
+        for (int i0 = j + lane; i0 - lane < f; i0 += 32 * U) {
+            double acc[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) acc[u] = 0.0;
+            for (int q = 0; q < k; q++) {
+                const double bq = __shfl_sync(0xffffffffu, b, q);
+                const double *Lq = Lp + q * ls + i0;
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    if (i0 - lane + 32 * u < f) acc[u] += (i0 + 32 * u < f ? Lq[32 * u] : 0.0) * bq;
+            }
+            double *e = F + (int64_t)j * ld + i0;
+#pragma unroll
+            for (int u = 0; u < U; u++) {
+                if (i0 + 32 * u >= f) continue;
+                if (leaf) {
+                    // 0 - acc without an FP64 instruction (0 - 0 is +0)
+                    const long long bits = dbits(acc[u]);
+                    e[32 * u] = (bits & kAbsMask) ? __longlong_as_double(bits ^ kSignBit) : 0.0;
+                } else {
+                    e[32 * u] = e[32 * u] - acc[u];
+                }
+            }
+        }
+    }
+    if (leaf) return;
+    for (int a = nr, na = asm_tiles(f); a < na; a++) {
+        const AsmItem ai = A.items[a0 + a];
+        __syncthreads();
+        for (int t = tid; t < 32 * k; t += kBodyThreads) {
+            const int q = t >> 5, c = ai.c_lo + (t & 31);
+            Bt[t & 31][q] = c < f ? Lp[q * ls + c] * Dg[c0 + q] : 0.0;
+        }
+        assemble_block(P, V, fronts, A, ai, pool, [&](int r, int c, double v) {
+            if (r < c) return;
+            const double *b = Bt[c - ai.c_lo];
+            double acc = 0.0;
+            for (int q = 0; q < k; q++) acc += Lp[q * ls + r] * b[q];
+            F[(int64_t)c * ld + r] = v - acc;
+        });
+    }
 }
 
 // Persistent level kernel: all large-front items of one tree level in one
@@ -1461,7 +1560,11 @@ void launch_thin_fronts(const DevPlan &P, const DevVals &V, double *fronts, doub
                         DevCtl *ctl, const int32_t *list, const int32_t *first_asm, const int32_t *slots,
                         const AsmLists &A, double *pws, int32_t count, int32_t nb, cudaStream_t st) {
     if (count <= 0) return;
-    k_thin_fronts<<<count, kBodyThreads, 0, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, first_asm, slots, A, pws, nb);
+    static uint64_t attr = 0;
+    constexpr int smem = kThinPanel * (int)sizeof(double);
+    if (first_on_device(attr))
+        cudaFuncSetAttribute(k_thin_fronts, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    k_thin_fronts<<<count, kBodyThreads, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, first_asm, slots, A, pws, nb);
 }
 
 void launch_large_level(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,

@@ -56,3 +56,36 @@ def test_children_at_class_and_block_edges(pkg, m, lengths):
         else:
             assert np.array_equal(base["D"], r["D"]) and np.array_equal(base["L"], r["L"])
         r["s"].close()
+
+
+def lp_with_thin_fronts(nlink, groups, private, seed):
+    """One column per group with `private` rows of its own and nlink dense rows:
+    leaves of 1 + private pivots and nlink more rows."""
+    rng = np.random.default_rng(seed)
+    rows, cols = [], []
+    for g in range(groups):
+        rows += list(private * g + np.arange(private)) + list(private * groups + np.arange(nlink))
+        cols += [g] * (private + nlink)
+    return _from_coo(private * groups + nlink, groups, rows, cols, rng.standard_normal(len(rows)), "thin")
+
+
+@pytest.mark.parametrize("nlink,groups,private", [(129, 6, 0), (130, 5, 3), (161, 4, 4), (300, 3, 12), (150, 3, 31),
+                                                  (490, 2, 20)])
+def test_thin_fronts(pkg, nlink, groups, private):
+    lp = lp_with_thin_fronts(nlink, groups, private, nlink)
+    theta = synth.theta_loguniform(lp.n, 5, -2.0, 2.0)
+    r7, r1 = synth.rhs_normal(lp.n, 6), synth.rhs_normal(lp.m, 7)
+    # each column first, then its private rows, then the dense rows
+    perm = [v for g in range(groups) for v in [g] + [lp.n + private * g + i for i in range(private)]]
+    perm = np.array(perm + list(lp.n + private * groups + np.arange(nlink)), dtype=np.int32)
+    base = None
+    for opts in (dict(schedule=pkg.IPM_SCHED_LEVELS, level_kernel=0), dict(schedule=pkg.IPM_SCHED_DEPENDENCY)):
+        r = run_pair(pkg, lp, theta, r7, r1, ordering=pkg.IPM_ORD_USER, user_perm=perm, amalg_zero_frac=0.0,
+                     **opts)
+        assert r["info"]["nfronts_thin"] > 0
+        check_pair(r, lp)
+        if base is None:
+            base = r
+        else:
+            assert np.array_equal(base["D"], r["D"]) and np.array_equal(base["L"], r["L"])
+        r["s"].close()
