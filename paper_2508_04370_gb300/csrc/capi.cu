@@ -105,6 +105,7 @@ struct ipm_ctx {
     int64_t device_bytes = 0;
     DevPlan dp{};
     DevCtl *ctl = nullptr;
+    DevCtl *h_ctl = nullptr;  // pinned: where the control block is read back to
     double *fronts = nullptr, *D = nullptr, *Dinv = nullptr, *dyn = nullptr;
     double *Doff = nullptr;      // pivoting mode: D(p+1, p) of 2x2 blocks
     int32_t *bsz = nullptr;      // pivoting mode: block sizes (1, 2, 0 at a 2x2 block's second position)
@@ -508,6 +509,8 @@ void free_device(ipm_ctx *c) {
     c->ev_pool.clear();
     c->ev_used = 0;
     c->prof_pending.clear();
+    if (c->h_ctl) cudaFreeHost(c->h_ctl);
+    c->h_ctl = nullptr;
     if (c->h_r7) cudaFreeHost(c->h_r7);
     c->h_r7 = nullptr;
     c->device_bytes = 0;
@@ -649,7 +652,7 @@ int build_solve_schedule(ipm_ctx *c, const std::vector<int32_t> &fwd_order, cons
     int32_t *d_fleaf, *d_bleaf;
     int rc;
     if ((rc = dupload(c, &d_nodes, nodes)) || (rc = dupload(c, &d_grp, grp)) || (rc = dupload(c, &d_gsrc, gsrc)) ||
-        (rc = dupload(c, &d_fwd, fwd)) || (rc = dupload(c, &d_bwd, bwd)) || (rc = dalloc(c, &d_yv, (size_t)P.N)) ||
+        (rc = dupload(c, &d_fwd, fwd)) || (rc = dupload(c, &d_bwd, bwd)) || (rc = dalloc(c, &d_yv, 2 * (size_t)P.N)) ||
         (rc = dalloc(c, &d_rpart, (size_t)nrpart)) ||
         (rc = dupload(c, &d_fleaf, fleaf)) || (rc = dupload(c, &d_bleaf, bleaf)) ||
         (rc = dupload(c, &c->inv_items, inv_items)) || (rc = dupload(c, &c->pair_items, pair_items)) ||
@@ -668,14 +671,18 @@ int build_solve_schedule(ipm_ctx *c, const std::vector<int32_t> &fwd_order, cons
     S.nfwd = (int32_t)fwd.size();
     S.nbwd = (int32_t)bwd.size();
     S.nsuper = ns;
-    S.sync = c->solve_sync;
-    S.yv = d_yv;
+    S.sync[0] = c->solve_sync;
+    S.sync[1] = c->solve_sync + 2 * ns + 1;
+    S.yv[0] = d_yv;
+    S.yv[1] = d_yv + P.N;
     S.nyv = P.N;
     S.rpart = d_rpart;
     S.nrpart = nrpart;
     S.fwd_leaf = d_fleaf;
     S.bwd_leaf = d_bleaf;
     S.Linv = c->linv;
+    launch_sweep_reset(S, 0);
+    if (cudaStreamSynchronize(0) != cudaSuccess) return to_err(cudaGetLastError());
     c->solve_maxf = single_maxf;
     c->solve_grid = std::max(1, std::min(std::max(S.nfwd, S.nbwd), c->sms * solve_ctas_per_sm(single_maxf)));
     return IPM_OK;
@@ -1270,7 +1277,7 @@ int setup_device(ipm_ctx *c) {
         (rc = dalloc(c, &c->slice_ws, 3 * (size_t)max_slice_blocks * (size_t)kSliceBlockBytes)) ||
         (rc = dalloc(c, &c->slice_exp, 3 * (size_t)std::max<int64_t>(max_slice_blocks, 1) * kSliceRows * 2)) ||
         (rc = dupload(c, &c->lvl_items, lvl_items)) || (rc = dalloc(c, &c->lvl_sync, (size_t)max_ncnt + 1)) ||
-        (rc = dalloc(c, &c->solve_sync, (size_t)3 * ns + 1)))
+        (rc = dalloc(c, &c->solve_sync, 2 * ((size_t)2 * ns + 1))))
         return rc;
     c->slice_part_blocks = max_slice_blocks;
     int32_t *d_sparent, *d_long, *d_mid;
@@ -1407,6 +1414,11 @@ int setup_device(ipm_ctx *c) {
         c->ne.Apos = d_apos;
         c->ne.Acp = d_acp;
         c->ne.Ari = d_ari;
+    }
+    if (!c->h_ctl && cudaMallocHost(&c->h_ctl, sizeof(DevCtl)) != cudaSuccess) {
+        cudaGetLastError();
+        c->h_ctl = nullptr;
+        return IPM_ERR_OOM;
     }
     cudaMemset(c->ctl, 0, sizeof(DevCtl));
     cudaMemset(c->fronts, 0, (size_t)std::max<int64_t>(P.front_doubles, 1) * sizeof(double));
@@ -1767,12 +1779,13 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
     return to_err(cudaGetLastError());
 }
 
-// x <- (L D L^T)^-1 x in the factorisation order: one persistent launch per
-// sweep (dependency-driven, see kernels_solve.cu).
-int solve_inplace(ipm_ctx *c, double *x, cudaStream_t st, int *nl) {
+// x <- (L D L^T)^-1 b in the factorisation order (b != x): one persistent launch
+// per sweep (dependency-driven, see kernels_solve.cu).
+int solve_sweeps(ipm_ctx *c, const double *b, double *x, cudaStream_t st, int *nl) {
     const Plan &P = c->plan;
     if (c->opt.pivoting) {
         // per-level sweeps with the fronts' interchanges and 1x1 / 2x2 blocks of D
+        cudaMemcpyAsync(x, b, P.N * sizeof(double), cudaMemcpyDeviceToDevice, st);
         for (int32_t l = 0; l < P.nlevels; l++) {
             const LevelWork &W = c->levels[l];
             Prof pr(c, IPM_K_FORWARD, W.fwd_w, st);
@@ -1796,38 +1809,34 @@ int solve_inplace(ipm_ctx *c, double *x, cudaStream_t st, int *nl) {
     }
     {
         Prof pr(c, IPM_K_FORWARD, fw, st);
-        launch_forward_persistent(c->sched, c->fronts, c->Dinv, x, c->upd, c->solve_maxf, c->solve_grid, c->ctl, st);
+        launch_forward_persistent(c->sched, c->fronts, c->Dinv, b, x, c->upd, c->solve_maxf, c->solve_grid, c->ctl, st);
     }
     {
         Prof pr(c, IPM_K_BACKWARD, bw, st);
         launch_backward_persistent(c->sched, c->fronts, x, c->solve_grid, c->ctl, st);
     }
-    *nl += 4;  // per sweep: the reset of its counters and chain values, then the sweep
+    *nl += 2;
     return to_err(cudaGetLastError());
 }
 
-// The GMRES refinement of a captured graph: a conditional node whose body
-// (captured on a second stream) runs only when classical refinement ended
-// above the target; inside it every kernel tests the device-side flags of
-// GmDev, so cycles and Arnoldi steps that are not needed return at entry.
-int capture_gmres(ipm_ctx *c, cudaStream_t st) {
-    const Plan &P = c->plan;
-    const int64_t N = P.N;
-    const int m = kGmresM;
-    const double target = c->opt.omega_target;
-    const int R = c->opt.gmres_restarts;
-    GmDev *gm = c->gm_dev;
+// A conditional node in the graph that `st` is capturing: the handle first (for
+// the kernel that sets the condition), then the node, whose body is captured
+// on a second stream until cudaStreamEndCapture.
+int conditional_handle(cudaStream_t st, cudaGraphConditionalHandle *h) {
+    cudaStreamCaptureStatus cs;
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, nullptr, nullptr, nullptr);
+    if (e != cudaSuccess || cs != cudaStreamCaptureStatusActive) return IPM_ERR_CUDA;
+    return to_err(cudaGraphConditionalHandleCreate(h, g, 0, 0));
+}
+int conditional_open(ipm_ctx *c, cudaStream_t st, cudaGraphConditionalHandle h, cudaStream_t *body_stream) {
     cudaStreamCaptureStatus cs;
     cudaGraph_t g = nullptr;
     const cudaGraphNode_t *deps = nullptr;
     const cudaGraphEdgeData *ed = nullptr;
     size_t nd = 0;
-    cudaError_t e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, nullptr, nullptr, nullptr);
-    if (e != cudaSuccess || cs != cudaStreamCaptureStatusActive) return IPM_ERR_CUDA;
-    cudaGraphConditionalHandle h;
-    if ((e = cudaGraphConditionalHandleCreate(&h, g, 0, 0)) != cudaSuccess) return to_err(e);
-    launch_gm_begin(c->ctl, gm, target, (unsigned long long)h, st);
-    if ((e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, &deps, &ed, &nd)) != cudaSuccess) return to_err(e);
+    cudaError_t e = cudaStreamGetCaptureInfo(st, &cs, nullptr, &g, &deps, &ed, &nd);
+    if (e != cudaSuccess) return to_err(e);
     cudaGraphNodeParams prm{};
     prm.type = cudaGraphNodeTypeConditional;
     prm.conditional.handle = h;
@@ -1843,14 +1852,36 @@ int capture_gmres(ipm_ctx *c, cudaStream_t st) {
         c->gm_stream = nullptr;
         return to_err(e);
     }
-    cudaStream_t s2 = c->gm_stream;
-    if ((e = cudaStreamBeginCaptureToGraph(s2, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed)) !=
-        cudaSuccess)
-        return to_err(e);
-    launch_copy_if(c->vx, c->vbest, (int32_t)N, nullptr, 0, s2);
+    *body_stream = c->gm_stream;
+    return to_err(cudaStreamBeginCaptureToGraph(c->gm_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+}
+int conditional_close(cudaStream_t body_stream) {
+    cudaGraph_t out = nullptr;
+    const cudaError_t e1 = cudaGetLastError(), e = cudaStreamEndCapture(body_stream, &out);
+    return to_err(e1 != cudaSuccess ? e1 : e);
+}
+
+// The GMRES refinement of a captured graph: a conditional node whose body
+// runs only when classical refinement ended above the target; inside it every
+// kernel tests the device-side flags of GmDev, so cycles and Arnoldi steps that
+// are not needed return at entry.
+int capture_gmres(ipm_ctx *c, cudaStream_t st) {
+    const Plan &P = c->plan;
+    const int64_t N = P.N;
+    const int m = kGmresM;
+    const double target = c->opt.omega_target;
+    const int R = c->opt.gmres_restarts;
+    GmDev *gm = c->gm_dev;
+    cudaGraphConditionalHandle h;
+    cudaStream_t s2;
+    int rc;
+    if ((rc = conditional_handle(st, &h))) return rc;
+    launch_gm_begin(c->ctl, gm, target, (unsigned long long)h, st);
+    if ((rc = conditional_open(c, st, h, &s2))) return rc;
+    launch_best_both(c->vx, c->vbest, (int32_t)N, c->ctl, s2);
     for (int r = 0; r <= R; r++) {
         // r = f - K x and omega of the current x; keep it if it improved
-        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, s2, &gm->stop);
+        launch_residual_omega(c->dp, c->vf, c->vx, nullptr, nullptr, c->vr, c->vad, c->ctl, s2, &gm->stop, true);
         launch_gm_cycle(c->ctl, gm, target, r, R, s2);
         launch_copy_if(c->vbest, c->vx, (int32_t)N, &gm->improved, 0, s2);
         if (r == R) break;
@@ -1859,12 +1890,11 @@ int capture_gmres(ipm_ctx *c, cudaStream_t st) {
         launch_scale_dev(c->gm_V, c->vr, gm, NAN, N, &gm->stop, s2);
         for (int j = 0; j < m; j++) {
             double *vj = c->gm_V + (int64_t)j * N, *zj = c->gm_Z + (int64_t)j * N, *vn = vj + N;
-            launch_copy_if(zj, vj, (int32_t)N, &gm->skip_inner, 1, s2);
-            launch_forward_persistent(c->sched, c->fronts, c->Dinv, zj, c->upd, c->solve_maxf, c->solve_grid, c->ctl,
-                                      s2, &gm->skip_inner);
+            launch_forward_persistent(c->sched, c->fronts, c->Dinv, vj, zj, c->upd, c->solve_maxf, c->solve_grid,
+                                      c->ctl, s2, &gm->skip_inner);
             launch_backward_persistent(c->sched, c->fronts, zj, c->solve_grid, c->ctl, s2,
                                        &gm->skip_inner);
-            launch_residual_omega(c->dp, c->gm_zero, zj, c->gm_w, c->vad, c->ctl, s2, &gm->skip_inner);
+            launch_residual_omega(c->dp, c->gm_zero, zj, nullptr, nullptr, c->gm_w, c->vad, c->ctl, s2, &gm->skip_inner);
             launch_scale_dev(vn, c->gm_w, gm, -1.0, N, &gm->skip_inner, s2);  // K z
             for (int pass = 0; pass < 2; pass++) {
                 launch_dots(vn, c->gm_V, N, j + 1, c->gm_part, gm->h, s2, &gm->skip_inner);
@@ -1879,13 +1909,8 @@ int capture_gmres(ipm_ctx *c, cudaStream_t st) {
         launch_combine_dev(c->vx, c->gm_Z, gm, N, s2);
     }
     launch_gm_end(c->ctl, gm, s2);
-    cudaGraph_t out = nullptr;
-    const cudaError_t e1 = cudaGetLastError();
-    e = cudaStreamEndCapture(s2, &out);
-    if (e1 != cudaSuccess) return to_err(e1);
-    return to_err(e);
+    return conditional_close(s2);
 }
-
 
 // GMRES refines an FP64-accurate factor (FP64 or sliced updates); a stalled
 // 3xTF32 factor is replaced by an FP64 one instead
@@ -1899,35 +1924,43 @@ bool gmres_allowed(const ipm_ctx *c) {
 // done (omega <= target, omega failed to halve, or the step limit).
 int solve_device_driven(ipm_ctx *c, const double *r7, const double *r1, double *dx, double *dy, cudaStream_t st) {
     const Plan &P = c->plan;
-    const int32_t N = P.N;
     const int32_t *done = &c->ctl->done;
-    const int32_t *improved = &c->ctl->improved;
     const double target = c->opt.omega_target;
     const int32_t rmax = c->opt.refine_max;
     if (P.form == 2) launch_ne_rhs(c->ne, c->dp.perm, c->Ax, r7, r1, c->vf, st);
     else launch_permute_in(c->dp, r7, r1, c->vf, st);
-    launch_copy_if(c->vx, c->vf, N, nullptr, 0, st);
-    launch_forward_persistent(c->sched, c->fronts, c->Dinv, c->vx, c->upd, c->solve_maxf, c->solve_grid, c->ctl, st);
-    launch_backward_persistent(c->sched, c->fronts, c->vx, c->solve_grid, c->ctl, st);
-    launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
+    double *x[2] = {c->vx, c->vbest};
+    launch_forward_persistent(c->sched, c->fronts, c->Dinv, c->vf, x[0], c->upd, c->solve_maxf, c->solve_grid, c->ctl, st);
+    launch_backward_persistent(c->sched, c->fronts, x[0], c->solve_grid, c->ctl, st);
+    launch_residual_omega(c->dp, c->vf, x[0], nullptr, nullptr, c->vr, c->vad, c->ctl, st);
     launch_refine_init(c->ctl, target, rmax, st);
-    launch_copy_if(c->vbest, c->vx, N, nullptr, 0, st);
-    for (int32_t step = 1; step <= rmax; step++) {
-        launch_copy_if(c->vc, c->vr, N, done, 1, st);
-        launch_forward_persistent(c->sched, c->fronts, c->Dinv, c->vc, c->upd, c->solve_maxf, c->solve_grid, c->ctl, st,
-                                  done);
-        launch_backward_persistent(c->sched, c->fronts, c->vc, c->solve_grid, c->ctl, st, done);
-        launch_axpy(c->vx, c->vc, N, st, done);
-        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st, done);
-        launch_refine_step(c->ctl, target, step, rmax, st);
-        launch_copy_if(c->vbest, c->vx, N, improved, 0, st);
+    auto refine = [&](int32_t step, cudaStream_t q, unsigned long long handle) {
+        launch_forward_persistent(c->sched, c->fronts, c->Dinv, c->vr, c->vc, c->upd, c->solve_maxf, c->solve_grid, c->ctl,
+                                  q, done);
+        launch_backward_persistent(c->sched, c->fronts, c->vc, c->solve_grid, c->ctl, q, done);
+        launch_residual_omega(c->dp, c->vf, x[(step - 1) & 1], c->vc, x[step & 1], c->vr, c->vad, c->ctl, q, done);
+        launch_refine_step(c->ctl, target, step, rmax, q, handle);
+    };
+    // a few steps in line, the others in a conditional node: a launch that
+    // returns at entry costs a replay about a microsecond, and most solves need
+    // three steps at most
+    constexpr int32_t kInline = 3;
+    int rc = 0;
+    cudaGraphConditionalHandle h = 0;
+    if (rmax > kInline && (rc = conditional_handle(st, &h))) return rc;
+    for (int32_t step = 1; step <= std::min(rmax, kInline); step++)
+        refine(step, st, step == kInline ? (unsigned long long)h : 0);
+    if (rmax > kInline) {
+        cudaStream_t s2;
+        if ((rc = conditional_open(c, st, h, &s2))) return rc;
+        for (int32_t step = kInline + 1; step <= rmax; step++) refine(step, s2, 0);
+        if ((rc = conditional_close(s2))) return rc;
     }
     if (c->gm_dev && gmres_allowed(c)) {
-        int rc = capture_gmres(c, st);
-        if (rc) return rc;
+        if ((rc = capture_gmres(c, st))) return rc;
     }
     launch_refine_finish(c->ctl, target, st);
-    launch_permute_out(c->dp, c->vbest, dx, dy, st);
+    launch_permute_out(c->dp, x[0], dx, dy, st, x[1], &c->ctl->best);
     if (P.form == 2) launch_ne_dx(c->ne, c->Ax, dy, r7, dx, st);
     return to_err(cudaGetLastError());
 }
@@ -2290,9 +2323,10 @@ done:
 }
 
 static int read_ctl(ipm_ctx *c, cudaStream_t st, DevCtl *h) {
-    cudaError_t e = cudaMemcpyAsync(h, c->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaMemcpyAsync(c->h_ctl, c->ctl, sizeof(DevCtl), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return to_err(e);
+    *h = *c->h_ctl;
     c->status_acc |= h->status;
     return IPM_OK;
 }
@@ -2362,8 +2396,8 @@ static int gmres_refine(ipm_ctx *c, cudaStream_t st, double &wbest, int *nl) {
     cudaMemcpyAsync(c->vx, c->vbest, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
     for (int restart = 0; restart <= c->opt.gmres_restarts; restart++) {
         // r = f - K x and omega of the current x
-        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
-        *nl += 2;
+        launch_residual_omega(c->dp, c->vf, c->vx, nullptr, nullptr, c->vr, c->vad, c->ctl, st, nullptr, true);
+        *nl += 3;
         DevCtl h{};
         if ((rc = read_ctl(c, st, &h))) return rc;
         if (h.status & kStatNonFinite) break;
@@ -2389,9 +2423,8 @@ static int gmres_refine(ipm_ctx *c, cudaStream_t st, double &wbest, int *nl) {
         int jdone = 0;
         for (int j = 0; j < m; j++) {
             double *vj = c->gm_V + (int64_t)j * N, *zj = c->gm_Z + (int64_t)j * N, *vn = vj + N;
-            cudaMemcpyAsync(zj, vj, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
-            if ((rc = solve_inplace(c, zj, st, nl))) return rc;
-            launch_residual_omega(c->dp, c->gm_zero, zj, c->gm_w, c->vad, c->ctl, st);  // -K z
+            if ((rc = solve_sweeps(c, vj, zj, st, nl))) return rc;
+            launch_residual_omega(c->dp, c->gm_zero, zj, nullptr, nullptr, c->gm_w, c->vad, c->ctl, st);  // -K z
             launch_scale(vn, c->gm_w, -1.0, N, st);
             *nl += 3;
             for (int pass = 0; pass < 2; pass++) {
@@ -2448,36 +2481,34 @@ static int solve_once(ipm_ctx *c, const double *r7, const double *r1, double *dx
     if (P.form == 2) launch_ne_rhs(c->ne, c->dp.perm, c->Ax, r7, r1, c->vf, st);  // r8 = r1 + A Theta~ r7
     else launch_permute_in(c->dp, r7, r1, c->vf, st);
     nl++;
-    cudaMemcpyAsync(c->vx, c->vf, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
-    if ((rc = solve_inplace(c, c->vx, st, &nl))) return rc;
+    double *x[2] = {c->vx, c->vbest};  // the best iterate, and the one formed from it
+    if ((rc = solve_sweeps(c, c->vf, x[0], st, &nl))) return rc;
+    const bool clear = c->opt.pivoting;  // (the persistent backward sweep clears the norms)
     {
         Prof pr(c, IPM_K_RESIDUAL, c->resid_w, st);
-        launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
+        launch_residual_omega(c->dp, c->vf, x[0], nullptr, nullptr, c->vr, c->vad, c->ctl, st, nullptr, clear);
     }
-    nl += 2;
+    nl += clear ? 3 : 2;
     DevCtl h{};
     if ((rc = read_ctl(c, st, &h))) return rc;
     double wbest = h.omega;
-    cudaMemcpyAsync(c->vbest, c->vx, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
-    int steps = 0;
+    int steps = 0, cur = 0;
     c->omega_hist[0] = h.omega;
     const double target = c->opt.omega_target;
     while (wbest > target && steps < c->opt.refine_max && !(h.status & kStatNonFinite)) {
-        cudaMemcpyAsync(c->vc, c->vr, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
-        if ((rc = solve_inplace(c, c->vc, st, &nl))) return rc;
-        launch_axpy(c->vx, c->vc, N, st);
+        if ((rc = solve_sweeps(c, c->vr, c->vc, st, &nl))) return rc;
         {
             Prof pr(c, IPM_K_RESIDUAL, c->resid_w, st);
-            launch_residual_omega(c->dp, c->vf, c->vx, c->vr, c->vad, c->ctl, st);
+            launch_residual_omega(c->dp, c->vf, x[cur], c->vc, x[1 - cur], c->vr, c->vad, c->ctl, st, nullptr, clear);
         }
-        nl += 3;
+        nl += clear ? 3 : 2;
         if ((rc = read_ctl(c, st, &h))) return rc;
         steps++;
         if (steps < 16) c->omega_hist[steps] = h.omega;
         const bool halved = h.omega <= 0.5 * wbest;
         if (h.omega < wbest) {
             wbest = h.omega;
-            cudaMemcpyAsync(c->vbest, c->vx, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
+            cur = 1 - cur;
         }
         if (!halved) break;
     }
@@ -2486,10 +2517,12 @@ static int solve_once(ipm_ctx *c, const double *r7, const double *r1, double *dx
     // later iterations keep, rather than paying GMRES iterations every solve
     c->gmres_iters = 0;
     if (wbest > target && gmres_allowed(c) && !(h.status & kStatNonFinite)) {
+        if (cur == 0) cudaMemcpyAsync(c->vbest, c->vx, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
+        cur = 1;
         if ((rc = gmres_refine(c, st, wbest, &nl))) return rc;
         steps += c->gmres_iters;
     }
-    launch_permute_out(c->dp, c->vbest, dx, dy, st);
+    launch_permute_out(c->dp, x[cur], dx, dy, st);
     nl++;
     c->refine_steps = steps;
     c->omega = wbest;
@@ -2984,7 +3017,7 @@ int ipm_solve_noalloc(ipm_ctx *c, const double *r7, const double *r1, double *dx
     launch_permute_in(c->dp, r7, r1, vf, st);
     cudaMemcpyAsync(vx, vf, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
     if ((rc = noalloc_sweeps(c, vx, upd, st))) return rc;
-    launch_residual_omega(c->dp, vf, vx, vr, vad, c->ctl, st);
+    launch_residual_omega(c->dp, vf, vx, nullptr, nullptr, vr, vad, c->ctl, st, nullptr, true);
     DevCtl h{};
     if ((rc = read_ctl(c, st, &h))) return rc;
     double wbest = h.omega;
@@ -2996,7 +3029,7 @@ int ipm_solve_noalloc(ipm_ctx *c, const double *r7, const double *r1, double *dx
         cudaMemcpyAsync(vc, vr, N * sizeof(double), cudaMemcpyDeviceToDevice, st);
         if ((rc = noalloc_sweeps(c, vc, upd, st))) return rc;
         launch_axpy(vx, vc, (int32_t)N, st);
-        launch_residual_omega(c->dp, vf, vx, vr, vad, c->ctl, st);
+        launch_residual_omega(c->dp, vf, vx, nullptr, nullptr, vr, vad, c->ctl, st, nullptr, true);
         if ((rc = read_ctl(c, st, &h))) return rc;
         steps++;
         if (steps < 16) c->omega_hist[steps] = h.omega;

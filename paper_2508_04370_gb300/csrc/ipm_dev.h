@@ -54,6 +54,7 @@ struct DevCtl {
     int32_t improved;      // the last step improved omega_best
     double omega_hist[16];
     int32_t gmres_iters;   // GMRES iterations of a graph-resident refinement
+    int32_t best;          // graph-resident refinement: which of its two iterates is the best
 };
 
 // Read-only plan arrays on the device (all indices in factorisation order).
@@ -166,10 +167,13 @@ struct SolveSched {
     const SolveItem *fwd, *bwd;
     int32_t nfwd, nbwd, nsuper;
     long long spin_limit;    // polls before a dependency wait gives up (kStatTimeout)
-    int32_t *sync;           // ticket + 2 x nsuper counters (forward: children done, items done;
-                             // backward: done flag, blocks done)
-    double *yv;              // the values split supernodes' blocks pass along their chain (y forward,
-                             // z backward), reset to an unset pattern before each sweep
+    // Per sweep (0 forward, 1 backward): ticket + 2 x nsuper counters (forward:
+    // children done, items done; backward: done flag, blocks done) and the values
+    // split supernodes' blocks pass along their chain (y forward, z backward),
+    // an unset pattern before the sweep.  Each sweep resets the other's at its
+    // start, so a pair of sweeps needs no reset launches.
+    int32_t *sync[2];
+    double *yv[2];
     int32_t nyv;
     double *rpart;           // backward sweep: the row chunks' sums, reset like yv
     int64_t nrpart;
@@ -357,11 +361,15 @@ void launch_backward(const DevPlan &P, const double *fronts, double *x, const in
                      int32_t maxf, cudaStream_t st);
 void launch_diag_inverse(const SolveSched &S, const double *fronts, double *Linv, const InvItem *items,
                          int32_t count, const InvItem *pairs, int32_t npairs, cudaStream_t st);
-void launch_forward_persistent(const SolveSched &S, const double *fronts, const double *Dinv, double *x, double *upd,
-                               int32_t maxf, int32_t grid, DevCtl *ctl, cudaStream_t st,
+// b: the right-hand side (not x); always followed by the backward sweep on x
+void launch_forward_persistent(const SolveSched &S, const double *fronts, const double *Dinv, const double *b, double *x,
+                               double *upd, int32_t maxf, int32_t grid, DevCtl *ctl, cudaStream_t st,
                                const int32_t *skip = nullptr);
+// (also clears ctl->dinf and ctl->omega for the residual that follows)
 void launch_backward_persistent(const SolveSched &S, const double *fronts, double *x, int32_t grid, DevCtl *ctl,
                                 cudaStream_t st, const int32_t *skip = nullptr);
+// both sweeps' counters and chain values to their state before a sweep
+void launch_sweep_reset(const SolveSched &S, cudaStream_t st);
 // GMRES refinement vectors (kernels_krylov.cu)
 constexpr int kMaxDots = 16;  // vectors per dot-product launch (restart length + 1 at most)
 constexpr int kGmresM = 8;    // GMRES restart length
@@ -414,14 +422,22 @@ void launch_omega_only(int32_t N, const double *r, const double *ad, const doubl
 // CTAs per SM of the persistent sweeps (maxf: the widest front that is one forward item)
 int32_t solve_ctas_per_sm(int32_t maxf);
 void launch_permute_in(const DevPlan &P, const double *r7, const double *r1, double *f, cudaStream_t st);
-void launch_permute_out(const DevPlan &P, const double *x, double *dx, double *dy, cudaStream_t st);
+// x1, sel: take x1 where *sel != 0
+void launch_permute_out(const DevPlan &P, const double *x, double *dx, double *dy, cudaStream_t st,
+                        const double *x1 = nullptr, const int32_t *sel = nullptr);
 // skip != nullptr: the kernels return at entry while *skip != 0 (graph-captured refinement)
-void launch_residual_omega(const DevPlan &P, const double *f, const double *x, double *r, double *ad, DevCtl *ctl,
-                           cudaStream_t st, const int32_t *skip = nullptr);
+// r = f - K (x + c), xn = x + c (c, xn null: r = f - K x); clear: not after a
+// backward sweep, which clears the norms
+void launch_residual_omega(const DevPlan &P, const double *f, const double *x, const double *c, double *xn, double *r,
+                           double *ad, DevCtl *ctl, cudaStream_t st, const int32_t *skip = nullptr, bool clear = false);
 void launch_axpy(double *x, const double *c, int32_t N, cudaStream_t st, const int32_t *skip = nullptr);
 void launch_refine_init(DevCtl *ctl, double target, int32_t max_steps, cudaStream_t st);
-void launch_refine_step(DevCtl *ctl, double target, int32_t step, int32_t max_steps, cudaStream_t st);
+// handle != 0: also sets a graph's conditional node to run while not done
+void launch_refine_step(DevCtl *ctl, double target, int32_t step, int32_t max_steps, cudaStream_t st,
+                        unsigned long long handle = 0);
 void launch_refine_finish(DevCtl *ctl, double target, cudaStream_t st);
+// both of a graph's iterates = the best one
+void launch_best_both(double *x0, double *x1, int32_t N, const DevCtl *ctl, cudaStream_t st);
 // dst = src when flag == nullptr or (*flag != 0) != invert
 void launch_copy_if(double *dst, const double *src, int32_t N, const int32_t *flag, int32_t invert, cudaStream_t st);
 

@@ -136,6 +136,7 @@ __global__ void k_gm_begin(DevCtl *ctl, GmDev *gm, double target, cudaGraphCondi
 
 // after r = f - K x and omega(x): keep x when it improved, decide whether to go on
 __global__ void k_gm_cycle(DevCtl *ctl, GmDev *gm, double target, int cycle, int last) {
+    if (cycle == 0) ctl->best = 1;  // the best iterate is kept in the second buffer from here on
     if (gm->stop) {
         gm->improved = 0;
         return;

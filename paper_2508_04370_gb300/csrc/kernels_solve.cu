@@ -330,11 +330,23 @@ __device__ __forceinline__ double poll_block(const double *p, int wp, DevCtl *ct
     return lane < wp ? v : 0.0;
 }
 
+// Sweep d's ticket and counters to zero, its chain values (and for the backward
+// sweep the row chunks' sums) to the unset pattern, by the grid of the other
+// sweep, which runs when d's last user has finished.
+__device__ __forceinline__ void reset_sweep(const SolveSched &S, int d) {
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    const double unset = __longlong_as_double((long long)kUnset);
+    for (int64_t i = i0; i < 2 * (int64_t)S.nsuper + 1; i += step) S.sync[d][i] = 0;
+    for (int64_t i = i0; i < S.nyv; i += step) S.yv[d][i] = unset;
+    if (d == 1)
+        for (int64_t i = i0; i < S.nrpart; i += step) S.rpart[i] = unset;
+}
+
 // Take the next ticket (thread 0) and publish its item and node to the CTA.
-__device__ __forceinline__ bool next_item(const SolveSched &S, const SolveItem *items, int nitems, SolveItem &it,
-                                          SolveNode &nd, SolveItem *sh_it, SolveNode *sh_nd) {
+__device__ __forceinline__ bool next_item(const SolveSched &S, int32_t *ticket, const SolveItem *items, int nitems,
+                                          SolveItem &it, SolveNode &nd, SolveItem *sh_it, SolveNode *sh_nd) {
     if (threadIdx.x == 0) {
-        const int t = atomicAdd(S.sync, 1);
+        const int t = atomicAdd(ticket, 1);
         SolveItem a{-1, -1};
         if (t < nitems) {
             a = items[t];
@@ -365,9 +377,9 @@ __device__ __forceinline__ void finish_forward(const SolveNode &nd, int s, int32
 
 // Row t of the front: its right-hand side (t < k) plus the children's
 // contributions, children ascending.
-__device__ __forceinline__ double gather_row(const SolveSched &S, const SolveNode &nd, const double *x,
+__device__ __forceinline__ double gather_row(const SolveSched &S, const SolveNode &nd, const double *b,
                                              const double *upd, int t) {
-    double a = t < nd.k ? x[nd.c0 + t] : 0.0;
+    double a = t < nd.k ? b[nd.c0 + t] : 0.0;
     const int64_t e1 = S.gat_rp[nd.rptr + t + 1];
     for (int64_t e = S.gat_rp[nd.rptr + t]; e < e1; e++) a += __ldcg(upd + S.gat_src[e]);
     return a;
@@ -499,13 +511,13 @@ __global__ void __launch_bounds__(256) k_pair_products(SolveSched S, const doubl
 // computes what the single-item path below computes, in the same order of
 // operations.
 __device__ __forceinline__ void leaf_forward(const SolveSched &S, int s, const double *__restrict__ fronts,
-                                             const double *__restrict__ Dinv, double *__restrict__ x, double *upd,
-                                             int32_t *cnt) {
+                                             const double *__restrict__ Dinv, const double *__restrict__ rhs,
+                                             double *__restrict__ x, double *upd, int32_t *cnt) {
     const int lane = threadIdx.x & 31;
     const SolveNode nd = S.node[s];
     const double *L = fronts + nd.off;
     const int f = nd.f, k = nd.k, ld = nd.ld, c0 = nd.c0;
-    double v = lane < k ? x[c0 + lane] : 0.0;
+    double v = lane < k ? rhs[c0 + lane] : 0.0;
     const double dinv = lane < k ? Dinv[c0 + lane] : 0.0;
     double acc = 0.0;  // rows below the block: sum_j L_ij y_j, subtracted at the end
     for (int j = 0; j < k; j++) {
@@ -623,6 +635,7 @@ __device__ __forceinline__ void apply_pair(const double *Mb, double *t, const do
 
 __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSched S, const double *__restrict__ fronts,
                                                                        const double *__restrict__ Dinv,
+                                                                       const double *__restrict__ rhs,
                                                                        double *__restrict__ x, double *upd,
                                                                        DevCtl *ctl, const int32_t *skip) {
     extern __shared__ double v[];
@@ -634,13 +647,15 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
     __shared__ SolveNode sh_nd;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (skip && *skip) return;
-    int32_t *cnt = S.sync + 1, *done = cnt + S.nsuper;
+    reset_sweep(S, 1);
+    double *yv = S.yv[0];
+    int32_t *cnt = S.sync[0] + 1, *done = cnt + S.nsuper;
     SolveItem it;
     SolveNode nd;
-    while (next_item(S, S.fwd, S.nfwd, it, nd, &sh_it, &sh_nd)) {
+    while (next_item(S, S.sync[0], S.fwd, S.nfwd, it, nd, &sh_it, &sh_nd)) {
         if (it.r == kLeafGroup) {
             const int ls = S.fwd_leaf[8 * it.s + warp];
-            if (ls >= 0) leaf_forward(S, ls, fronts, Dinv, x, upd, cnt);
+            if (ls >= 0) leaf_forward(S, ls, fronts, Dinv, rhs, x, upd, cnt);
             __syncthreads();
             continue;
         }
@@ -666,7 +681,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
                 for (int q = 0; q < 4; q++)
                     if (e0 + q < e1) g[q] = S.gat_src[e0 + q];
                 if (tid < w) {
-                    a0 = x[c0 + b0 + tid];
+                    a0 = rhs[c0 + b0 + tid];
                     dinv = Dinv[c0 + b0 + tid];
                 }
             }
@@ -680,7 +695,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
                 for (int64_t e = e0 + 4; e < e1; e++) a += __ldcg(upd + S.gat_src[e]);
                 v[tid] = a;
             }
-            for (int t = tid + kSolveThreads; t < nr; t += kSolveThreads) v[t] = gather_row(S, nd, x, upd, t);
+            for (int t = tid + kSolveThreads; t < nr; t += kSolveThreads) v[t] = gather_row(S, nd, rhs, upd, t);
             if (b > (pair ? 1 : 0)) {
                 // fan-in of the finished blocks b' < b (b' < b - 1 with W_b): warp w
                 // applies columns 4w..4w+3 of each
@@ -692,7 +707,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
 #pragma unroll
                     for (int c = 0; c < 4; c++)
                         lv[c] = lane < w ? L[(int64_t)(32 * bp + 4 * warp + c) * ld + b0 + lane] : 0.0;
-                    if (warp == 0) ys[bp & 1][lane] = poll_block(S.yv + c0 + 32 * bp, 32, ctl, S.spin_limit);
+                    if (warp == 0) ys[bp & 1][lane] = poll_block(yv + c0 + 32 * bp, 32, ctl, S.spin_limit);
                     __syncthreads();
                     if (lane < w) {
 #pragma unroll
@@ -714,7 +729,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
             __syncthreads();
             if (pair) {
                 // y_b = X_b v' - W_b y_{b-1}, y_{b-1} being the last block to finish
-                if (warp == 0) ys[0][lane] = poll_block(S.yv + c0 + 32 * (b - 1), 32, ctl, S.spin_limit);  // full block
+                if (warp == 0) ys[0][lane] = poll_block(yv + c0 + 32 * (b - 1), 32, ctl, S.spin_limit);  // full block
                 __syncthreads();
                 apply_pair(Wb, v, ys[0], part, w, false);
                 __syncthreads();
@@ -730,7 +745,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
             for (int q = tid; q < nr; q += kSolveThreads) {
                 if (q < w) {
                     const double y = v[q];
-                    if (!single) publish_value(S.yv + c0 + b0 + q, y);
+                    if (!single) publish_value(yv + c0 + b0 + q, y);
                     x[c0 + b0 + q] = y * dinv;  // q == tid here
                 } else {
                     __stcg(upd + nd.upd + (q - k), v[q]);
@@ -753,7 +768,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
             if (tid == 0) wait_count(&cnt[s], nd.nchild, ctl, S.spin_limit);
             __syncthreads();
             double u0 = 0.0;
-            if (warp == 0 && ok) u0 = gather_row(S, nd, x, upd, i);
+            if (warp == 0 && ok) u0 = gather_row(S, nd, rhs, upd, i);
             double acc = 0.0;
             for (int bp = 0; bp < nd.nblk; bp++) {
                 const int wp = min(32, k - 32 * bp);
@@ -761,7 +776,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_forward_persistent(SolveSc
 #pragma unroll
                 for (int c = 0; c < 4; c++)
                     lv[c] = (ok && 4 * warp + c < wp) ? L[(int64_t)(32 * bp + 4 * warp + c) * ld + i] : 0.0;
-                if (warp == 0) ys[bp & 1][lane] = poll_block(S.yv + c0 + 32 * bp, wp, ctl, S.spin_limit);
+                if (warp == 0) ys[bp & 1][lane] = poll_block(yv + c0 + 32 * bp, wp, ctl, S.spin_limit);
                 __syncthreads();
                 if (ok) {
 #pragma unroll
@@ -848,10 +863,16 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
     __shared__ SolveNode sh_nd;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (skip && *skip) return;
-    int32_t *flag = S.sync + 1, *tcnt = flag + S.nsuper;
+    reset_sweep(S, 0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the residual that follows
+        ctl->dinf = 0.0;
+        ctl->omega = 0.0;
+    }
+    double *yv = S.yv[1];
+    int32_t *flag = S.sync[1] + 1, *tcnt = flag + S.nsuper;
     SolveItem it;
     SolveNode nd;
-    while (next_item(S, S.bwd, S.nbwd, it, nd, &sh_it, &sh_nd)) {
+    while (next_item(S, S.sync[1], S.bwd, S.nbwd, it, nd, &sh_it, &sh_nd)) {
         if (it.r == kLeafGroup) {
             const int ls = S.bwd_leaf[8 * it.s + warp];
             if (ls >= 0) leaf_backward(S, ls, fronts, x, flag, ctl);
@@ -924,7 +945,7 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
             const double *Lc = L + (int64_t)(b0 + lane) * ld + 32 * bp + 4 * warp;
 #pragma unroll
             for (int c = 0; c < 4; c++) lv[c] = (lane < w && 4 * warp + c < wp) ? Lc[c] : 0.0;
-            if (warp == 0) zs[bp & 1][lane] = poll_block(S.yv + c0 + 32 * bp, wp, ctl, S.spin_limit);
+            if (warp == 0) zs[bp & 1][lane] = poll_block(yv + c0 + 32 * bp, wp, ctl, S.spin_limit);
             __syncthreads();
             if (lane < w) {
 #pragma unroll
@@ -948,14 +969,14 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
         if (pair) {
             // z_b = X_b^T z'' - V_b^T z_{b+1}, z_{b+1} being the last block to finish
             const int wn = min(32, k - 32 * (b + 1));  // block b + 1 may be the last, partial one
-            if (warp == 0) zs[0][lane] = poll_block(S.yv + c0 + 32 * (b + 1), wn, ctl, S.spin_limit);
+            if (warp == 0) zs[0][lane] = poll_block(yv + c0 + 32 * (b + 1), wn, ctl, S.spin_limit);
             __syncthreads();
             apply_pair(Wb, z, zs[0], part, w, true);
             __syncthreads();
         }
         for (int q = tid; q < w; q += kSolveThreads) {
             __stcg(x + c0 + b0 + q, z[q]);
-            if (nd.nblk > 1) publish_value(S.yv + c0 + b0 + q, z[q]);
+            if (nd.nblk > 1) publish_value(yv + c0 + b0 + q, z[q]);
         }
         // publish: the blocks of a split supernode count themselves done
         // (release); block 0, the last of the chain, acquires all of them
@@ -979,16 +1000,9 @@ __global__ void __launch_bounds__(kSolveThreads, 5) k_backward_persistent(SolveS
     }
 }
 
-// Before a persistent sweep: the ticket and the counters to zero, the block
-// values of the chains and the row chunks' sums to the unset pattern.
-__global__ void k_sweep_reset(int32_t *__restrict__ sync, int32_t ncnt, double *__restrict__ yv, int32_t nyv,
-                              double *__restrict__ rpart, int64_t nrpart) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < ncnt || i < nyv || i < nrpart;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (i < ncnt) sync[i] = 0;
-        if (i < nyv) yv[i] = __longlong_as_double((long long)kUnset);
-        if (i < nrpart) rpart[i] = __longlong_as_double((long long)kUnset);
-    }
+__global__ void k_sweep_reset(SolveSched S) {
+    reset_sweep(S, 0);
+    reset_sweep(S, 1);
 }
 
 // f (factorisation order) from [r7; r1] (original order).
@@ -1000,7 +1014,9 @@ __global__ void k_permute_in(const int32_t *__restrict__ perm, int N, int n, con
     }
 }
 __global__ void k_permute_out(const int32_t *__restrict__ perm, int N, int n, const double *__restrict__ x,
-                              double *__restrict__ dx, double *__restrict__ dy, int form) {
+                              const double *__restrict__ x1, const int32_t *sel, double *__restrict__ dx,
+                              double *__restrict__ dy, int form) {
+    if (sel && *sel) x = x1;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
         const int o = perm[i];
         if (form == 2) dy[o] = x[i];
@@ -1012,10 +1028,13 @@ __global__ void k_permute_out(const int32_t *__restrict__ perm, int N, int n, co
 // r = f - K x and ad = |K||x| in the factorisation order, from the entries'
 // values that the factorisation's norm stored (12 bytes per entry, and no
 // division by Theta); also the running max of |x| (ctl->dinf, as ordered bits
-// of a non-negative double).  Two FP64 instructions per entry.
+// of a non-negative double).  Two FP64 instructions per entry.  With a
+// correction c it takes x + c (added again for every entry: the sum's own pass,
+// a launch and a copy of the iterate cost more) and writes it to xn.
 __global__ void __launch_bounds__(rows::kThreads) k_residual(DevPlan P, const double *__restrict__ f,
-                                                             const double *__restrict__ x, double *__restrict__ r,
-                                                             double *__restrict__ ad, DevCtl *ctl,
+                                                             const double *__restrict__ x,
+                                                             const double *__restrict__ c, double *__restrict__ xn,
+                                                             double *__restrict__ r, double *__restrict__ ad, DevCtl *ctl,
                                                              const int32_t *skip) {
     if (skip && *skip) return;
     __shared__ double sh[rows::kThreads / 32][2];
@@ -1028,7 +1047,8 @@ __global__ void __launch_bounds__(rows::kThreads) k_residual(DevPlan P, const do
         const int64_t p1 = P.kp[i + 1];
 #pragma unroll 4
         for (int64_t p = P.kp[i] + t; p < p1; p += nt) {
-            const double v = P.kval[p], xj = x[P.kj[p]];
+            const int j = P.kj[p];
+            const double v = P.kval[p], xj = c ? x[j] + c[j] : x[j];
             a[0] += v * xj;
             a[1] += fabs(v) * fabs(xj);
         }
@@ -1038,7 +1058,9 @@ __global__ void __launch_bounds__(rows::kThreads) k_residual(DevPlan P, const do
         if (!isfinite(ri)) bad = true;
         r[i] = ri;
         ad[i] = a[1];
-        xm = fmax(xm, fabs(x[i]));
+        const double xi = c ? x[i] + c[i] : x[i];
+        if (c) xn[i] = xi;
+        xm = fmax(xm, fabs(xi));
     };
     double a[2];
     if (w.cta >= 0) {
@@ -1094,10 +1116,12 @@ __global__ void k_axpy(double *__restrict__ x, const double *__restrict__ c, int
 }
 
 // Device-side refinement control (used when the solve is captured in a CUDA
-// graph and no host decision is possible).  After the first residual:
-// best = x, omega_best = omega, done = omega <= target.  After step k:
-// keep x as best if omega improved; done once omega <= target, omega failed
-// to halve, or k = max_steps.  Kernels of later steps exit at entry when done.
+// graph and no host decision is possible).  Step k forms its iterate in buffer
+// k % 2 from the other one, the best so far (a step runs only after one that
+// halved omega).  After the first residual: best = 0, omega_best = omega, done =
+// omega <= target.  After step k: best = k % 2 if omega improved; done once
+// omega <= target, omega failed to halve, or k = max_steps.  Kernels of later
+// steps exit at entry when done.
 __global__ void k_refine_init(DevCtl *ctl, double target, int max_steps) {
     const double w = ctl->omega;
     ctl->omega_best = w;
@@ -1105,12 +1129,14 @@ __global__ void k_refine_init(DevCtl *ctl, double target, int max_steps) {
     ctl->steps = 0;
     ctl->gmres_iters = 0;
     ctl->improved = 1;
+    ctl->best = 0;
     ctl->done = (w <= target || max_steps <= 0) ? 1 : 0;
 }
 
-__global__ void k_refine_step(DevCtl *ctl, double target, int step, int max_steps) {
+__global__ void k_refine_step(DevCtl *ctl, double target, int step, int max_steps, unsigned long long handle) {
     if (ctl->done) {
         ctl->improved = 0;
+        if (handle) cudaGraphSetConditional((cudaGraphConditionalHandle)handle, 0);
         return;
     }
     const double w = ctl->omega;
@@ -1118,8 +1144,12 @@ __global__ void k_refine_step(DevCtl *ctl, double target, int step, int max_step
     if (step < 16) ctl->omega_hist[step] = w;
     const bool halved = w <= 0.5 * ctl->omega_best;
     ctl->improved = w < ctl->omega_best ? 1 : 0;
-    if (ctl->improved) ctl->omega_best = w;
+    if (ctl->improved) {
+        ctl->omega_best = w;
+        ctl->best = step & 1;
+    }
     ctl->done = (!halved || ctl->omega_best <= target || step >= max_steps) ? 1 : 0;
+    if (handle) cudaGraphSetConditional((cudaGraphConditionalHandle)handle, ctl->done ? 0 : 1);
 }
 
 __global__ void k_refine_finish(DevCtl *ctl, double target) {
@@ -1131,6 +1161,14 @@ __global__ void k_copy_if(double *__restrict__ dst, const double *__restrict__ s
                           int invert) {
     if (flag && ((*flag != 0) == (invert != 0))) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) dst[i] = src[i];
+}
+
+__global__ void k_best_both(double *__restrict__ x0, double *__restrict__ x1, int N, const DevCtl *ctl) {
+    const bool one = ctl->best != 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        if (one) x0[i] = x1[i];
+        else x1[i] = x0[i];
+    }
 }
 
 __global__ void k_clear_norms(DevCtl *ctl, const int32_t *skip) {
@@ -1195,26 +1233,20 @@ void launch_backward_bk(const DevPlan &P, const double *fronts, const int32_t *l
     k_backward_bk<<<count, kSolveThreads, (size_t)maxf * sizeof(double), st>>>(P, fronts, lperm, x, list);
 }
 
-void launch_sweep_reset(const SolveSched &S, int32_t ncnt, int64_t nrpart, cudaStream_t st) {
-    const int64_t n = S.nyv > nrpart ? S.nyv : nrpart, grid = (n + 255) / 256 < 304 ? (n + 255) / 256 : 304;
-    k_sweep_reset<<<grid > 0 ? (int)grid : 1, 256, 0, st>>>(S.sync, ncnt, S.yv, S.nyv, S.rpart, nrpart);
-}
+void launch_sweep_reset(const SolveSched &S, cudaStream_t st) { k_sweep_reset<<<304, 256, 0, st>>>(S); }
 
-void launch_forward_persistent(const SolveSched &S, const double *fronts, const double *Dinv, double *x, double *upd,
-                               int32_t maxf, int32_t grid, DevCtl *ctl, cudaStream_t st, const int32_t *skip) {
+void launch_forward_persistent(const SolveSched &S, const double *fronts, const double *Dinv, const double *b, double *x,
+                               double *upd, int32_t maxf, int32_t grid, DevCtl *ctl, cudaStream_t st,
+                               const int32_t *skip) {
     static uint64_t attr = 0;
     if (first_on_device(attr))
         cudaFuncSetAttribute(k_forward_persistent, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmemLimit);
-    // sync[0] = ticket; then per supernode: finished children, finished items
-    launch_sweep_reset(S, 2 * S.nsuper + 1, 0, st);
     const size_t smem = (size_t)(maxf > kRectRows ? maxf : kRectRows) * sizeof(double);
-    k_forward_persistent<<<grid, kSolveThreads, smem, st>>>(S, fronts, Dinv, x, upd, ctl, skip);
+    k_forward_persistent<<<grid, kSolveThreads, smem, st>>>(S, fronts, Dinv, b, x, upd, ctl, skip);
 }
 
 void launch_backward_persistent(const SolveSched &S, const double *fronts, double *x, int32_t grid, DevCtl *ctl,
                                 cudaStream_t st, const int32_t *skip) {
-    // sync[0] = ticket; then per supernode: done flag, finished blocks
-    launch_sweep_reset(S, 2 * S.nsuper + 1, S.nrpart, st);
     k_backward_persistent<<<grid, kSolveThreads, kBackSmem, st>>>(S, fronts, x, ctl, skip);
 }
 
@@ -1222,20 +1254,16 @@ void launch_permute_in(const DevPlan &P, const double *r7, const double *r1, dou
     k_permute_in<<<(P.N + 255) / 256, 256, 0, st>>>(P.perm, P.N, P.n, r7, r1, f, P.form);
 }
 
-void launch_permute_out(const DevPlan &P, const double *x, double *dx, double *dy, cudaStream_t st) {
-    k_permute_out<<<(P.N + 255) / 256, 256, 0, st>>>(P.perm, P.N, P.n, x, dx, dy, P.form);
+void launch_permute_out(const DevPlan &P, const double *x, double *dx, double *dy, cudaStream_t st, const double *x1,
+                        const int32_t *sel) {
+    k_permute_out<<<(P.N + 255) / 256, 256, 0, st>>>(P.perm, P.N, P.n, x, x1, sel, dx, dy, P.form);
 }
 
-void launch_residual_omega(const DevPlan &P, const double *f, const double *x, double *r, double *ad, DevCtl *ctl,
-                           cudaStream_t st, const int32_t *skip) {
+void launch_residual_omega(const DevPlan &P, const double *f, const double *x, const double *c, double *xn, double *r,
+                           double *ad, DevCtl *ctl, cudaStream_t st, const int32_t *skip, bool clear) {
     const int grid = (P.N + 255) / 256 < 608 ? (P.N + 255) / 256 : 608;
-    if (!skip) {
-        cudaMemsetAsync(&ctl->dinf, 0, sizeof(double), st);
-        cudaMemsetAsync(&ctl->omega, 0, sizeof(double), st);
-    } else {
-        k_clear_norms<<<1, 1, 0, st>>>(ctl, skip);
-    }
-    k_residual<<<rows::grid(P.N, P.nmid, P.nlong), rows::kThreads, 0, st>>>(P, f, x, r, ad, ctl, skip);
+    if (clear) k_clear_norms<<<1, 1, 0, st>>>(ctl, skip);
+    k_residual<<<rows::grid(P.N, P.nmid, P.nlong), rows::kThreads, 0, st>>>(P, f, x, c, xn, r, ad, ctl, skip);
     k_omega<<<grid, 256, 0, st>>>(P.N, r, ad, P.kabs, f, ctl, skip);
 }
 
@@ -1253,8 +1281,13 @@ void launch_refine_init(DevCtl *ctl, double target, int32_t max_steps, cudaStrea
     k_refine_init<<<1, 1, 0, st>>>(ctl, target, max_steps);
 }
 
-void launch_refine_step(DevCtl *ctl, double target, int32_t step, int32_t max_steps, cudaStream_t st) {
-    k_refine_step<<<1, 1, 0, st>>>(ctl, target, step, max_steps);
+void launch_refine_step(DevCtl *ctl, double target, int32_t step, int32_t max_steps, cudaStream_t st,
+                        unsigned long long handle) {
+    k_refine_step<<<1, 1, 0, st>>>(ctl, target, step, max_steps, handle);
+}
+
+void launch_best_both(double *x0, double *x1, int32_t N, const DevCtl *ctl, cudaStream_t st) {
+    k_best_both<<<(N + 255) / 256 < 608 ? (N + 255) / 256 : 608, 256, 0, st>>>(x0, x1, N, ctl);
 }
 
 void launch_refine_finish(DevCtl *ctl, double target, cudaStream_t st) { k_refine_finish<<<1, 1, 0, st>>>(ctl, target); }
