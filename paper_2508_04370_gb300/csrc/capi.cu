@@ -806,7 +806,24 @@ int setup_device(ipm_ctx *c) {
     // The assembly items of large front s, one per 32 columns x kAsmRows rows of
     // its lower part, appended to asm_items (the terms' lists are built once
     // per front; a front's items may be appended again).
-    std::vector<std::vector<std::pair<int32_t, int64_t>>> points;  // per item: destination, arena position
+    using Points = std::vector<std::pair<int32_t, int64_t>>;  // destination, arena position; children ascending
+    auto add_segments = [&](Points &pt, int64_t &seg0, int64_t &seg1) {
+        std::stable_sort(pt.begin(), pt.end(),
+                         [](const std::pair<int32_t, int64_t> &x, const std::pair<int32_t, int64_t> &y) {
+                             return x.first < y.first;
+                         });
+        seg0 = (int64_t)seg_dst.size();
+        for (size_t u = 0; u < pt.size(); u++) {
+            if (u == 0 || pt[u].first != pt[u - 1].first) {
+                if (u > 0) seg_ptr.push_back((int64_t)seg_src.size());
+                seg_dst.push_back(pt[u].first);
+            }
+            seg_src.push_back(pt[u].second);
+        }
+        if (!pt.empty()) seg_ptr.push_back((int64_t)seg_src.size());
+        seg1 = (int64_t)seg_dst.size();
+    };
+    std::vector<Points> points;                                    // per item
     std::vector<std::vector<AsmChild>> block_child;                // per column block
     auto add_asm = [&](int32_t s) {
         const int32_t ld = P.sn_ld[s], f = P.sn_f[s], ntile = asm_tiles(f), nblk = (f + 31) / 32;
@@ -862,24 +879,33 @@ int setup_device(ipm_ctx *c) {
             for (int32_t rb = 32 * cb / kAsmRows; rb * kAsmRows < f; rb++, t++) {
                 ai.r_lo = std::max(rb * kAsmRows, ai.c_lo);
                 ai.r_hi = std::min((rb + 1) * kAsmRows, f);
-                std::vector<std::pair<int32_t, int64_t>> &pt = points[t];
-                std::stable_sort(pt.begin(), pt.end(), [](const std::pair<int32_t, int64_t> &x, const std::pair<int32_t, int64_t> &y) {
-                    return x.first < y.first;
-                });
-                ai.seg0 = (int64_t)seg_dst.size();
-                for (size_t u = 0; u < pt.size(); u++) {
-                    if (u == 0 || pt[u].first != pt[u - 1].first) {
-                        if (u > 0) seg_ptr.push_back((int64_t)seg_src.size());
-                        seg_dst.push_back(pt[u].first);
-                    }
-                    seg_src.push_back(pt[u].second);
-                }
-                if (!pt.empty()) seg_ptr.push_back((int64_t)seg_src.size());
-                ai.seg1 = (int64_t)seg_dst.size();
+                add_segments(points[t], ai.seg0, ai.seg1);
                 asm_items.push_back(ai);
             }
         }
     };
+    // the small fronts' lists
+    std::vector<int64_t> small_seg(2 * (size_t)P.nsuper, 0);
+    std::vector<int32_t> small_big(P.nsuper, 0);
+    if (!c->opt.pivoting) {
+        Points pt;
+        for (int32_t s = 0; s < P.nsuper; s++) {
+            if (P.sn_large[s]) continue;
+            pt.clear();
+            small_big[s] = P.child_ptr[s];
+            for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
+                const int32_t ch = P.child_list[q], kc = P.sn_k[ch], cc = P.sn_f[ch] - kc, ldc = P.sn_ld[ch];
+                if (cc > kPointRows) continue;
+                small_big[s]++;
+                const int32_t *m = P.relmap.data() + P.map_off[ch];
+                const int64_t cb0 = P.sn_off[ch] + (int64_t)kc * ldc + kc;
+                for (int32_t jj = 0; jj < cc; jj++)
+                    for (int32_t ii = jj; ii < cc; ii++)
+                        pt.push_back({m[jj] * P.sn_ld[s] + m[ii], cb0 + (int64_t)jj * ldc + ii});
+            }
+            add_segments(pt, small_seg[2 * (size_t)s], small_seg[2 * (size_t)s + 1]);
+        }
+    }
     // One step of the large-front path: for each (front s, panel start p0)
     // of fp, the diagonal block of the panel, the triangular solve of the rows
     // below it and the update tiles of the front's trailing part.
@@ -1266,6 +1292,7 @@ int setup_device(ipm_ctx *c) {
         (rc = dupload(c, (AsmItem **)&c->al.items, asm_items)) || (rc = dupload(c, (int32_t **)&c->al.seg_dst, seg_dst)) ||
         (rc = dupload(c, (int64_t **)&c->al.seg_ptr, seg_ptr)) || (rc = dupload(c, (int64_t **)&c->al.src, seg_src)) ||
         (rc = dupload(c, (AsmChild **)&c->al.child, asm_child)) || (rc = dupload(c, (int32_t **)&c->al.rt, asm_rt)) ||
+        (rc = dupload(c, (int64_t **)&c->al.small, small_seg)) || (rc = dupload(c, (int32_t **)&c->al.small_big, small_big)) ||
         (rc = dupload(c, &c->panel_items, panel_items)) ||
         (rc = dupload(c, &c->trsm_items, trsm_items)) || (rc = dupload(c, &c->trsm_slots, trsm_slots)) ||
         (rc = dalloc(c, &c->panel_ws, (size_t)std::max(nslots, 1) * kPanelWsHost)) ||
@@ -1546,7 +1573,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             cudaStream_t sq = q == 0 ? st : c->cls[(q - 1) & 1];
             if (q > 0) cudaStreamWaitEvent(sq, fork, 0);
             Prof pr(c, IPM_K_SMALL_FRONTS, C.w, sq);
-            launch_small_fronts(c->dp, V, c->fronts, c->D, c->Dinv, c->dyn, c->ctl, c->lvl_small + C.off, C.cnt,
+            launch_small_fronts(c->dp, V, c->fronts, c->D, c->Dinv, c->dyn, c->ctl, c->al, c->lvl_small + C.off, C.cnt,
                                 c->opt.nb, C.maxf, c->tune_threads[C.cls], sq);
             nl++;
             if (q > 0) {

@@ -233,6 +233,10 @@ struct AsmLists {
     const int64_t *src;
     const AsmChild *child;
     const int32_t *rt;
+    // small fronts (k_small_fronts): segments [small[2 s], small[2 s + 1]), with
+    // destinations column * ld + row, and the front's first large child
+    const int64_t *small;
+    const int32_t *small_big;
 };
 struct TileItem {
     int32_t s;
@@ -294,8 +298,8 @@ struct FactorItem {
 // factorisation (kernels_factor.cu)
 void launch_norm1(const DevPlan &P, const DevVals &V, DevCtl *ctl, double eps_piv, cudaStream_t st);
 void launch_small_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
-                         DevCtl *ctl, const int32_t *list, int32_t count, int32_t nb, int32_t maxf, int32_t threads,
-                         cudaStream_t st);
+                         DevCtl *ctl, const AsmLists &A, const int32_t *list, int32_t count, int32_t nb, int32_t maxf,
+                         int32_t threads, cudaStream_t st);
 void launch_large_assemble(const DevPlan &P, const DevVals &V, double *fronts, const AsmLists &A, int64_t first,
                            int32_t count, cudaStream_t st);
 // panel step 1 (diagonal block of the panel [item.p0, item.p0 + nb), one item

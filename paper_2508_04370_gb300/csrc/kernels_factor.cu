@@ -195,12 +195,36 @@ __device__ __forceinline__ void bar_arrive_parity(int parity) {
 // apply the rank-1 update to the rest of the pivot block's columns (all rows
 // below, which also performs the triangular solve of the rows under the
 // block); after each block of 32 pivots all threads apply the block to the
-// trailing lower part.
+// trailing lower part.  The children's entries come as lists per destination
+// (children of more than kPointRows rows one by one): a front of 60 rows has up
+// to 35 children, and each cost a chain of global reads and a barrier.
+//
+// Small children's entries, one thread per destination: T[d] += the arena
+// values of d's list, children ascending.
+__device__ __forceinline__ void sum_points(const AsmLists &A, int64_t g0, int64_t g1, int nthreads,
+                                           const double *fronts, double *T) {
+    for (int64_t g = g0 + threadIdx.x; g < g1; g += nthreads) {
+        const int d = A.seg_dst[g];
+        const int64_t e = A.seg_ptr[g + 1];
+        double v = T[d];
+        int64_t q = A.seg_ptr[g];
+        for (; q + 4 <= e; q += 4) {
+            double c[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) c[u] = __ldcg(fronts + A.src[q + u]);
+#pragma unroll
+            for (int u = 0; u < 4; u++) v += c[u];
+        }
+        for (; q < e; q++) v += __ldcg(fronts + A.src[q]);
+        T[d] = v;
+    }
+}
+
 template <int NT>
 __global__ void __launch_bounds__(NT) k_small_fronts(DevPlan P, DevVals V, double *__restrict__ fronts,
                                                       double *__restrict__ Dg, double *__restrict__ Dig,
-                                                      double *__restrict__ dyng,
-                                                      DevCtl *ctl, const int32_t *__restrict__ list, int nb) {
+                                                      double *__restrict__ dyng, DevCtl *ctl, AsmLists A,
+                                                      const int32_t *__restrict__ list, int nb) {
     extern __shared__ double smem[];
     __shared__ double wcol[128];  // fronts up to 128 rows use this kernel
     __shared__ double dq[32];
@@ -218,7 +242,9 @@ __global__ void __launch_bounds__(NT) k_small_fronts(DevPlan P, DevVals V, doubl
     for (int64_t q = P.orig_ptr[s] + tid; q < P.orig_ptr[s + 1]; q += NT)
         F[P.orig_dst[q]] = orig_value(P, V, P.orig_src[q]);
     __syncthreads();
-    for (int q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
+    sum_points(A, A.small[2 * s], A.small[2 * s + 1], NT, fronts, F);
+    __syncthreads();
+    for (int q = A.small_big[s]; q < P.child_ptr[s + 1]; q++) {
         const int c = P.child_list[q];
         const int kc = P.sn_k[c], ldc = P.sn_ld[c];
         const int cc = P.sn_f[c] - kc;
@@ -332,21 +358,7 @@ __device__ __forceinline__ void assemble_block(const DevPlan &P, const DevVals &
         if (r >= r_lo && r < r_hi) T[R * (c - c_lo) + r - rbase] = orig_value(P, V, P.orig_src[q]);
     }
     __syncthreads();
-    for (int64_t g = ai.seg0 + tid; g < ai.seg1; g += NT) {
-        const int d = A.seg_dst[g];
-        const int64_t e = A.seg_ptr[g + 1];
-        double v = T[d];
-        int64_t q = A.seg_ptr[g];
-        for (; q + 4 <= e; q += 4) {
-            double c[4];
-#pragma unroll
-            for (int u = 0; u < 4; u++) c[u] = __ldcg(fronts + A.src[q + u]);
-#pragma unroll
-            for (int u = 0; u < 4; u++) v += c[u];
-        }
-        for (; q < e; q++) v += __ldcg(fronts + A.src[q]);
-        T[d] = v;
-    }
+    sum_points(A, ai.seg0, ai.seg1, NT, fronts, T);
     __syncthreads();
     // large children: lane j holds the front column of the child's column a + j,
     // and the front rows of the child's rows i0 and i0 + 32
@@ -1500,8 +1512,8 @@ __global__ void k_factor_stats_bk(const double *__restrict__ D, const double *__
 }  // namespace
 
 void launch_small_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
-                         DevCtl *ctl, const int32_t *list, int32_t count, int32_t nb, int32_t maxf, int32_t threads,
-                         cudaStream_t st) {
+                         DevCtl *ctl, const AsmLists &A, const int32_t *list, int32_t count, int32_t nb, int32_t maxf,
+                         int32_t threads, cudaStream_t st) {
     if (count <= 0) return;
     const int ldmax = (maxf + 3) & ~3;
     const size_t smem = (size_t)ldmax * maxf * sizeof(double);
@@ -1512,15 +1524,23 @@ void launch_small_fronts(const DevPlan &P, const DevVals &V, double *fronts, dou
         cudaFuncSetAttribute(k_small_fronts<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         cudaFuncSetAttribute(k_small_fronts<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     }
-    // default: one warp per front up to f = 32, two up to 64, four beyond;
-    // the autotuner may choose any of 32, 64, 128, 256 (same arithmetic per
-    // entry whatever the width)
-    if (threads <= 0) threads = maxf <= 32 ? 32 : maxf <= 64 ? 64 : 128;
+    // default: one warp per front up to f = 32, two up to 64, four beyond, and
+    // more where the launch leaves SMs idle: a front's pivots then run on all four
+    // sub-partitions' FP64 pipes (factorisation of a 31 x 31 grid with 12 levels
+    // of 10 to 600 fronts 0.86 -> 0.72 ms; a 64 x 64 grid, whose lower levels
+    // fill the chip, loses 1% with the wide CTAs there).  The autotuner may
+    // choose any of 32, 64, 128, 256 (same arithmetic per entry whatever the width).
+    if (threads <= 0) {
+        threads = maxf <= 32 ? 32 : maxf <= 64 ? 64 : 128;
+        if (count <= 608) threads *= 2;
+        if (count <= 152) threads *= 2;
+        if (threads > 256) threads = 256;
+    }
     switch (threads) {
-        case 32: k_small_fronts<32><<<count, 32, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, nb); break;
-        case 64: k_small_fronts<64><<<count, 64, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, nb); break;
-        case 256: k_small_fronts<256><<<count, 256, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, nb); break;
-        default: k_small_fronts<128><<<count, 128, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, nb); break;
+        case 32: k_small_fronts<32><<<count, 32, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, A, list, nb); break;
+        case 64: k_small_fronts<64><<<count, 64, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, A, list, nb); break;
+        case 256: k_small_fronts<256><<<count, 256, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, A, list, nb); break;
+        default: k_small_fronts<128><<<count, 128, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, A, list, nb); break;
     }
 }
 

@@ -89,3 +89,21 @@ def test_thin_fronts(pkg, nlink, groups, private):
         else:
             assert np.array_equal(base["D"], r["D"]) and np.array_equal(base["L"], r["L"])
         r["s"].close()
+
+
+@pytest.mark.parametrize("m", [5, 32, 33, 64, 65, 66, 97])
+def test_small_front_children(pkg, m):
+    """A front of m rows under children of 1 to m contribution rows (lists up to
+    64 rows, one by one beyond), every CTA width with the same bits."""
+    lp = lp_with_columns(m, [1 + (7 * j) % m for j in range(3 * m)] + [m, max(m - 1, 1)], m)
+    theta = synth.theta_loguniform(lp.n, 5, -3.0, 3.0)
+    r = run_pair(pkg, lp, theta, synth.rhs_normal(lp.n, 6), synth.rhs_normal(lp.m, 7), ordering=pkg.IPM_ORD_NATURAL)
+    assert r["info"]["nfronts_small"] > 0
+    check_pair(r, lp)
+    s = r["s"]
+    for width in (32, 64, 128, 256):
+        pkg.ipm_set_launch_shapes(s.ctx, [width] * 3)
+        s.factorise(theta, 1e-8, 1e-8)
+        L, D, _ = s.factor()
+        assert np.array_equal(D, r["D"]) and np.array_equal(L, r["L"])
+    s.close()
