@@ -371,7 +371,7 @@ int ipm_solve_noalloc(ipm_ctx *ctx, const double *r7_dev, const double *r1_dev, 
  *   - the level-kernel threshold: a tree level runs its large fronts in one
  *     persistent launch when their FP64 work at 1 TFLOP/s is below ratio x
  *     (35 us per 32-column panel of its widest front); candidates 0 (never),
- *     0.25, 0.5 (default), 1, 2, 1e30 (always);
+ *     0.25, 0.5, 1 (default), 2, 1e30 (always);
  *   - the threads per small-front CTA of each size class present (f <= 32:
  *     32 or 64; f <= 64: 64 or 128; f <= 128: 128 or 256);
  *   - the level kernel's CTAs per SM: as many as fit (default) or one (see

@@ -32,7 +32,7 @@ struct StepWork {
     int64_t panel_off;  // diagonal-block items (one per front)
     int32_t panel_cnt;
     int64_t trsm_off;   // row-chunk items below the diagonal blocks
-    int32_t trsm_cnt;
+    int32_t trsm_cnt, trsm_rows;
     int64_t tile_off;   // FP64 update tiles: the first tile_cnt1 (strips) cover the next panel's
     int32_t tile_cnt;   // columns (lookahead, on the critical path), the rest the
     int32_t tile_cnt1;  // remaining trailing columns (a third stream)
@@ -72,8 +72,9 @@ struct LevelWork {
     // The level kernel pays off where a level's large fronts are bound by
     // their pivot chains (about 35 us per 32-column panel): a level takes it
     // when its FP64 front work at ~1 TFLOP/s is below tune_ratio times its
-    // longest chain (0.5 unless ipm_autotune chose otherwise).  Levels with
-    // more work run one launch per step at full occupancy.
+    // longest chain (1 unless ipm_autotune chose otherwise: a random 1537 x 3843
+    // LP's root level of 0.73 GFLOP and 41 panels takes 1.92 ms with it and 2.42
+    // by steps).  Levels with more work run one launch per step at full occupancy.
     int32_t lvl_chain = 0;  // 32-column panels of the level's widest large front
     Work lvl_w;             // algorithmic work of the level's large fronts (assembly and factorisation)
 };
@@ -144,7 +145,7 @@ struct ipm_ctx {
     // sub-partition's FP64 pipe to one CTA's pivot chain; two keep more
     // trailing tiles in flight.
     int32_t tune_threads[3] = {0, 0, 0};
-    double tune_ratio = 0.5;
+    double tune_ratio = 1.0;
     int32_t tune_lvl_per_sm = 0;
     double tune_ms = 0.0;
     bool mixed_active = false;  // tensor-core updates in use (mixed precision, no fallback yet)
@@ -918,6 +919,12 @@ int setup_device(ipm_ctx *c) {
         S.tc_off = (int64_t)tc_items.size();
         S.alt_off = (int64_t)alt_items.size();
         S.st_off = (int64_t)sliced_segs.size();
+        // rows of a triangular-solve item: 32 (four per warp, fewer FMAs a row), or 8
+        // where a step has so few rows that 32 leave SMs idle
+        int64_t step_rows = 0;
+        for (const auto &e : fp) step_rows += P.sn_f[e.first] - std::min(e.second + c->opt.nb, P.sn_k[e.first]);
+        const int32_t trsm_rows = step_rows > kTrsmFewRows ? kTrsmItemRowsHost : kTrsmRowsHost;
+        S.trsm_rows = trsm_rows;
         int32_t nblk = 0;  // slice blocks of this step
         std::vector<SlicedRun> t1, t2;  // sliced runs: next panel's columns / the rest (whole rows, cut below)
         std::vector<TileItem> u1, u2, a1, a2;  // lookahead / remaining tiles of this step
@@ -945,8 +952,8 @@ int setup_device(ipm_ctx *c) {
             const bool pair_second = tpan < npair && tpan % 2 == 1;
             // sliced fronts: the triangular solve writes the digit slices of the rows it finishes
             const int32_t sbase = (tc && sliced && p1 < f) ? (nblk << 1) | (pair_second ? 1 : 0) : -1;
-            for (int32_t r = p1; r < f; r += kTrsmItemRowsHost) {
-                trsm_items.push_back({s, r, std::min(r + kTrsmItemRowsHost, f), p0});
+            for (int32_t r = p1; r < f; r += trsm_rows) {
+                trsm_items.push_back({s, r, std::min(r + trsm_rows, f), p0});
                 trsm_slots.push_back(slot_of[s]);
                 trsm_sbase.push_back(sbase);
             }
@@ -1225,7 +1232,7 @@ int setup_device(ipm_ctx *c) {
         int32_t lk_steps = 0;
         for (const LevelWork &W : c->levels)
             if (c->opt.level_kernel && W.lvl_cnt > 0 &&
-                W.lvl_w.flops / 1.0e12 < c->tune_ratio * W.lvl_chain * 35e-6)
+                W.lvl_w.flops / 1.0e12 < 0.5 * W.lvl_chain * 35e-6)  // clearly bound by their chains
                 lk_steps += (int32_t)W.steps.size();
         c->dep_sched = !c->opt.pivoting && P.nlarge > 0 &&
                        (c->opt.schedule == IPM_SCHED_DEPENDENCY ||
@@ -1623,7 +1630,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             // on the sliced path the solve also writes the slices of the rows it finishes
             Prof pr(c, IPM_K_LARGE_PANEL, S.trsm_w, sd);
             launch_panel_trsm(c->dp, c->fronts, c->trsm_items + S.trsm_off, c->trsm_slots + S.trsm_off, S.trsm_cnt,
-                              c->opt.nb, c->panel_ws, sd, c->trsm_sbase + S.trsm_off, use_sliced ? ws : nullptr,
+                              S.trsm_rows, c->opt.nb, c->panel_ws, sd, c->trsm_sbase + S.trsm_off, use_sliced ? ws : nullptr,
                               wexp, c->D, c->ctl);
             nl++;
         }

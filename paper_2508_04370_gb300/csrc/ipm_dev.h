@@ -306,16 +306,17 @@ void launch_large_assemble(const DevPlan &P, const DevVals &V, double *fronts, c
 // per front; item.r1 = workspace slot)
 void launch_panel_diag(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                        DevCtl *ctl, const PanelItem *items, int32_t count, int32_t nb, double *pws, cudaStream_t st);
-// panel step 2 (rows below, kTrsmRowsHost rows per item; slots[i] = workspace slot of item i)
+// panel step 2 (rows below, up to `rows` rows per item; slots[i] = workspace slot of item i)
 // sbase[i] >= 0 (with sws non-null): item i also writes the digit slices of
 // its rows into the sliced update's work space (slice blocks from
 // sbase[i] >> 1; bit 0 set: the second panel of a pair, two chunks)
 void launch_panel_trsm(const DevPlan &P, double *fronts, const PanelItem *items, const int32_t *slots, int32_t count,
-                       int32_t nb, const double *pws, cudaStream_t st, const int32_t *sbase = nullptr,
+                       int32_t rows, int32_t nb, const double *pws, cudaStream_t st, const int32_t *sbase = nullptr,
                        uint8_t *sws = nullptr, int32_t *sexp = nullptr, const double *D = nullptr,
                        DevCtl *ctl = nullptr);
 constexpr int kTrsmRowsHost = 8;       // rows of a triangular-solve chunk of the level kernel
-constexpr int kTrsmItemRowsHost = 32;  // rows of a triangular-solve item of the one-launch-per-step kernel
+constexpr int kTrsmItemRowsHost = 32;  // rows of a triangular-solve item of the one-launch-per-step kernel,
+constexpr int64_t kTrsmFewRows = 2432; // or of a chunk where the step has no more rows than this (two chunks per SM)
 constexpr int kPanelWsHost = 32 * 33 + 32;
 void launch_large_update_strip(const DevPlan &P, double *fronts, const double *D, const TileItem *items,
                                int32_t count, int32_t w, cudaStream_t st);

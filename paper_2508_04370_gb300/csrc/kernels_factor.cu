@@ -920,6 +920,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_panel_diag(DevPlan P, DevVals 
     body_diag(P, V, fronts, Dg, Dig, dyng, ctl, it.s, it.p0, nb, pws + (int64_t)it.r1 * kPanelWs, pool);
 }
 
+template <int RW>
 __global__ void __launch_bounds__(kBodyThreads) k_panel_trsm(DevPlan P, double *__restrict__ fronts,
                                                               const PanelItem *__restrict__ items,
                                                               const int32_t *slots, int nb,
@@ -933,8 +934,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_panel_trsm(DevPlan P, double *
     if (sws && sbase[blockIdx.x] >= 0)
         so = SliceOut{sws, sexp, sbase[blockIdx.x] >> 1, sbase[blockIdx.x] & 1, min(it.p0 + nb, P.sn_k[it.s]), Dg,
                       ctl};
-    body_trsm<kTrsmItemRows / kTrsmRows>(P, fronts, it.s, it.r0, it.r1, it.p0, nb,
-                                         pws + (int64_t)slots[blockIdx.x] * kPanelWs, pool, so);
+    body_trsm<RW>(P, fronts, it.s, it.r0, it.r1, it.p0, nb, pws + (int64_t)slots[blockIdx.x] * kPanelWs, pool, so);
 }
 
 __global__ void __launch_bounds__(kBodyThreads) k_large_update(DevPlan P, double *__restrict__ fronts,
@@ -1558,10 +1558,14 @@ void launch_panel_diag(const DevPlan &P, const DevVals &V, double *fronts, doubl
 }
 
 void launch_panel_trsm(const DevPlan &P, double *fronts, const PanelItem *items, const int32_t *slots, int32_t count,
-                       int32_t nb, const double *pws, cudaStream_t st, const int32_t *sbase,
+                       int32_t rows, int32_t nb, const double *pws, cudaStream_t st, const int32_t *sbase,
                        uint8_t *sws, int32_t *sexp, const double *D, DevCtl *ctl) {
     if (count <= 0) return;
-    k_panel_trsm<<<count, kBodyThreads, 0, st>>>(P, fronts, items, slots, nb, pws, sbase, sws, sexp, D, ctl);
+    if (rows > kTrsmRows)
+        k_panel_trsm<kTrsmItemRows / kTrsmRows>
+            <<<count, kBodyThreads, 0, st>>>(P, fronts, items, slots, nb, pws, sbase, sws, sexp, D, ctl);
+    else
+        k_panel_trsm<1><<<count, kBodyThreads, 0, st>>>(P, fronts, items, slots, nb, pws, sbase, sws, sexp, D, ctl);
 }
 
 void launch_large_update(const DevPlan &P, double *fronts, const double *D, const TileItem *items, int32_t count,

@@ -416,40 +416,90 @@ __device__ __forceinline__ void diag_backward(const double *Lb, double *z, int w
 }
 
 // Explicit inverse X = L11^-1 of the unit lower-triangular w x w diagonal
-// block b of supernode s (w <= 32), one warp per block, computed once per
-// factorisation: lane j builds column j by
-//   X_jj = 1,   X_ij = -sum_{j <= t < i} L_it X_tj   (i > j),
-// rows in increasing order.  Stored column-major 32 x 32 (X_ij at 32 j + i),
-// zero above the diagonal, identity outside [0, w).  The sweeps then apply a
-// block as a matrix-vector product spread over four warps instead of a
-// substitution of w dependent steps.
-constexpr int kInvWarps = 2;
-__global__ void __launch_bounds__(32 * kInvWarps) k_diag_inverse(SolveSched S, const double *__restrict__ fronts,
-                                                                 double *__restrict__ Linv,
-                                                                 const InvItem *__restrict__ items, int count) {
-    __shared__ double Ls[kInvWarps][32][33];  // [row i][column t] of the strictly lower block
-    __shared__ double Xs[kInvWarps][32][33];  // [row t][column j] of X
-    const int wl = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int idx = blockIdx.x * kInvWarps + wl;
-    if (idx >= count) return;  // whole warps; no CTA barrier below
-    const InvItem it = items[idx];
+// block b of supernode s (w <= 32), one CTA of four warps per block, computed
+// once per factorisation: the four 8 x 8 diagonal blocks column by column
+//   X_jj = 1,   X_ij = -sum_{j <= t < i} L_it X_tj   (i > j)
+// (one warp, eight lanes per block), then twice X_21 = -X_22 (L_21 X_11) for
+// blocks of 8 and of 16.  The dependent FMAs are 28 + 2 x 8 + 2 x 32 where a warp per
+// block needed 496 (64 cycles each: 41 us at the end of every factorisation,
+// 64 x 64 grid 51 us with the products below; 17 and 27 now).  Stored
+// column-major 32 x 32 (X_ij at 32 j + i), zero above the diagonal, identity
+// outside [0, w).  The sweeps then apply a block as a matrix-vector product
+// spread over four warps instead of a substitution of w dependent steps.
+constexpr int kInvThreads = 128;
+__global__ void __launch_bounds__(kInvThreads) k_diag_inverse(SolveSched S, const double *__restrict__ fronts,
+                                                              double *__restrict__ Linv,
+                                                              const InvItem *__restrict__ items) {
+    __shared__ double Ls[32][33], Xs[32][33], Ts[16][17 * 2];  // [row][column]
+    const int tid = threadIdx.x, lane = tid & 31;
+    const InvItem it = items[blockIdx.x];
     const SolveNode nd = S.node[it.s];
     const int b0 = 32 * it.b, w = min(32, nd.k - b0), ld = nd.ld;
     const double *L = fronts + nd.off;
-    for (int t = 0; t < 32; t++) {
-        Ls[wl][lane][t] = (t < w && lane > t && lane < w) ? L[(int64_t)(b0 + t) * ld + b0 + lane] : 0.0;
-        Xs[wl][t][lane] = t == lane ? 1.0 : 0.0;
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        const int t = (tid >> 5) + 4 * q;  // column
+        Ls[lane][t] = (t < w && lane > t && lane < w) ? L[(int64_t)(b0 + t) * ld + b0 + lane] : 0.0;
+        Xs[lane][t] = t == lane ? 1.0 : 0.0;
     }
-    __syncwarp();
-    for (int i = 1; i < w; i++) {
-        double acc = 0.0;
-        for (int t = 0; t < i; t++) acc += Ls[wl][i][t] * Xs[wl][t][lane];  // Xs[t][lane] = 0 for t < lane
-        __syncwarp();
-        if (lane < i) Xs[wl][i][lane] = -acc;
-        __syncwarp();
+    __syncthreads();
+    if (tid < 32) {
+        const int r0 = lane & 24, j = lane & 7;  // lane j of each 8 x 8 block: its column j
+        double x[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            double acc = 0.0;
+#pragma unroll
+            for (int t = 0; t < i; t++) acc += Ls[r0 + i][r0 + t] * x[t];
+            x[i] = i == j ? 1.0 : i > j ? -acc : 0.0;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++) Xs[r0 + i][r0 + j] = x[i];
     }
+    __syncthreads();
+    {
+        // 16 x 16: thread -> block pair h, output (i, j) of its 8 x 8 off-diagonal block
+        const int h = 16 * (tid >> 6), i = tid & 7, j = (tid >> 3) & 7;
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; q++) t += Ls[h + 8 + i][h + q] * Xs[h + q][h + j];
+        Ts[i][(h >> 1) + j] = t;
+        __syncthreads();
+        double x = 0.0;
+#pragma unroll
+        for (int q = 0; q < 8; q++) x += Xs[h + 8 + i][h + 8 + q] * Ts[q][(h >> 1) + j];
+        __syncthreads();
+        Xs[h + 8 + i][h + j] = -x;
+    }
+    __syncthreads();
+    {
+        // 32 x 32: two outputs of the 16 x 16 off-diagonal block per thread
+        const int i = tid & 15, j = tid >> 4;
+        double t0 = 0.0, t1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < 16; q++) {
+            t0 += Ls[16 + i][q] * Xs[q][j];
+            t1 += Ls[16 + i][q] * Xs[q][j + 8];
+        }
+        Ts[i][j] = t0;
+        Ts[i][j + 8] = t1;
+        __syncthreads();
+        t0 = t1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < 16; q++) {
+            t0 += Xs[16 + i][16 + q] * Ts[q][j];
+            t1 += Xs[16 + i][16 + q] * Ts[q][j + 8];
+        }
+        Xs[16 + i][j] = -t0;
+        Xs[16 + i][j + 8] = -t1;
+    }
+    __syncthreads();
     double *X = Linv + it.dst;
-    for (int j = 0; j < 32; j++) X[32 * j + lane] = Xs[wl][lane][j];
+#pragma unroll
+    for (int q = 0; q < 8; q++) {
+        const int j = (tid >> 5) + 4 * q;
+        X[32 * j + lane] = Xs[lane][j];
+    }
 }
 
 // Diagonal-block storage in Linv: a supernode with one block keeps its X
@@ -491,16 +541,19 @@ __global__ void __launch_bounds__(256) k_pair_products(SolveSched S, const doubl
         }
         __syncthreads();
         double *out = X + (pass == 0 ? 1024 : 2048);
-        const int i = tid & 31;
+        // (X is lower triangular: the terms beyond its diagonal are left out, a row
+        // of W and a column of V per warp so that the count is the warp's)
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            const int j = (tid >> 5) + 8 * c;
+            const int u = (tid >> 5) + 8 * c, l = tid & 31;
             double a = 0.0;
-            if (pass == 0)
-                for (int t = 0; t < 32; t++) a += Xs[i][t] * Ls[t][j];
-            else
-                for (int t = 0; t < 32; t++) a += Ls[i][t] * Xs[t][j];
-            out[32 * j + i] = a;
+            if (pass == 0) {
+                for (int t = 0; t <= u; t++) a += Xs[u][t] * Ls[t][l];
+                out[32 * l + u] = a;  // W(u, l)
+            } else {
+                for (int t = u; t < 32; t++) a += Ls[l][t] * Xs[t][u];
+                out[32 * u + l] = a;  // V(l, u)
+            }
         }
     }
 }
@@ -1210,7 +1263,7 @@ int32_t solve_ctas_per_sm(int32_t maxf) {
 void launch_diag_inverse(const SolveSched &S, const double *fronts, double *Linv, const InvItem *items,
                          int32_t count, const InvItem *pairs, int32_t npairs, cudaStream_t st) {
     if (count <= 0) return;
-    k_diag_inverse<<<(count + kInvWarps - 1) / kInvWarps, 32 * kInvWarps, 0, st>>>(S, fronts, Linv, items, count);
+    k_diag_inverse<<<count, kInvThreads, 0, st>>>(S, fronts, Linv, items);
     if (npairs > 0) k_pair_products<<<npairs, 256, 0, st>>>(S, fronts, Linv, pairs, npairs);
 }
 
