@@ -1087,7 +1087,7 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
 // launch.  CTAs take tickets in the host's order, wait (thread 0, bounded
 // spin on acquire loads) until the item's counters reach their thresholds,
 // run the item's body, and add the item's increment to its completion
-// counter (release: every thread fences its writes before the barrier).
+// counter (release: thread 0 fences after the CTA barrier).
 // Every item waits only on items with smaller tickets, which were taken by
 // running CTAs, so the launch completes whatever the grid size.  A wait
 // that runs out sets kStatTimeout and the item proceeds (its results are
@@ -1131,8 +1131,7 @@ __global__ void __launch_bounds__(kBodyThreads) k_large_level(DevPlan P, DevVals
             sh_it = a;
         }
         __syncthreads();
-        const FactorItem it = sh_it;
-        __syncthreads();
+        const FactorItem it = sh_it;  // (rewritten after the barriers below)
         if (it.kind < 0) break;
         if (tid == 0) {
             if (it.wait0 >= 0) wait_counter(cnt + it.wait0, it.need0, ctl, limit);
@@ -1155,9 +1154,14 @@ __global__ void __launch_bounds__(kBodyThreads) k_large_level(DevPlan P, DevVals
             case kItemStrip: body_strip(P, fronts, Dg, it.s, it.a, it.b, it.t * nb, nb, pool); break;
             default: body_tile(P, fronts, Dg, it.s, it.a, it.b, it.t * nb, nb, pool); break;
         }
-        __threadfence();
+        // publish: the CTA barrier orders every thread's stores before thread 0's
+        // fence, which makes them visible device-wide before the counter
+        // (cumulativity); a fence in every thread cost the chain more
         __syncthreads();
-        if (tid == 0 && it.sig >= 0) atomicAdd(cnt + it.sig, it.add);
+        if (tid == 0 && it.sig >= 0) {
+            __threadfence();
+            atomicAdd(cnt + it.sig, it.add);
+        }
     }
 }
 
