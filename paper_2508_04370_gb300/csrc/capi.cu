@@ -123,6 +123,9 @@ struct ipm_ctx {
     AsmLists al{};  // assembly items of the large fronts and their terms
     int32_t *trsm_slots = nullptr;
     int32_t *trsm_sbase = nullptr;     // sliced path: first slice block of each TRSM item's front (-1: none)
+    int32_t *rank1_list = nullptr;  // rank-one leaves (k_rank_one)
+    int32_t rank1_cnt = 0;
+    Work rank1_w;
     int32_t *thin_list = nullptr, *thin_asm = nullptr, *thin_slot = nullptr;  // thin fronts by level
     double *panel_ws = nullptr;
     TileItem *tile_items = nullptr, *tc_items = nullptr, *alt_items = nullptr;
@@ -300,7 +303,7 @@ void long_rows(const V &ptr, std::vector<int32_t> &lng, std::vector<int32_t> &mi
     }
 }
 
-// Items of the persistent level kernel for the large fronts of level l, in
+// Items of the persistent level kernel for the large fronts of a level, in
 // ticket order: all assembly items, then per pivot block t the diagonal
 // blocks, the triangular solves, the remaining trailing tiles of block t-1
 // and the lookahead strips of block t (after the last block, the remaining
@@ -314,14 +317,14 @@ void long_rows(const V &ptr, std::vector<int32_t> &lng, std::vector<int32_t> &mi
 //   update (t, ib, jb):   all solve chunks of blocks <= t, tile >= 8 t.
 // Tiles lie on the front's 32-grid; updates skip the columns < p1 (the
 // panel's own columns) of a grid tile that a partial last panel cuts.
-void build_level_items(const Plan &P, int32_t l, LevelWork &W, const std::vector<int32_t> &slot_of,
+void build_level_items(const Plan &P, const std::vector<int32_t> &large, LevelWork &W, const std::vector<int32_t> &slot_of,
                        std::vector<FactorItem> &items, std::vector<int32_t> &cbase) {
     constexpr int32_t B = kUpdTile;  // == nb == 32
     W.lvl_off = (int64_t)items.size();
-    const int32_t t0 = P.lvl_large_ptr[l], t1 = P.lvl_large_ptr[l + 1];
+    const int32_t t0 = 0, t1 = (int32_t)large.size();
     int32_t ncnt = 0, maxsteps = 0;
     for (int32_t q = t0; q < t1; q++) {
-        const int32_t s = P.lvl_large[q], nblk = (P.sn_f[s] + B - 1) / B;
+        const int32_t s = large[q], nblk = (P.sn_f[s] + B - 1) / B;
         cbase[s] = ncnt;
         ncnt += 3 + nblk * (nblk + 1) / 2;
         maxsteps = std::max(maxsteps, (P.sn_k[s] + B - 1) / B);
@@ -344,7 +347,7 @@ void build_level_items(const Plan &P, int32_t l, LevelWork &W, const std::vector
     // assembly, in the order of the level's AsmItems
     int64_t ai = W.asm_off;
     for (int32_t q = t0; q < t1; q++) {
-        const int32_t s = P.lvl_large[q];
+        const int32_t s = large[q];
         for (int32_t u = 0; u < asm_tiles(P.sn_f[s]); u++) {
             FactorItem it = item(kItemAssemble, s, 0, 0, 0, (int32_t)ai++);
             it.sig = cbase[s];
@@ -371,7 +374,7 @@ void build_level_items(const Plan &P, int32_t l, LevelWork &W, const std::vector
     // updates of block t of front s: tiles (ib, jb >= first) with the
     // lookahead column block as strips when la
     auto updates = [&](int32_t q, int32_t t, bool lookahead) {
-        const int32_t s = P.lvl_large[q], k = P.sn_k[s], f = P.sn_f[s];
+        const int32_t s = large[q], k = P.sn_k[s], f = P.sn_f[s];
         if (t * B >= k) return;
         const int32_t p1 = std::min((t + 1) * B, k);
         if (p1 >= f) return;
@@ -414,7 +417,7 @@ void build_level_items(const Plan &P, int32_t l, LevelWork &W, const std::vector
     for (int32_t t = 0; t <= maxsteps; t++) {
         if (t < maxsteps) {
             for (int32_t q = t0; q < t1; q++) {
-                const int32_t s = P.lvl_large[q];
+                const int32_t s = large[q];
                 if (t * B >= P.sn_k[s]) continue;
                 FactorItem it = item(kItemDiag, s, t, 0, 0, slot_of[s]);
                 if (t == 0) {
@@ -429,7 +432,7 @@ void build_level_items(const Plan &P, int32_t l, LevelWork &W, const std::vector
                 items.push_back(it);
             }
             for (int32_t q = t0; q < t1; q++) {
-                const int32_t s = P.lvl_large[q], k = P.sn_k[s], f = P.sn_f[s];
+                const int32_t s = large[q], k = P.sn_k[s], f = P.sn_f[s];
                 if (t * B >= k) continue;
                 const int32_t p1 = std::min((t + 1) * B, k);
                 for (int32_t r = p1; r < f; r = chunk_end(r, f)) {
@@ -779,8 +782,24 @@ int setup_device(ipm_ctx *c) {
     std::vector<int32_t> trsm_slots, trsm_sbase, slot_of(P.nsuper, -1);
     std::vector<int32_t> thin_list, thin_asm, thin_slot;
     int32_t nslots = 0;
+    // Rank-one leaves: large fronts of one column without children whose parent's
+    // assembly takes their entries from l and u (assemble_block) instead of from
+    // a contribution block; one launch at the start of a factorisation
+    // finishes all of them, and they take no part in the levels' and steps' lists.
+    // (One column only: a second would double the assembly's FP64 work per
+    // entry.  Small parents and point lists read stored entries.)
+    std::vector<int8_t> rank1(P.nsuper, 0);
+    std::vector<int32_t> rank1_list;
+    for (int32_t s = 0; s < P.nsuper; s++) {
+        const int32_t p = P.sn_parent[s];
+        if (c->opt.pivoting || !P.sn_large[s] || P.sn_k[s] != 1 || P.child_ptr[s] != P.child_ptr[s + 1] ||
+            P.sn_f[s] - 1 <= kPointRows || p < 0 || !P.sn_large[p])
+            continue;
+        rank1[s] = 1;
+        rank1_list.push_back(s);
+    }
     for (int32_t s = 0; s < P.nsuper; s++)
-        if (P.sn_large[s]) slot_of[s] = nslots++;
+        if (P.sn_large[s] && !rank1[s]) slot_of[s] = nslots++;
     std::vector<TileItem> tile_items, tc_items, alt_items;
     std::vector<SlicedRun> sliced_runs;
     std::vector<SlicedSeg> sliced_segs;
@@ -799,8 +818,9 @@ int setup_device(ipm_ctx *c) {
         fr.bytes = 8.0 * f * (f + 1) / 2 + 12.0 * (double)(P.orig_ptr[s + 1] - P.orig_ptr[s]);
         for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
             const double cc = P.sn_f[P.child_list[q]] - P.sn_k[P.child_list[q]];
-            fr.bytes += 8.0 * cc * (cc + 1) / 2 + 4.0 * cc;
-            fr.flops += cc * (cc + 1) / 2;
+            const bool r1 = rank1[P.child_list[q]];
+            fr.bytes += (r1 ? 16.0 * cc : 8.0 * cc * (cc + 1) / 2) + 4.0 * cc;
+            fr.flops += (r1 ? 2 : 1) * cc * (cc + 1) / 2;
         }
         return fr;
     };
@@ -825,7 +845,7 @@ int setup_device(ipm_ctx *c) {
         seg1 = (int64_t)seg_dst.size();
     };
     std::vector<Points> points;                                    // per item
-    std::vector<std::vector<AsmChild>> block_child;                // per column block
+    std::vector<std::vector<AsmChild>> block_child, block_rank1;   // per column block
     auto add_asm = [&](int32_t s) {
         const int32_t ld = P.sn_ld[s], f = P.sn_f[s], ntile = asm_tiles(f), nblk = (f + 31) / 32;
         if (first_item[s] >= 0) {
@@ -837,14 +857,14 @@ int setup_device(ipm_ctx *c) {
         }
         first_item[s] = (int64_t)asm_items.size();
         if ((int32_t)points.size() < ntile) points.resize(ntile);
-        if ((int32_t)block_child.size() < nblk) block_child.resize(nblk);
+        if ((int32_t)block_child.size() < nblk) block_child.resize(nblk), block_rank1.resize(nblk);
         std::vector<int32_t> first_tile(nblk);  // item of the block's first rows
         for (int32_t cb = 0, t = 0; cb < nblk; cb++) {
             first_tile[cb] = t;
             t += (f + kAsmRows - 1) / kAsmRows - 32 * cb / kAsmRows;
         }
         for (int32_t t = 0; t < ntile; t++) points[t].clear();
-        for (int32_t cb = 0; cb < nblk; cb++) block_child[cb].clear();
+        for (int32_t cb = 0; cb < nblk; cb++) block_child[cb].clear(), block_rank1[cb].clear();
         for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
             const int32_t ch = P.child_list[q], kc = P.sn_k[ch], cc = P.sn_f[ch] - kc, ldc = P.sn_ld[ch];
             const int32_t *m = P.relmap.data() + P.map_off[ch];
@@ -863,7 +883,8 @@ int setup_device(ipm_ctx *c) {
             for (int32_t a = 0, b; a < cc; a = b) {
                 const int32_t cb = m[a] / 32;
                 for (b = a; b < cc && m[b] / 32 == cb; b++) {}
-                block_child[cb].push_back({cb0, P.map_off[ch], ldc, a, b, rt});
+                if (rank1[ch]) block_rank1[cb].push_back({P.sn_off[ch] + 1, P.map_off[ch], ldc, a, b, rt});
+                else block_child[cb].push_back({cb0, P.map_off[ch], ldc, a, b, rt});
             }
         }
         const int32_t *d0 = P.orig_dst.data() + P.orig_ptr[s], *d1 = P.orig_dst.data() + P.orig_ptr[s + 1];
@@ -877,6 +898,8 @@ int setup_device(ipm_ctx *c) {
             ai.ch0 = (int32_t)asm_child.size();
             asm_child.insert(asm_child.end(), block_child[cb].begin(), block_child[cb].end());
             ai.ch1 = (int32_t)asm_child.size();
+            asm_child.insert(asm_child.end(), block_rank1[cb].begin(), block_rank1[cb].end());
+            ai.ch2 = (int32_t)asm_child.size();
             for (int32_t rb = 32 * cb / kAsmRows; rb * kAsmRows < f; rb++, t++) {
                 ai.r_lo = std::max(rb * kAsmRows, ai.c_lo);
                 ai.r_hi = std::min((rb + 1) * kAsmRows, f);
@@ -1116,22 +1139,23 @@ int setup_device(ipm_ctx *c) {
         // one CTA each, instead of through the steps
         W.asm_off = (int64_t)asm_items.size();
         int32_t maxsteps = 0;
-        std::vector<int32_t> main_fronts;
+        std::vector<int32_t> main_fronts, large;
+        for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++)
+            if (!rank1[P.lvl_large[t]]) large.push_back(P.lvl_large[t]);
         W.thin_off = (int64_t)thin_list.size();
         auto is_thin = [&](int32_t s) {
             return P.sn_k[s] <= c->opt.nb && P.sn_f[s] <= kThinMaxF &&
                    !(c->opt.precision != IPM_PREC_FP64 && P.sn_f[s] >= c->opt.mixed_min_front);
         };
-        int32_t inner = 0;  // thin fronts with children
-        for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++) {
-            const int32_t s = P.lvl_large[t];
+        int32_t inner = 0, leaves = 0;  // thin fronts with children, without
+        for (int32_t s : large) {
             inner += is_thin(s) && P.child_ptr[s] < P.child_ptr[s + 1];
+            leaves += is_thin(s) && P.child_ptr[s] == P.child_ptr[s + 1];
         }
         std::vector<std::pair<double, int32_t>> thin;  // work, front
-        for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++) {
-            const int32_t s = P.lvl_large[t];
+        for (int32_t s : large) {
             add_asm(s);
-            if (is_thin(s) && (P.child_ptr[s] == P.child_ptr[s + 1] || inner >= kThinInner)) {
+            if (is_thin(s) && (P.child_ptr[s] == P.child_ptr[s + 1] ? leaves : inner) >= kThinMin) {
                 thin.push_back({(double)P.sn_k[s] * P.sn_f[s] * P.sn_f[s], s});
                 const Work fr = front_work(s);
                 W.thin_w.flops += fr.flops;
@@ -1171,11 +1195,10 @@ int setup_device(ipm_ctx *c) {
             W.steps.push_back(S);
             if (S.tc_cnt > 0 || S.st_cnt > 0) W.has_tc = true;
         }
-        build_level_items(P, l, W, slot_of, lvl_items, cbase);
+        build_level_items(P, large, W, slot_of, lvl_items, cbase);
         {
             int32_t chain = 0;
-            for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++) {
-                const int32_t s = P.lvl_large[t];
+            for (int32_t s : large) {
                 const Work fr = front_work(s);
                 W.lvl_w.flops += fr.flops;
                 W.lvl_w.bytes += fr.bytes;
@@ -1204,6 +1227,10 @@ int setup_device(ipm_ctx *c) {
         for (int32_t l = 0; l < P.nlevels; l++) {
             for (int32_t t = P.lvl_large_ptr[l]; t < P.lvl_large_ptr[l + 1]; t++) {
                 const int32_t s = P.lvl_large[t];
+                if (rank1[s]) {
+                    gend[s] = -2;  // done before the first step
+                    continue;
+                }
                 int32_t g = 0;
                 for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
                     const int32_t ch = P.child_list[q];
@@ -1242,7 +1269,7 @@ int setup_device(ipm_ctx *c) {
             // fronts by start step; the active set advances one panel per step
             std::vector<std::vector<int32_t>> starting(T);
             for (int32_t s = 0; s < ns; s++)
-                if (P.sn_large[s]) starting[g0[s]].push_back(s);
+                if (P.sn_large[s] && !rank1[s]) starting[g0[s]].push_back(s);
             std::vector<int32_t> active;
             std::vector<std::pair<int32_t, int32_t>> fp;
             for (int32_t g = 0; g < T; g++) {
@@ -1270,7 +1297,13 @@ int setup_device(ipm_ctx *c) {
         }
     }
     c->steps_levels = steps_levels;
-    c->nfronts_thin = (int32_t)thin_list.size();
+    c->nfronts_thin = (int32_t)(thin_list.size() + rank1_list.size());
+    c->rank1_cnt = (int32_t)rank1_list.size();
+    c->rank1_w = Work();
+    for (int32_t s : rank1_list) {
+        c->rank1_w.flops += P.sn_f[s];
+        c->rank1_w.bytes += 28.0 * P.sn_f[s];
+    }
     std::vector<int64_t> upd_off(P.upd_off.begin(), P.upd_off.end());
     // children in the order their entries are summed: those the large fronts'
     // assembly takes as point lists first (the pivoting mode, without that
@@ -1307,7 +1340,7 @@ int setup_device(ipm_ctx *c) {
         (rc = dupload(c, &c->alt_items, alt_items)) || (rc = dupload(c, &c->bwd_order, bwd_order)) ||
         (rc = dupload(c, &c->trsm_sbase, trsm_sbase)) || (rc = dupload(c, &c->sliced_runs, sliced_runs)) || (rc = dupload(c, &c->sliced_segs, sliced_segs)) ||
         (rc = dupload(c, &c->thin_list, thin_list)) || (rc = dupload(c, &c->thin_asm, thin_asm)) ||
-        (rc = dupload(c, &c->thin_slot, thin_slot)) ||
+        (rc = dupload(c, &c->thin_slot, thin_slot)) || (rc = dupload(c, &c->rank1_list, rank1_list)) ||
         (rc = dalloc(c, &c->slice_ws, 3 * (size_t)max_slice_blocks * (size_t)kSliceBlockBytes)) ||
         (rc = dalloc(c, &c->slice_exp, 3 * (size_t)std::max<int64_t>(max_slice_blocks, 1) * kSliceRows * 2)) ||
         (rc = dupload(c, &c->lvl_items, lvl_items)) || (rc = dalloc(c, &c->lvl_sync, (size_t)max_ncnt + 1)) ||
@@ -1566,6 +1599,11 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
     }
     cudaStream_t sd = c->side, sd2 = c->side2, sd3 = c->side3;
     size_t sidx = 0;
+    if (c->rank1_cnt > 0) {
+        Prof pr(c, IPM_K_LARGE_PANEL, c->rank1_w, st);
+        launch_rank_one(c->dp, V, c->fronts, c->D, c->Dinv, c->dyn, c->ctl, c->rank1_list, c->rank1_cnt, st);
+        nl++;
+    }
     cudaEventRecord(c->dep_ev[0], st);
     cudaStreamWaitEvent(sd, c->dep_ev[0], 0);
     cudaEvent_t last_small = nullptr, last_large = nullptr;

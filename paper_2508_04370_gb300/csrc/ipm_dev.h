@@ -208,13 +208,13 @@ struct PanelItem {
 // among [o0, o1) (those of the columns) that lie in its rows; the entries of
 // the small children (contribution blocks of up to kPointRows rows) as one list
 // of arena positions per destination, [seg0, seg1) of AsmLists; the large
-// children [ch0, ch1).  Device child lists hold the small children before the
+// children [ch0, ch1); the rank-one leaves [ch1, ch2).  Device child lists hold the small children before the
 // large ones, so every path adds in this order.
 constexpr int kAsmRows = 64;
 constexpr int kPointRows = 64;
 struct AsmItem {
     int64_t o0, o1, seg0, seg1;
-    int32_t ch0, ch1, s, c_lo, c_hi, r_lo, r_hi;
+    int32_t ch0, ch1, ch2, s, c_lo, c_hi, r_lo, r_hi;
 };
 __host__ __device__ inline int32_t asm_tiles(int32_t f) {  // items of a front of f rows
     const int32_t nc = (f + 31) / 32, nr = (f + kAsmRows - 1) / kAsmRows;
@@ -222,6 +222,8 @@ __host__ __device__ inline int32_t asm_tiles(int32_t f) {  // items of a front o
 }
 // A large child's part in a block of columns: its columns [a, b) land there;
 // rt + i is where its rows of the front's i-th block of kAsmRows rows begin.
+// (Of a rank-one leaf cb is its column of L, row 1 first, and cb + ldc the
+// column -u, u = L d: entry (i, j) of its contribution is l_i (-u_j).)
 struct AsmChild {
     int64_t cb, map;  // its contribution block in the arena, its row map
     int32_t ldc, a, b, rt;
@@ -325,12 +327,17 @@ constexpr int64_t kWarpRow = 32;       // and longer than this a warp each (rows
 // thin fronts (k <= nb, f <= kThinMaxF), one CTA per front: list[i] the front,
 // first_asm[i] its first assembly item, slots[i] its panel workspace slot
 constexpr int kThinMaxF = 512;
-// Thin fronts with children take that path only where a level has this many:
-// one CTA assembles its front block by block (0.5 to 2 ms with ten to a hundred
-// children of 300 rows), where the per-step launches spread the blocks over the
-// chip (40 block-angular blocks with 300 dense rows, three levels of 10 to 200
-// such fronts: 5.9 ms as thin fronts, 1.2 through the steps).
-constexpr int kThinInner = 1024;
+// Leaves, and fronts with children, take that path only where a level has this
+// many of them: one CTA does its front block by block (0.5 to 2 ms assembling
+// ten to a hundred children of 300 rows, 0.3 ms for the products of a leaf of 16
+// columns and 360 rows), where the per-step launches spread the blocks over the
+// chip (40 block-angular blocks with 300 dense rows: three levels of 10 to 200
+// fronts with children 5.9 ms as thin fronts, 1.2 through the steps; 614 leaves
+// of 2 to 25 columns 1.59 ms against 1.06).
+constexpr int kThinMin = 1024;
+// rank-one leaves (large fronts of one column without children under a large front)
+void launch_rank_one(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
+                     DevCtl *ctl, const int32_t *list, int32_t count, cudaStream_t st);
 void launch_thin_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                         DevCtl *ctl, const int32_t *list, const int32_t *first_asm, const int32_t *slots,
                         const AsmLists &A, double *pws, int32_t count, int32_t nb, cudaStream_t st);

@@ -407,6 +407,48 @@ __device__ __forceinline__ void assemble_block(const DevPlan &P, const DevVals &
             m = n;
         }
     }
+    // rank-one leaves: formed here from their columns l and -u (the same
+    // FP64 work as adding a stored block), the next child's on their way
+    // while one is added
+    struct Rank1 {
+        double l0, l1, nu;
+        int a, col, i0, r0, r1;
+    };
+    auto leaf = [&](int q) {
+        const AsmChild C = A.child[min(q, ai.ch2 - 1)];
+        Rank1 m;
+        const int ilo = A.rt[C.rt + rbase / R], ihi = A.rt[C.rt + rbase / R + 1];
+        const int32_t *map = P.relmap + C.map;
+        const double *L = fronts + C.cb;
+        m.a = C.a;
+        const bool in = C.a + lane < C.b;
+        m.col = in ? __ldg(map + C.a + lane) - c_lo : -1;
+        m.nu = in ? __ldcg(L + C.ldc + C.a + lane) : 0.0;
+        m.i0 = ilo + lane;
+        m.r0 = m.i0 < ihi ? __ldg(map + m.i0) - rbase : -1;
+        m.r1 = m.i0 + 32 < ihi ? __ldg(map + m.i0 + 32) - rbase : -1;
+        m.l0 = m.i0 < ihi ? __ldcg(L + m.i0) : 0.0;
+        m.l1 = m.i0 + 32 < ihi ? __ldcg(L + m.i0 + 32) : 0.0;
+        return m;
+    };
+    if (ai.ch1 < ai.ch2) {
+        Rank1 m = leaf(ai.ch1);
+        for (int q = ai.ch1; q < ai.ch2; q++) {
+            const Rank1 n = leaf(q + 1);
+            unsigned mine = __ballot_sync(0xffffffffu, m.col >= 0 && (m.col & 7) == warp);
+            while (mine) {  // uniform over the warp
+                const int j = __ffs(mine) - 1;
+                mine &= mine - 1;
+                const int jj = m.a + j;
+                double *Tc = T + R * __shfl_sync(0xffffffffu, m.col, j);
+                const double nu = __shfl_sync(0xffffffffu, m.nu, j);
+                if (m.r0 >= 0 && m.i0 >= jj) Tc[m.r0] = fma(m.l0, nu, Tc[m.r0]);
+                if (m.r1 >= 0 && m.i0 + 32 >= jj) Tc[m.r1] = fma(m.l1, nu, Tc[m.r1]);
+            }
+            __syncwarp();
+            m = n;
+        }
+    }
     __syncthreads();
     for (int t = tid; t < 32 * R; t += NT) {
         const int c = c_lo + t / R, r = rbase + t % R;
@@ -953,6 +995,59 @@ __global__ void __launch_bounds__(kBodyThreads) k_large_update_strip(DevPlan P, 
     body_strip(P, fronts, Dg, it.s, it.i0, it.j0, it.p0, w, pool);
 }
 
+// A rank-one leaf: a large front of one column without children (a long
+// column of an LP, eliminated first).  Its contribution -l d l' is not formed
+// here: it would be f^2 / 2 numbers to write and read again, where the parent's
+// assembly needs one FMA per entry from l and u = l d (the unscaled column) just
+// as it needs one addition per stored entry.  So this kernel only scales the
+// column by the pivot's reciprocal (the pivot rule of body_diag with no other
+// candidate in the block) and leaves -u in the front's second column, and is
+// bound by its loads.  7,702 leaves of 300 rows (40 block-angular blocks with 300
+// dense rows): 33 us, and the assembly of their 40 parents no slower, where
+// forming their 2.8 GB of blocks took 1.9 ms of the factorisation's 7.9.
+constexpr int kRankOneThreads = 128;
+
+__global__ void __launch_bounds__(kRankOneThreads) k_rank_one(DevPlan P, DevVals V, double *__restrict__ fronts,
+                                                              double *__restrict__ Dg, double *__restrict__ Dig,
+                                                              double *__restrict__ dyng, DevCtl *ctl,
+                                                              const int32_t *__restrict__ list) {
+    __shared__ double sh_r;
+    const int s = list[blockIdx.x];
+    const int f = P.sn_f[s], ld = P.sn_ld[s], c0 = P.sn_c0[s];
+    const int tid = threadIdx.x;
+    double *F = fronts + P.sn_off[s];
+    const int64_t o0 = P.orig_ptr[s], o1 = P.orig_ptr[s + 1];
+    if (o1 - o0 < f) {
+        for (int i = tid; i < f; i += kRankOneThreads) F[i] = 0.0;
+        __syncthreads();
+    }
+    for (int64_t q = o0 + tid; q < o1; q += kRankOneThreads) F[P.orig_dst[q]] = orig_value(P, V, P.orig_src[q]);
+    __syncthreads();
+    if (tid == 0) {
+        const int sp = P.sign[c0];
+        const double d = F[0] + (sp < 0 ? -V.rho : V.delta);
+        const long long db = dbits(d), b1b = dbits(pivot_floor(P, ctl, c0));
+        const long long sdb = sp < 0 ? db ^ kSignBit : db;
+        const long long tb = gt_nonneg(sdb, b1b) ? sdb : b1b;
+        const long long dnb = sp < 0 ? tb ^ kSignBit : tb;
+        const double dn = __longlong_as_double(dnb), r = recip_pivot(dn);
+        const bool fin = (db & kAbsMask) < kInfBits && (dnb & kAbsMask) < kInfBits && (dnb & kAbsMask) != 0;
+        if (!fin) atomicOr(&ctl->status, kStatNonFinite);
+        F[0] = dn;
+        Dg[c0] = dn;
+        Dig[c0] = r;
+        dyng[c0] = dnb == db ? 0.0 : dn - d;
+        sh_r = r;
+    }
+    __syncthreads();
+    const double r = sh_r;
+    for (int i = 1 + tid; i < f; i += kRankOneThreads) {
+        const double u = F[i];
+        F[i] = u * r;
+        F[ld + i] = __longlong_as_double(dbits(u) ^ kSignBit);
+    }
+}
+
 // A thin front (one pivot block, k <= nb, f <= kThinMaxF) whole in one CTA.
 // Every entry gets the operations of the per-step path in its order, so the
 // front's values are those of that path bit for bit; what differs is what
@@ -960,11 +1055,9 @@ __global__ void __launch_bounds__(kBodyThreads) k_large_update_strip(DevPlan P, 
 // block is formed and written in one pass (0 minus the products where the front
 // has no children, assembled and updated block by block in shared memory
 // otherwise), and up to kThinCols pivot columns a thread solves a row by
-// itself.  With the per-step bodies in sequence a leaf of one column and 302
-// rows took about 0.9 ms of a CTA's time in barriers and round trips; now its
-// 46,000 products bound it (FP64, two per clock and SM).  40 block-angular
-// blocks with 300 dense rows: the launch of 8,317 leaves takes 3.4 ms (1.1 at the
-// FP64 rate), 17 ms with all thin fronts in the per-step bodies' sequence.
+// itself.  The products of a leaf bound it (FP64, two per clock and SM): 614
+// leaves of 2 to 25 columns and 300 to 376 rows take 1.6 ms (0.5 at the FP64
+// rate), too few to even out over the SMs; hence kThinMin.
 constexpr int kThinCols = 4;
 constexpr int kThinPanel = 6144;  // doubles of L kept (three CTAs per SM fit)
 __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevVals V, double *__restrict__ fronts,
@@ -1582,6 +1675,12 @@ void launch_large_update_strip(const DevPlan &P, double *fronts, const double *D
                                int32_t count, int32_t w, cudaStream_t st) {
     if (count <= 0) return;
     k_large_update_strip<<<count, kBodyThreads, 0, st>>>(P, fronts, D, items, w);
+}
+
+void launch_rank_one(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
+                     DevCtl *ctl, const int32_t *list, int32_t count, cudaStream_t st) {
+    if (count <= 0) return;
+    k_rank_one<<<count, kRankOneThreads, 0, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list);
 }
 
 void launch_thin_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,

@@ -70,7 +70,7 @@ def lp_with_thin_fronts(nlink, groups, private, seed):
 
 
 @pytest.mark.parametrize("nlink,groups,private", [(129, 6, 0), (130, 5, 3), (161, 4, 4), (300, 3, 12), (150, 3, 31),
-                                                  (490, 2, 20)])
+                                                  (490, 2, 20), (130, 1040, 3), (161, 1030, 5), (170, 1030, 31)])
 def test_thin_fronts(pkg, nlink, groups, private):
     lp = lp_with_thin_fronts(nlink, groups, private, nlink)
     theta = synth.theta_loguniform(lp.n, 5, -2.0, 2.0)
@@ -82,6 +82,28 @@ def test_thin_fronts(pkg, nlink, groups, private):
     for opts in (dict(schedule=pkg.IPM_SCHED_LEVELS, level_kernel=0), dict(schedule=pkg.IPM_SCHED_DEPENDENCY)):
         r = run_pair(pkg, lp, theta, r7, r1, ordering=pkg.IPM_ORD_USER, user_perm=perm, amalg_zero_frac=0.0,
                      **opts)
+        if groups >= 1024 or private == 0:  # fewer go through the steps
+            assert r["info"]["nfronts_thin"] > 0
+        check_pair(r, lp)
+        if base is None:
+            base = r
+        else:
+            assert np.array_equal(base["D"], r["D"]) and np.array_equal(base["L"], r["L"])
+        r["s"].close()
+
+
+@pytest.mark.parametrize("m,lengths", [(129, [129, 128, 129]), (160, [159, 131, 140, 129, 64, 160, 150]), (193, [193, 130, 160, 161, 192]),
+                                       (300, [129 + 7 * j for j in range(24)] + [65, 64, 1])])
+def test_rank_one_leaves(pkg, m, lengths):
+    """One-column leaves on subsets of m dense rows (runs and scattered rows, so
+    that blocks take all, some and none of a child's rows), beside stored ones."""
+    lp = lp_with_columns(m, lengths, m)
+    theta = synth.theta_loguniform(lp.n, 5, -3.0, 3.0)
+    r7, r1 = synth.rhs_normal(lp.n, 6), synth.rhs_normal(lp.m, 7)
+    base = None
+    for opts in (dict(schedule=pkg.IPM_SCHED_LEVELS, level_kernel=0), dict(schedule=pkg.IPM_SCHED_LEVELS, level_kernel=1),
+                 dict(schedule=pkg.IPM_SCHED_DEPENDENCY)):
+        r = run_pair(pkg, lp, theta, r7, r1, ordering=pkg.IPM_ORD_NATURAL, amalg_zero_frac=0.0, **opts)
         assert r["info"]["nfronts_thin"] > 0
         check_pair(r, lp)
         if base is None:
