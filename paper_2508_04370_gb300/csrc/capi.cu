@@ -1681,13 +1681,13 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             cudaStreamWaitEvent(sd2, ev_in, 0);
             if (rest_tiles > 0) {
                 Prof pr(c, IPM_K_LARGE_UPDATE, S.tile_w, sd2);
-                launch_large_update(c->dp, c->fronts, c->D, c->tile_items + S.tile_off + S.tile_cnt1, rest_tiles,
+                launch_large_update(c->dp, c->fronts, c->tile_items + S.tile_off + S.tile_cnt1, rest_tiles,
                                     c->opt.nb, sd2);
                 nl++;
             }
             if (rest_alt > 0) {
                 Prof pr(c, IPM_K_LARGE_UPDATE, S.alt_w, sd2);
-                launch_large_update(c->dp, c->fronts, c->D, c->alt_items + S.alt_off + S.alt_cnt1, rest_alt,
+                launch_large_update(c->dp, c->fronts, c->alt_items + S.alt_off + S.alt_cnt1, rest_alt,
                                     c->opt.nb, sd2);
                 nl++;
             }
@@ -1711,13 +1711,13 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
         if (sidx >= 3 && sliced_rest[sidx - 3]) cudaStreamWaitEvent(sd, sliced_rest[sidx - 3], 0);
         if (S.tile_cnt1 > 0) {
             Prof pr(c, IPM_K_LARGE_UPDATE, S.tile_w1, sd);
-            launch_large_update_strip(c->dp, c->fronts, c->D, c->tile_items + S.tile_off, S.tile_cnt1, c->opt.nb,
+            launch_large_update_strip(c->dp, c->fronts, c->tile_items + S.tile_off, S.tile_cnt1, c->opt.nb,
                                       sd);
             nl++;
         }
         if ((S.tc_cnt > 0 || S.st_cnt > 0) && !c->mixed_active && S.alt_cnt1 > 0) {
             Prof pr(c, IPM_K_LARGE_UPDATE, S.alt_w1, sd);
-            launch_large_update_strip(c->dp, c->fronts, c->D, c->alt_items + S.alt_off, S.alt_cnt1, c->opt.nb, sd);
+            launch_large_update_strip(c->dp, c->fronts, c->alt_items + S.alt_off, S.alt_cnt1, c->opt.nb, sd);
             nl++;
         } else if (use_sliced) {
             if (S.st_cnt1 > 0) {

@@ -320,7 +320,7 @@ constexpr int kTrsmRowsHost = 8;       // rows of a triangular-solve chunk of th
 constexpr int kTrsmItemRowsHost = 32;  // rows of a triangular-solve item of the one-launch-per-step kernel,
 constexpr int64_t kTrsmFewRows = 2432; // or of a chunk where the step has no more rows than this (two chunks per SM)
 constexpr int kPanelWsHost = 32 * 33 + 32;
-void launch_large_update_strip(const DevPlan &P, double *fronts, const double *D, const TileItem *items,
+void launch_large_update_strip(const DevPlan &P, double *fronts, const TileItem *items,
                                int32_t count, int32_t w, cudaStream_t st);
 constexpr int64_t kLongColumn = 2048;  // longer sums over a sparse row take a CTA each
 constexpr int64_t kWarpRow = 32;       // and longer than this a warp each (rows_common.cuh)
@@ -346,7 +346,7 @@ void launch_large_level(const DevPlan &P, const DevVals &V, double *fronts, doub
                         const AsmLists &A, double *pws, int32_t nb, int32_t grid, long long spin_limit,
                         cudaStream_t st);
 const void *large_level_kernel();
-void launch_large_update(const DevPlan &P, double *fronts, const double *D, const TileItem *items, int32_t count,
+void launch_large_update(const DevPlan &P, double *fronts, const TileItem *items, int32_t count,
                          int32_t w, cudaStream_t st);
 void launch_large_update_tc(const DevPlan &P, double *fronts, const double *D, const TileItem *items, int32_t count,
                             int32_t w, DevCtl *ctl, cudaStream_t st);

@@ -695,6 +695,13 @@ __device__ __forceinline__ void body_diag(const DevPlan &P, const DevVals &V, do
 // level kernel hold kTrsmRows); warp w solves rows w, w + 8, w + 16 and
 // w + 24 together, four independent chains on the same L_11, so a CTA costs
 // about one chain's latency.
+//
+// The unscaled u_iq = l_iq d_q, which the FP64 updates take as their second
+// operand, is left at the mirrored place (row p0 + q, column i of the front's
+// unused upper part): a product per operand entry and tile was 3% of the updates'
+// FP64 work, which bounds them.  A factorisation of the 10-period staircase in
+// FP64 takes 74.2 ms instead of 77.0, of 64 random LPs at once 15.0 instead of
+// 15.5.  (Not for rows that are sliced for the tensor cores.)
 constexpr int kTrsmRows = 8;
 constexpr int kTrsmItemRows = 32;
 static_assert(kTrsmRows == kTrsmRowsHost && kTrsmItemRows == kTrsmItemRowsHost, "host and device row chunks differ");
@@ -774,8 +781,12 @@ __device__ __forceinline__ void body_trsm(const DevPlan &P, double *__restrict__
                 for (int b = c >> 3; b < 4; b++)
                     if (8 * b + e > c) t[b] -= u * Wd[(8 * b + e) * 33 + c];
             }
+            double *U = F + (int64_t)(r0 + rr) * ld + p0;
 #pragma unroll
-            for (int b = 0; b < 4; b++) T[8 * b + e][rr] = t[b] * Wd[32 * 33 + 8 * b + e];
+            for (int b = 0; b < 4; b++) {
+                if (!so.ws && rr < nr && 8 * b + e < w) U[8 * b + e] = t[b];
+                T[8 * b + e][rr] = t[b] * Wd[32 * 33 + 8 * b + e];
+            }
         }
         __syncwarp();
     } else if (warp < nr) {
@@ -789,6 +800,7 @@ __device__ __forceinline__ void body_trsm(const DevPlan &P, double *__restrict__
             const double u = __shfl_sync(0xffffffffu, t, c);
             if (lane > c) t -= u * Lr[c];
         }
+        if (!so.ws && lane < w) F[(int64_t)(r0 + warp) * ld + p0 + lane] = t;
         T[lane][warp] = t * Wd[32 * 33 + lane];
         __syncwarp();
     }
@@ -823,18 +835,18 @@ __device__ __forceinline__ void body_trsm(const DevPlan &P, double *__restrict__
 }
 
 // Trailing update of the lower part of columns [p1, f) by the panel
-// [p0, p0+w): C(i, j) -= sum_q L(i,q) d_q L(j,q), one kUpdTile x kUpdTile
+// [p0, p0+w): C(i, j) -= sum_q L(i,q) u(j,q), u = L d, one kUpdTile x kUpdTile
 // tile at (i0, j0), 16 x 16 threads with 2 x 2 outputs each.  FP64 runs at
 // about 2 FMA per clock per SM on this GPU, so tiles are small (32 x 32) to
 // put every SM to work.
 __device__ __forceinline__ void body_tile(const DevPlan &P, double *__restrict__ fronts,
-                                          const double *__restrict__ Dg, int s, int i0, int j0, int p0, int w,
+                                          int s, int i0, int j0, int p0, int w,
                                           double *pool) {
     constexpr int T = kUpdTile;
     static_assert(T == 32, "16 x 16 threads, 2 x 2 outputs");
     double(*As)[T + 1] = reinterpret_cast<double(*)[T + 1]>(pool);
     double(*Bs)[T + 1] = reinterpret_cast<double(*)[T + 1]>(pool + 32 * (T + 1));
-    const int f = P.sn_f[s], ld = P.sn_ld[s], c0 = P.sn_c0[s];
+    const int f = P.sn_f[s], ld = P.sn_ld[s];
     w = min(w, P.sn_k[s] - p0);  // ragged last panel
     double *F = fronts + P.sn_off[s];
     const int tid = threadIdx.x;
@@ -855,21 +867,20 @@ __device__ __forceinline__ void body_tile(const DevPlan &P, double *__restrict__
     {
         // all loads in flight before the shared-memory stores
         constexpr int U = 32 * T / kBodyThreads;
-        double va[U], vb[U], vd[U];
+        double va[U], vb[U];
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int t = tid + u * kBodyThreads, q = t / T, r = t % T;
-            const int i = i0 + r, j = j0 + r;
-            const bool qa = q < w;
-            va[u] = (qa && i < f) ? __ldcg(F + (int64_t)(p0 + q) * ld + i) : 0.0;
-            vb[u] = (qa && j < f) ? __ldcg(F + (int64_t)(p0 + q) * ld + j) : 0.0;
-            vd[u] = qa ? __ldcg(Dg + c0 + p0 + q) : 0.0;
+            const int i = i0 + r, j = j0 + q;
+            va[u] = (q < w && i < f) ? __ldcg(F + (int64_t)(p0 + q) * ld + i) : 0.0;
+            // u_jr at its mirrored place (columns before the panel's end have none)
+            vb[u] = (r < w && j < f && j >= p0 + w) ? __ldcg(F + (int64_t)j * ld + p0 + r) : 0.0;
         }
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int t = tid + u * kBodyThreads, q = t / T, r = t % T;
             As[q][r] = va[u];
-            Bs[q][r] = vb[u] * vd[u];
+            Bs[r][q] = vb[u];
         }
     }
     __syncthreads();
@@ -901,13 +912,13 @@ __device__ __forceinline__ void body_tile(const DevPlan &P, double *__restrict__
 // whole 32 x 32 tile is 32k FP64 FMAs, about 8 us on one SM of this GPU;
 // strips spread those few tiles over eight times as many SMs.
 __device__ __forceinline__ void body_strip(const DevPlan &P, double *__restrict__ fronts,
-                                           const double *__restrict__ Dg, int s, int i0, int j0, int p0, int w,
+                                           int s, int i0, int j0, int p0, int w,
                                            double *pool) {
     constexpr int T = kUpdTile, C = kStripCols;
     static_assert(T == 32 && 32 * C <= kBodyThreads, "one row per lane, one column per warp");
     double(*As)[T + 1] = reinterpret_cast<double(*)[T + 1]>(pool);
     double(*Bs)[C] = reinterpret_cast<double(*)[C]>(pool + 32 * (T + 1));
-    const int f = P.sn_f[s], ld = P.sn_ld[s], c0 = P.sn_c0[s];
+    const int f = P.sn_f[s], ld = P.sn_ld[s];
     w = min(w, P.sn_k[s] - p0);
     double *F = fronts + P.sn_off[s];
     const int tid = threadIdx.x;
@@ -920,18 +931,15 @@ __device__ __forceinline__ void body_strip(const DevPlan &P, double *__restrict_
             const int t = tid + u * kBodyThreads, q = t / T, r = t % T;
             va[u] = (q < w && i0 + r < f) ? __ldcg(F + (int64_t)(p0 + q) * ld + i0 + r) : 0.0;
         }
-        double vb = 0.0, vd = 0.0;
-        const int q = tid / C, cc = tid % C, j = j0 + cc;
-        if (tid < 32 * C && q < w && j < f) {
-            vb = __ldcg(F + (int64_t)(p0 + q) * ld + j);
-            vd = __ldcg(Dg + c0 + p0 + q);
-        }
+        double vb = 0.0;
+        const int q = tid & 31, cc = tid >> 5, j = j0 + cc;
+        if (cc < C && q < w && j < f && j >= p0 + w) vb = __ldcg(F + (int64_t)j * ld + p0 + q);
 #pragma unroll
         for (int u = 0; u < U; u++) {
             const int t = tid + u * kBodyThreads;
             As[t / T][t % T] = va[u];
         }
-        if (tid < 32 * C) Bs[q][cc] = vb * vd;
+        if (cc < C) Bs[q][cc] = vb;
     }
     __syncthreads();
     const int r = tid & 31, cc = tid >> 5;
@@ -980,19 +988,17 @@ __global__ void __launch_bounds__(kBodyThreads) k_panel_trsm(DevPlan P, double *
 }
 
 __global__ void __launch_bounds__(kBodyThreads) k_large_update(DevPlan P, double *__restrict__ fronts,
-                                                                const double *__restrict__ Dg,
                                                                 const TileItem *__restrict__ items, int w) {
     __shared__ double pool[kPoolDoubles];
     const TileItem it = items[blockIdx.x];
-    body_tile(P, fronts, Dg, it.s, it.i0, it.j0, it.p0, w, pool);
+    body_tile(P, fronts, it.s, it.i0, it.j0, it.p0, w, pool);
 }
 
 __global__ void __launch_bounds__(kBodyThreads) k_large_update_strip(DevPlan P, double *__restrict__ fronts,
-                                                                        const double *__restrict__ Dg,
                                                                         const TileItem *__restrict__ items, int w) {
     __shared__ double pool[kPoolDoubles];
     const TileItem it = items[blockIdx.x];
-    body_strip(P, fronts, Dg, it.s, it.i0, it.j0, it.p0, w, pool);
+    body_strip(P, fronts, it.s, it.i0, it.j0, it.p0, w, pool);
 }
 
 // A rank-one leaf: a large front of one column without children (a long
@@ -1051,7 +1057,7 @@ __global__ void __launch_bounds__(kRankOneThreads) k_rank_one(DevPlan P, DevVals
 // A thin front (one pivot block, k <= nb, f <= kThinMaxF) whole in one CTA.
 // Every entry gets the operations of the per-step path in its order, so the
 // front's values are those of that path bit for bit; what differs is what
-// moves: the rows of L and L d are kept in shared memory, the contribution
+// moves: the rows of L are kept in shared memory, the contribution
 // block is formed and written in one pass (0 minus the products where the front
 // has no children, assembled and updated block by block in shared memory
 // otherwise), and up to kThinCols pivot columns a thread solves a row by
@@ -1069,9 +1075,9 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
                                                                AsmLists A, double *__restrict__ pws, int nb) {
     extern __shared__ double panel[];
     __shared__ double pool[kPoolDoubles];
-    __shared__ double Bt[32][33];  // L(c, q) d_q of a block's columns
+    __shared__ double Bt[32][33];  // u(c, q) of a block's columns
     const int s = list[blockIdx.x];
-    const int f = P.sn_f[s], k = P.sn_k[s], ld = P.sn_ld[s], c0 = P.sn_c0[s];
+    const int f = P.sn_f[s], k = P.sn_k[s], ld = P.sn_ld[s];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     double *F = fronts + P.sn_off[s];
     const int64_t a0 = first_asm[blockIdx.x];
@@ -1108,7 +1114,10 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
             }
 #pragma unroll
             for (int q = 0; q < kThinCols; q++)
-                if (q < k) F[(int64_t)q * ld + i] = u[q] * ws[32 * 33 + q];
+                if (q < k) {
+                    F[(int64_t)i * ld + q] = u[q];
+                    F[(int64_t)q * ld + i] = u[q] * ws[32 * 33 + q];
+                }
         }
         __syncthreads();
     } else {
@@ -1129,9 +1138,11 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
     // columns of the contribution block with nothing assembled beside them: all
     // of a leaf's, else those of the first block (whose values are in the slab)
     const int c_end = leaf ? f : min(32, f);
-    const double dq = lane < k ? Dg[c0 + lane] : 0.0;
+    auto u_of = [&](int j) { return j < c_end && lane < k ? __ldcg(F + (int64_t)j * ld + lane) : 0.0; };
+    double bn = u_of(k + warp);
     for (int j = k + warp; j < c_end; j += kBodyThreads / 32) {
-        const double b = lane < k ? Lp[lane * ls + j] * dq : 0.0;
+        const double b = bn;
+        bn = u_of(j + kBodyThreads / 32);
         constexpr int U = 4;  // rows a lane carries together
         for (int i0 = j + lane; i0 - lane < f; i0 += 32 * U) {
             double acc[U];
@@ -1162,9 +1173,9 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
     for (int a = nr, na = asm_tiles(f); a < na; a++) {
         const AsmItem ai = A.items[a0 + a];
         __syncthreads();
-        for (int t = tid; t < 32 * k; t += kBodyThreads) {
-            const int q = t >> 5, c = ai.c_lo + (t & 31);
-            Bt[t & 31][q] = c < f ? Lp[q * ls + c] * Dg[c0 + q] : 0.0;
+        for (int t = tid; t < 32 * 32; t += kBodyThreads) {
+            const int q = t & 31, c = ai.c_lo + (t >> 5);
+            if (q < k) Bt[t >> 5][q] = c < f ? __ldcg(F + (int64_t)c * ld + q) : 0.0;
         }
         assemble_block(P, V, fronts, A, ai, pool, [&](int r, int c, double v) {
             if (r < c) return;
@@ -1244,8 +1255,8 @@ __global__ void __launch_bounds__(kBodyThreads) k_large_level(DevPlan P, DevVals
             case kItemTrsm:
                 body_trsm<1>(P, fronts, it.s, it.a, it.b, it.t * nb, nb, pws + (int64_t)it.aux * kPanelWs, pool);
                 break;
-            case kItemStrip: body_strip(P, fronts, Dg, it.s, it.a, it.b, it.t * nb, nb, pool); break;
-            default: body_tile(P, fronts, Dg, it.s, it.a, it.b, it.t * nb, nb, pool); break;
+            case kItemStrip: body_strip(P, fronts, it.s, it.a, it.b, it.t * nb, nb, pool); break;
+            default: body_tile(P, fronts, it.s, it.a, it.b, it.t * nb, nb, pool); break;
         }
         // publish: the CTA barrier orders every thread's stores before thread 0's
         // fence, which makes them visible device-wide before the counter
@@ -1665,16 +1676,16 @@ void launch_panel_trsm(const DevPlan &P, double *fronts, const PanelItem *items,
         k_panel_trsm<1><<<count, kBodyThreads, 0, st>>>(P, fronts, items, slots, nb, pws, sbase, sws, sexp, D, ctl);
 }
 
-void launch_large_update(const DevPlan &P, double *fronts, const double *D, const TileItem *items, int32_t count,
+void launch_large_update(const DevPlan &P, double *fronts, const TileItem *items, int32_t count,
                          int32_t w, cudaStream_t st) {
     if (count <= 0) return;
-    k_large_update<<<count, kBodyThreads, 0, st>>>(P, fronts, D, items, w);
+    k_large_update<<<count, kBodyThreads, 0, st>>>(P, fronts, items, w);
 }
 
-void launch_large_update_strip(const DevPlan &P, double *fronts, const double *D, const TileItem *items,
+void launch_large_update_strip(const DevPlan &P, double *fronts, const TileItem *items,
                                int32_t count, int32_t w, cudaStream_t st) {
     if (count <= 0) return;
-    k_large_update_strip<<<count, kBodyThreads, 0, st>>>(P, fronts, D, items, w);
+    k_large_update_strip<<<count, kBodyThreads, 0, st>>>(P, fronts, items, w);
 }
 
 void launch_rank_one(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
