@@ -53,6 +53,7 @@
 
 #include <cstdint>
 
+#include "digit_sum.h"
 #include "ipm_dev.h"
 #include "tc_common.cuh"
 #include "sliced_common.cuh"
@@ -80,9 +81,9 @@ __device__ __forceinline__ double int_scaled(long long t, int e, bool &far) {
 }
 
 // 128 a + b for accumulators a, b: FP32 integers below 2^22.
-__device__ __forceinline__ int acc_pair(uint32_t a, uint32_t b) {
-    const int ia = __float_as_int(__uint_as_float(a) + 12582912.0f), ib = __float_as_int(__uint_as_float(b) + 12582912.0f);
-    return ia * 128 + (ib - (int)(129u * 0x4B400000u));
+__device__ __forceinline__ int32_t acc_pair(uint32_t a, uint32_t b) {
+    return sliced::digit_pair(__float_as_uint(__uint_as_float(a) + 12582912.0f),
+                              __float_as_uint(__uint_as_float(b) + 12582912.0f));
 }
 
 // C(i, j) -= sum_q L(i, q) d_q L(j, q), i >= j, for runs of 128 x 32 tiles.
@@ -311,13 +312,13 @@ __global__ void __maxnreg__(112)
                 // dropped are far below the truncation of the digit products with
                 // t + u >= 8.  S_4..S_7 first, to keep the registers low.
                 uint32_t v[4][8];
-                long long t[8];
+                int64_t t[8];
 #pragma unroll
                 for (int d = 0; d < 4; d++) tc::tmem_ld8(lane_base + (uint32_t)((d + 4) * kSliceCols + c0), v[d]);
                 tc::tmem_wait_ld();
 #pragma unroll
                 for (int c = 0; c < 8; c++)
-                    t[c] = (long long)acc_pair(v[0][c], v[1][c]) * 64 + (acc_pair(v[2][c], v[3][c]) >> 8);
+                    t[c] = sliced::digit_low(acc_pair(v[0][c], v[1][c]), acc_pair(v[2][c], v[3][c]));
 #pragma unroll
                 for (int d = 0; d < 4; d++) tc::tmem_ld8(lane_base + (uint32_t)(d * kSliceCols + c0), v[d]);
                 tc::tmem_wait_ld();
@@ -328,10 +329,8 @@ __global__ void __maxnreg__(112)
                     if (lane == 0) tc::mbar_arrive(&bar_empty[st]);
                 }
 #pragma unroll
-                for (int c = 0; c < 8; c++) {
-                    t[c] += (long long)acc_pair(v[2][c], v[3][c]) * (1 << 20);
-                    t[c] += (long long)acc_pair(v[0][c], v[1][c]) << 34;
-                }
+                for (int c = 0; c < 8; c++)
+                    t[c] = sliced::digit_sum(t[c], acc_pair(v[0][c], v[1][c]), acc_pair(v[2][c], v[3][c]));
                 double x[8];
                 unsigned far = 0;
 #pragma unroll
