@@ -164,7 +164,8 @@ typedef struct ipm_info {
     int64_t nnz_ne_seen;                    /* entries of A A^T counted before the chooser stopped */
     int32_t precision_fallbacks;            /* mixed path: refactorisations in FP64 so far */
     int32_t mixed_active;                   /* 1 while tensor-core updates are in use */
-    int32_t tune_small_threads[3];          /* threads per small-front CTA, size classes f <= 32, 64, 128 */
+    int32_t tune_small_threads[3];          /* threads per small-front CTA, size classes f <= 32, 64, 128 (the
+                                               base width where tune_small_by_count is 1) */
     double tune_level_ratio;                /* level-kernel threshold (see ipm_autotune) */
     double tune_ms;                         /* best factorisation time the autotuner measured; 0 before */
     double amalg_zero_frac;                 /* amalgamation threshold the analysis used */
@@ -177,6 +178,9 @@ typedef struct ipm_info {
     int32_t nfronts_thin;                   /* large fronts of one pivot block (k <= 32, f <= 512, FP64 updates)
                                                that a level outside the level kernel runs whole, one CTA each, and
                                                the one-column leaves under a large front */
+    int32_t tune_small_by_count[3];         /* 1: each launch of the class takes the base width times 4 with at
+                                               most one front per SM, times 2 with at most four (256 threads at
+                                               most); 0: the one width reported above */
 } ipm_info;
 
 /* Fill *opt with the defaults listed above. */
@@ -373,8 +377,10 @@ int ipm_solve_noalloc(ipm_ctx *ctx, const double *r7_dev, const double *r1_dev, 
  *     persistent launch when their FP64 work at 1 TFLOP/s is below ratio x
  *     (35 us per 32-column panel of its widest front); candidates 0 (never),
  *     0.25, 0.5, 1 (default), 2, 1e30 (always);
- *   - the threads per small-front CTA of each size class present (f <= 32:
- *     32 or 64; f <= 64: 64 or 128; f <= 128: 128 or 256);
+ *   - the threads per small-front CTA of each size class present: by each
+ *     launch's number of fronts (default, see ipm_set_launch_shapes), or one
+ *     width for the class (f <= 32: 32 or 64; f <= 64: 64 or 128; f <= 128:
+ *     128 or 256);
  *   - the level kernel's CTAs per SM: as many as fit (default) or one (see
  *     ipm_set_level_ctas).
  * The choices never change the arithmetic of any entry: the factors are the
@@ -389,7 +395,9 @@ int ipm_autotune(ipm_ctx *ctx, const double *theta_dev, double rho, double delta
 /* Set the launch shapes ipm_autotune would choose, e.g. to reproduce a
  * configuration: small_threads (host, 3 entries, may be NULL to keep) gives
  * the threads per small-front CTA of the size classes f <= 32, 64, 128, each
- * 32, 64, 128, 256 or 0 (the default 32 / 64 / 128); level_ratio >= 0 sets
+ * 32, 64, 128, 256 or 0 (the default: 32 / 64 / 128, times 4 in a launch of at
+ * most one front per SM and times 2 at up to four, at most 256; ipm_get_info
+ * reports this as tune_small_by_count); level_ratio >= 0 sets
  * the level-kernel threshold (a negative value keeps it).  Results are the
  * same bit for bit whatever the shapes.  Takes effect at the next
  * factorisation (not in an already captured graph).

@@ -85,13 +85,14 @@ class ipm_info(ct.Structure):
         ("tune_small_threads", ct.c_int32 * 3), ("tune_level_ratio", ct.c_double), ("tune_ms", ct.c_double),
         ("amalg_zero_frac", ct.c_double), ("tune_level_ctas_per_sm", ct.c_int32), ("graph_kernels", ct.c_int32),
         ("schedule", ct.c_int32), ("steps_levels", ct.c_int32), ("steps_dependency", ct.c_int32),
-        ("nfronts_thin", ct.c_int32),
+        ("nfronts_thin", ct.c_int32), ("tune_small_by_count", ct.c_int32 * 3),
     ]
 
     def as_dict(self):
         d = {name: getattr(self, name) for name, _ in self._fields_}
         d["omega_hist"] = list(self.omega_hist)[: min(16, max(self.refine_steps - self.gmres_iters + 1, 1))]
         d["tune_small_threads"] = list(self.tune_small_threads)
+        d["tune_small_by_count"] = [bool(v) for v in self.tune_small_by_count]
         return d
 
 

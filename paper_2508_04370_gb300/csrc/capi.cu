@@ -143,7 +143,7 @@ struct ipm_ctx {
     int32_t lvl_grid = 1;  // CTAs of the level kernel: every SM full
     int32_t sms = 1;       // SMs of the device
     // choices of ipm_autotune: threads per small-front CTA by size class
-    // (0: 32 / 64 / 128), the level-kernel threshold and the level kernel's
+    // (0: by the launch's count, small_front_threads), the level-kernel threshold and the level kernel's
     // CTAs per SM (0: as many as fit).  One CTA per SM leaves each SM
     // sub-partition's FP64 pipe to one CTA's pivot chain; two keep more
     // trailing tiles in flight.
@@ -946,7 +946,7 @@ int setup_device(ipm_ctx *c) {
         // where a step has so few rows that 32 leave SMs idle
         int64_t step_rows = 0;
         for (const auto &e : fp) step_rows += P.sn_f[e.first] - std::min(e.second + c->opt.nb, P.sn_k[e.first]);
-        const int32_t trsm_rows = step_rows > kTrsmFewRows ? kTrsmItemRowsHost : kTrsmRowsHost;
+        const int32_t trsm_rows = step_rows > (int64_t)kTrsmFewRows * c->sms ? kTrsmItemRowsHost : kTrsmRowsHost;
         S.trsm_rows = trsm_rows;
         int32_t nblk = 0;  // slice blocks of this step
         std::vector<SlicedRun> t1, t2;  // sliced runs: next panel's columns / the rest (whole rows, cut below)
@@ -1619,7 +1619,10 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             if (q > 0) cudaStreamWaitEvent(sq, fork, 0);
             Prof pr(c, IPM_K_SMALL_FRONTS, C.w, sq);
             launch_small_fronts(c->dp, V, c->fronts, c->D, c->Dinv, c->dyn, c->ctl, c->al, c->lvl_small + C.off, C.cnt,
-                                c->opt.nb, C.maxf, c->tune_threads[C.cls], sq);
+                                c->opt.nb, C.maxf,
+                                c->tune_threads[C.cls] > 0 ? c->tune_threads[C.cls]
+                                                           : small_front_threads(C.cls, C.cnt, c->sms),
+                                sq);
             nl++;
             if (q > 0) {
                 cudaEvent_t join = c->dep_ev[2 + 5 * l + (q - 1)];
@@ -2361,13 +2364,14 @@ int ipm_autotune(ipm_ctx *c, const double *theta_dev, double rho, double delta, 
             }
         }
         c->tune_ratio = pick;
-        const int32_t widths[3][2] = {{32, 64}, {64, 128}, {128, 256}};
+        // by the launches' counts, or one width for the whole class
+        const int32_t widths[3][3] = {{0, 32, 64}, {0, 64, 128}, {0, 128, 256}};
         for (int b = 0; b < 3; b++) {
             if (!present[b]) continue;
             const int32_t t0 = c->tune_threads[b];
             int32_t keep = t0;
             for (int32_t w : widths[b]) {
-                if (w == t0 || (t0 == 0 && w == widths[b][0])) continue;  // 0 is the first width
+                if (w == t0) continue;
                 c->tune_threads[b] = w;
                 double ms;
                 if ((rc = measure(ms))) goto done;
@@ -2705,8 +2709,8 @@ int ipm_get_info(ipm_ctx *c, ipm_info *out) {
     out->refine_steps = c->refine_steps;
     out->gmres_iters = c->gmres_iters;
     for (int b = 0; b < 3; b++) {
-        const int32_t dflt = b == 0 ? 32 : b == 1 ? 64 : 128;
-        out->tune_small_threads[b] = c->tune_threads[b] > 0 ? c->tune_threads[b] : dflt;
+        out->tune_small_by_count[b] = c->tune_threads[b] == 0;
+        out->tune_small_threads[b] = c->tune_threads[b] > 0 ? c->tune_threads[b] : kSmallBaseWidth[b];
     }
     out->tune_level_ratio = c->tune_ratio;
     out->tune_level_ctas_per_sm = c->dev_ready ? level_grid(c) / c->sms : 0;

@@ -299,6 +299,19 @@ struct FactorItem {
 // ---------------------------------------------------------------- launches
 // factorisation (kernels_factor.cu)
 void launch_norm1(const DevPlan &P, const DevVals &V, DevCtl *ctl, double eps_piv, cudaStream_t st);
+// Threads per CTA of a small-front launch (32, 64, 128 or 256; the same arithmetic
+// per entry whatever the width).  By default one warp per front up to f = 32, two
+// up to 64, four beyond, and more where the launch leaves SMs idle (at most four
+// fronts per SM, at most one): a front's pivots then run on all four
+// sub-partitions' FP64 pipes (factorisation of a 31 x 31 grid with 12 levels of
+// 10 to 600 fronts 0.86 -> 0.72 ms; a 64 x 64 grid, whose lower levels fill the
+// chip, loses 1% with the wide CTAs there, so the autotuner tries the fixed
+// widths too).
+constexpr int32_t kSmallBaseWidth[3] = {32, 64, 128};  // by size class f <= 32, 64, 128
+inline int32_t small_front_threads(int32_t cls, int32_t count, int32_t sms) {
+    const int32_t w = kSmallBaseWidth[cls] * (count <= sms ? 4 : count <= 4 * sms ? 2 : 1);
+    return w < 256 ? w : 256;
+}
 void launch_small_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                          DevCtl *ctl, const AsmLists &A, const int32_t *list, int32_t count, int32_t nb, int32_t maxf,
                          int32_t threads, cudaStream_t st);
@@ -318,7 +331,7 @@ void launch_panel_trsm(const DevPlan &P, double *fronts, const PanelItem *items,
                        DevCtl *ctl = nullptr);
 constexpr int kTrsmRowsHost = 8;       // rows of a triangular-solve chunk of the level kernel
 constexpr int kTrsmItemRowsHost = 32;  // rows of a triangular-solve item of the one-launch-per-step kernel,
-constexpr int64_t kTrsmFewRows = 2432; // or of a chunk where the step has no more rows than this (two chunks per SM)
+constexpr int32_t kTrsmFewRows = 16;   // or of a chunk where the step has no more rows per SM than this (two chunks)
 constexpr int kPanelWsHost = 32 * 33 + 32;
 void launch_large_update_strip(const DevPlan &P, double *fronts, const TileItem *items,
                                int32_t count, int32_t w, cudaStream_t st);

@@ -1632,18 +1632,6 @@ void launch_small_fronts(const DevPlan &P, const DevVals &V, double *fronts, dou
         cudaFuncSetAttribute(k_small_fronts<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         cudaFuncSetAttribute(k_small_fronts<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     }
-    // default: one warp per front up to f = 32, two up to 64, four beyond, and
-    // more where the launch leaves SMs idle: a front's pivots then run on all four
-    // sub-partitions' FP64 pipes (factorisation of a 31 x 31 grid with 12 levels
-    // of 10 to 600 fronts 0.86 -> 0.72 ms; a 64 x 64 grid, whose lower levels
-    // fill the chip, loses 1% with the wide CTAs there).  The autotuner may
-    // choose any of 32, 64, 128, 256 (same arithmetic per entry whatever the width).
-    if (threads <= 0) {
-        threads = maxf <= 32 ? 32 : maxf <= 64 ? 64 : 128;
-        if (count <= 608) threads *= 2;
-        if (count <= 152) threads *= 2;
-        if (threads > 256) threads = 256;
-    }
     switch (threads) {
         case 32: k_small_fronts<32><<<count, 32, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, A, list, nb); break;
         case 64: k_small_fronts<64><<<count, 64, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, A, list, nb); break;
