@@ -175,12 +175,14 @@ typedef struct ipm_info {
                                                IPM_SCHED_DEPENDENCY */
     int32_t steps_levels;                   /* 32-column steps of the large fronts in the level order */
     int32_t steps_dependency;               /* ... in the dependency order */
-    int32_t nfronts_thin;                   /* large fronts of one pivot block (k <= 32, f <= 512, FP64 updates)
-                                               that a level outside the level kernel runs whole, one CTA each, and
-                                               the one-column leaves under a large front */
+    int32_t nfronts_thin;                   /* large fronts run whole, one CTA each: the thin leaves (one pivot block,
+                                               FP64 updates) of levels outside the level kernel that have many,
+                                               and the rank-one leaves */
     int32_t tune_small_by_count[3];         /* 1: each launch of the class takes the base width times 4 with at
                                                most one front per SM, times 2 with at most four (256 threads at
                                                most); 0: the one width reported above */
+    int32_t nfronts_rank_one;               /* of nfronts_thin, the one-column leaves under a large front (f > 65):
+                                               their contributions are formed in the parent's assembly */
 } ipm_info;
 
 /* Fill *opt with the defaults listed above. */

@@ -86,6 +86,7 @@ class ipm_info(ct.Structure):
         ("amalg_zero_frac", ct.c_double), ("tune_level_ctas_per_sm", ct.c_int32), ("graph_kernels", ct.c_int32),
         ("schedule", ct.c_int32), ("steps_levels", ct.c_int32), ("steps_dependency", ct.c_int32),
         ("nfronts_thin", ct.c_int32), ("tune_small_by_count", ct.c_int32 * 3),
+        ("nfronts_rank_one", ct.c_int32),
     ]
 
     def as_dict(self):

@@ -126,7 +126,7 @@ struct ipm_ctx {
     int32_t *rank1_list = nullptr;  // rank-one leaves (k_rank_one)
     int32_t rank1_cnt = 0;
     Work rank1_w;
-    int32_t *thin_list = nullptr, *thin_asm = nullptr, *thin_slot = nullptr;  // thin fronts by level
+    int32_t *thin_list = nullptr, *thin_slot = nullptr;  // thin fronts by level
     double *panel_ws = nullptr;
     TileItem *tile_items = nullptr, *tc_items = nullptr, *alt_items = nullptr;
     SlicedRun *sliced_runs = nullptr;  // sliced tensor-core path: runs of output tiles
@@ -780,7 +780,7 @@ int setup_device(ipm_ctx *c) {
     std::vector<int64_t> seg_ptr(1, 0), seg_src;
     std::vector<int64_t> first_item(P.nsuper, -1);  // a front's assembly items in asm_items
     std::vector<int32_t> trsm_slots, trsm_sbase, slot_of(P.nsuper, -1);
-    std::vector<int32_t> thin_list, thin_asm, thin_slot;
+    std::vector<int32_t> thin_list, thin_slot;
     int32_t nslots = 0;
     // Rank-one leaves: large fronts of one column without children whose parent's
     // assembly takes their entries from l and u (assemble_block) instead of from
@@ -1134,9 +1134,9 @@ int setup_device(ipm_ctx *c) {
             W.bwd_w.flops += 2.0 * (lnz - f);
             W.bwd_w.bytes += 8.0 * lnz + 8.0 * (f + k);
         }
-        // large fronts; the thin ones (one pivot block, f <= kThinMaxF, FP64
-        // updates) of a level that does not take the level kernel run whole,
-        // one CTA each, instead of through the steps
+        // large fronts; many thin leaves (thin_leaf, FP64 updates) of a level that
+        // does not take the level kernel run whole, one CTA each, instead of through
+        // the steps
         W.asm_off = (int64_t)asm_items.size();
         int32_t maxsteps = 0;
         std::vector<int32_t> main_fronts, large;
@@ -1144,18 +1144,15 @@ int setup_device(ipm_ctx *c) {
             if (!rank1[P.lvl_large[t]]) large.push_back(P.lvl_large[t]);
         W.thin_off = (int64_t)thin_list.size();
         auto is_thin = [&](int32_t s) {
-            return P.sn_k[s] <= c->opt.nb && P.sn_f[s] <= kThinMaxF &&
+            return P.child_ptr[s] == P.child_ptr[s + 1] && thin_leaf(P.sn_k[s], P.sn_f[s], c->opt.nb) &&
                    !(c->opt.precision != IPM_PREC_FP64 && P.sn_f[s] >= c->opt.mixed_min_front);
         };
-        int32_t inner = 0, leaves = 0;  // thin fronts with children, without
-        for (int32_t s : large) {
-            inner += is_thin(s) && P.child_ptr[s] < P.child_ptr[s + 1];
-            leaves += is_thin(s) && P.child_ptr[s] == P.child_ptr[s + 1];
-        }
+        int32_t leaves = 0;
+        for (int32_t s : large) leaves += is_thin(s);
         std::vector<std::pair<double, int32_t>> thin;  // work, front
         for (int32_t s : large) {
             add_asm(s);
-            if (is_thin(s) && (P.child_ptr[s] == P.child_ptr[s + 1] ? leaves : inner) >= kThinMin) {
+            if (leaves >= kThinMin && is_thin(s)) {
                 thin.push_back({(double)P.sn_k[s] * P.sn_f[s] * P.sn_f[s], s});
                 const Work fr = front_work(s);
                 W.thin_w.flops += fr.flops;
@@ -1171,7 +1168,6 @@ int setup_device(ipm_ctx *c) {
         });
         for (const auto &e : thin) {
             thin_list.push_back(e.second);
-            thin_asm.push_back((int32_t)first_item[e.second]);
             thin_slot.push_back(slot_of[e.second]);
         }
         W.asm_cnt = (int32_t)(asm_items.size() - W.asm_off);
@@ -1297,8 +1293,8 @@ int setup_device(ipm_ctx *c) {
         }
     }
     c->steps_levels = steps_levels;
-    c->nfronts_thin = (int32_t)(thin_list.size() + rank1_list.size());
     c->rank1_cnt = (int32_t)rank1_list.size();
+    c->nfronts_thin = (int32_t)thin_list.size() + c->rank1_cnt;
     c->rank1_w = Work();
     for (int32_t s : rank1_list) {
         c->rank1_w.flops += P.sn_f[s];
@@ -1339,8 +1335,7 @@ int setup_device(ipm_ctx *c) {
         (rc = dupload(c, &c->tile_items, tile_items)) || (rc = dupload(c, &c->tc_items, tc_items)) ||
         (rc = dupload(c, &c->alt_items, alt_items)) || (rc = dupload(c, &c->bwd_order, bwd_order)) ||
         (rc = dupload(c, &c->trsm_sbase, trsm_sbase)) || (rc = dupload(c, &c->sliced_runs, sliced_runs)) || (rc = dupload(c, &c->sliced_segs, sliced_segs)) ||
-        (rc = dupload(c, &c->thin_list, thin_list)) || (rc = dupload(c, &c->thin_asm, thin_asm)) ||
-        (rc = dupload(c, &c->thin_slot, thin_slot)) || (rc = dupload(c, &c->rank1_list, rank1_list)) ||
+        (rc = dupload(c, &c->thin_list, thin_list)) || (rc = dupload(c, &c->thin_slot, thin_slot)) || (rc = dupload(c, &c->rank1_list, rank1_list)) ||
         (rc = dalloc(c, &c->slice_ws, 3 * (size_t)max_slice_blocks * (size_t)kSliceBlockBytes)) ||
         (rc = dalloc(c, &c->slice_exp, 3 * (size_t)std::max<int64_t>(max_slice_blocks, 1) * kSliceRows * 2)) ||
         (rc = dupload(c, &c->lvl_items, lvl_items)) || (rc = dalloc(c, &c->lvl_sync, (size_t)max_ncnt + 1)) ||
@@ -1825,8 +1820,7 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             if (W.thin_cnt > 0) {
                 Prof pr(c, IPM_K_LARGE_PANEL, W.thin_w, sd);
                 launch_thin_fronts(c->dp, V, c->fronts, c->D, c->Dinv, c->dyn, c->ctl, c->thin_list + W.thin_off,
-                                   c->thin_asm + W.thin_off, c->thin_slot + W.thin_off, c->al,
-                                   c->panel_ws, W.thin_cnt, c->opt.nb, sd);
+                                   c->thin_slot + W.thin_off, c->panel_ws, W.thin_cnt, c->opt.nb, sd);
                 nl++;
             }
             prev_rest = nullptr;
@@ -2719,6 +2713,7 @@ int ipm_get_info(ipm_ctx *c, ipm_info *out) {
     out->steps_levels = c->steps_levels;
     out->steps_dependency = c->steps_dependency;
     out->nfronts_thin = c->nfronts_thin;
+    out->nfronts_rank_one = c->rank1_cnt;
     out->tune_ms = c->tune_ms;
     out->omega = c->omega;
     for (int i = 0; i < 16; i++) out->omega_hist[i] = c->omega_hist[i];

@@ -337,23 +337,33 @@ void launch_large_update_strip(const DevPlan &P, double *fronts, const TileItem 
                                int32_t count, int32_t w, cudaStream_t st);
 constexpr int64_t kLongColumn = 2048;  // longer sums over a sparse row take a CTA each
 constexpr int64_t kWarpRow = 32;       // and longer than this a warp each (rows_common.cuh)
-// thin fronts (k <= nb, f <= kThinMaxF), one CTA per front: list[i] the front,
-// first_asm[i] its first assembly item, slots[i] its panel workspace slot
-constexpr int kThinMaxF = 512;
-// Leaves, and fronts with children, take that path only where a level has this
-// many of them: one CTA does its front block by block (0.5 to 2 ms assembling
-// ten to a hundred children of 300 rows, 0.3 ms for the products of a leaf of 16
-// columns and 360 rows), where the per-step launches spread the blocks over the
-// chip (40 block-angular blocks with 300 dense rows: three levels of 10 to 200
-// fronts with children 5.9 ms as thin fronts, 1.2 through the steps; 614 leaves
-// of 2 to 25 columns 1.59 ms against 1.06).
-constexpr int kThinMin = 1024;
+// Thin leaves: large fronts without children of one pivot block and f <=
+// kThinMaxF rows, whole in one CTA each (k_thin_fronts: list[i] the front,
+// slots[i] its panel workspace slot) where a level has kThinMin of them; fewer
+// leave SMs idle where the steps spread a front's blocks over the chip.  Only
+// up to kThinCols columns, or kThinWide rows: factorisations with 1,024 leaves
+// and 4,000 leaves as thin fronts and through the steps take (ms)
+//   k = 2:  130 dense rows 1.65 / 1.82 and 6.4 / 7.1, 300 rows 2.48 / 2.85 and
+//           9.2 / 10.6, 450 rows 3.06 / 3.55 and 11.1 / 13.2;
+//   k = 4:  1.70 / 1.90 and 6.6 / 7.4, 2.67 / 3.04 and 10.2 / 11.6, 3.47 / 3.97 and
+//           12.7 / 14.8;
+//   k = 9:  2.11 / 2.02 and 7.88 / 7.84, 3.73 / 3.48 and 13.9 / 13.2, 5.3 / 5.0 and
+//           19.7 / 18.7;
+//   k = 32: 2.81 / 2.82 and 9.8 / 10.3, 6.9 / 5.6 and 22.5 / 21.6, 12.4 / 9.7 and
+//           39.0 / 37.0.
+// Fronts with children go through the steps (300 to 2,200 of them per level with 1
+// to 30 columns over 2 to 6 children: whole in a CTA 5% faster to 17% slower;
+// the 981 of a 200-block LP 20.4 against 19.5 for its factorisation).
+constexpr int kThinMaxF = 512, kThinMin = 1024, kThinCols = 4, kThinWide = 224;
+inline bool thin_leaf(int32_t k, int32_t f, int32_t nb) {
+    return k <= nb && f <= kThinMaxF && (k <= kThinCols || f <= kThinWide);
+}
 // rank-one leaves (large fronts of one column without children under a large front)
 void launch_rank_one(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                      DevCtl *ctl, const int32_t *list, int32_t count, cudaStream_t st);
 void launch_thin_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
-                        DevCtl *ctl, const int32_t *list, const int32_t *first_asm, const int32_t *slots,
-                        const AsmLists &A, double *pws, int32_t count, int32_t nb, cudaStream_t st);
+                        DevCtl *ctl, const int32_t *list, const int32_t *slots, double *pws, int32_t count, int32_t nb,
+                        cudaStream_t st);
 void launch_large_level(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
                         DevCtl *ctl, const FactorItem *items, int32_t count, int32_t *sync, int32_t ncounters,
                         const AsmLists &A, double *pws, int32_t nb, int32_t grid, long long spin_limit,

@@ -340,13 +340,13 @@ constexpr int kPoolDoubles = 2 * 32 * 33 + 32;  // a 32 x 32 update tile's two o
 // children's order without CTA barriers, the next child's maps fetched
 // while this one's entries arrive.  50-period staircase: the assembly launches
 // of a factorisation take 5.6 ms instead of 23.7 (10.8 GB).
-template <class Out>  // out(r, c, v): stores the assembled value v of front entry (r, c)
-__device__ __forceinline__ void assemble_block(const DevPlan &P, const DevVals &V, const double *fronts,
-                                               const AsmLists &A, const AsmItem &ai, double *pool, Out out) {
+__device__ __forceinline__ void body_assemble(const DevPlan &P, const DevVals &V, double *fronts, const AsmLists &A,
+                                              const AsmItem &ai, double *pool) {
     constexpr int NT = kBodyThreads, R = kAsmRows;
     static_assert(32 * R <= kPoolDoubles && NT / 32 == 8, "the block fits the pool, four columns per warp");
     double *T = pool;  // column c, row r at T[R (c - c_lo) + r % R]
     const int ld = P.sn_ld[ai.s];
+    double *F = fronts + P.sn_off[ai.s];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int c_lo = ai.c_lo, r_lo = ai.r_lo, r_hi = ai.r_hi, rbase = r_lo & ~(R - 1);
 #pragma unroll
@@ -452,15 +452,8 @@ __device__ __forceinline__ void assemble_block(const DevPlan &P, const DevVals &
     __syncthreads();
     for (int t = tid; t < 32 * R; t += NT) {
         const int c = c_lo + t / R, r = rbase + t % R;
-        if (c < ai.c_hi && r >= r_lo && r < r_hi) out(r, c, T[t]);
+        if (c < ai.c_hi && r >= r_lo && r < r_hi) F[(int64_t)c * ld + r] = T[t];
     }
-}
-
-__device__ __forceinline__ void body_assemble(const DevPlan &P, const DevVals &V, double *__restrict__ fronts,
-                                              const AsmLists &A, const AsmItem &ai, double *pool) {
-    const int ld = P.sn_ld[ai.s];
-    double *F = fronts + P.sn_off[ai.s];
-    assemble_block(P, V, fronts, A, ai, pool, [&](int r, int c, double v) { F[(int64_t)c * ld + r] = v; });
 }
 
 // The nb x nb diagonal block of panel [p0, p0 + nb) of front s as a
@@ -1054,50 +1047,34 @@ __global__ void __launch_bounds__(kRankOneThreads) k_rank_one(DevPlan P, DevVals
     }
 }
 
-// A thin front (one pivot block, k <= nb, f <= kThinMaxF) whole in one CTA.
-// Every entry gets the operations of the per-step path in its order, so the
-// front's values are those of that path bit for bit; what differs is what
-// moves: the rows of L are kept in shared memory, the contribution
-// block is formed and written in one pass (0 minus the products where the front
-// has no children, assembled and updated block by block in shared memory
-// otherwise), and up to kThinCols pivot columns a thread solves a row by
-// itself.  The products of a leaf bound it (FP64, two per clock and SM): 614
-// leaves of 2 to 25 columns and 300 to 376 rows take 1.6 ms (0.5 at the FP64
-// rate), too few to even out over the SMs; hence kThinMin.
-constexpr int kThinCols = 4;
+// A thin leaf (a front without children, one pivot block, f <= kThinMaxF) whole
+// in one CTA.  Every entry gets the operations of the per-step path in its
+// order, so the front's values are those of that path bit for bit; what differs
+// is what moves: the rows of L are kept in shared memory, the contribution block
+// is formed and written in one pass (0 minus the products, where the steps zero
+// it, read it and write it), and up to kThinCols pivot columns a thread solves a
+// row by itself.  Bound by that write for a few columns, by the products
+// (FP64, two per clock and SM) for many; where each side wins: thin_leaf.
 constexpr int kThinPanel = 6144;  // doubles of L kept (three CTAs per SM fit)
 __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevVals V, double *__restrict__ fronts,
                                                                double *__restrict__ Dg, double *__restrict__ Dig,
                                                                double *__restrict__ dyng, DevCtl *ctl,
                                                                const int32_t *__restrict__ list,
-                                                               const int32_t *__restrict__ first_asm,
                                                                const int32_t *__restrict__ slots,
-                                                               AsmLists A, double *__restrict__ pws, int nb) {
+                                                               double *__restrict__ pws, int nb) {
     extern __shared__ double panel[];
     __shared__ double pool[kPoolDoubles];
-    __shared__ double Bt[32][33];  // u(c, q) of a block's columns
     const int s = list[blockIdx.x];
     const int f = P.sn_f[s], k = P.sn_k[s], ld = P.sn_ld[s];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     double *F = fronts + P.sn_off[s];
-    const int64_t a0 = first_asm[blockIdx.x];
-    const bool leaf = P.child_ptr[s] == P.child_ptr[s + 1];
-    const int nr = (f + kAsmRows - 1) / kAsmRows;  // the first column block's items
-    if (leaf) {
-        // originals lie in the pivot columns
-        for (int c = warp; c < k; c += kBodyThreads / 32)
-            for (int r = c + lane; r < f; r += 32) F[(int64_t)c * ld + r] = 0.0;
-        __syncthreads();
-        for (int64_t q = P.orig_ptr[s] + tid; q < P.orig_ptr[s + 1]; q += kBodyThreads)
-            F[P.orig_dst[q]] = orig_value(P, V, P.orig_src[q]);
-        __syncthreads();
-    } else {
-        for (int a = 0; a < nr; a++) {
-            const AsmItem ai = A.items[a0 + a];
-            body_assemble(P, V, fronts, A, ai, pool);
-            __syncthreads();
-        }
-    }
+    // originals lie in the pivot columns
+    for (int c = warp; c < k; c += kBodyThreads / 32)
+        for (int r = c + lane; r < f; r += 32) F[(int64_t)c * ld + r] = 0.0;
+    __syncthreads();
+    for (int64_t q = P.orig_ptr[s] + tid; q < P.orig_ptr[s + 1]; q += kBodyThreads)
+        F[P.orig_dst[q]] = orig_value(P, V, P.orig_src[q]);
+    __syncthreads();
     double *ws = pws + (int64_t)slots[blockIdx.x] * kPanelWs;
     body_diag(P, V, fronts, Dg, Dig, dyng, ctl, s, 0, nb, ws, pool);
     __syncthreads();
@@ -1135,12 +1112,9 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
             for (int i = k + tid; i < f; i += kBodyThreads) panel[q * f + i] = F[(int64_t)q * ld + i];
         __syncthreads();
     }
-    // columns of the contribution block with nothing assembled beside them: all
-    // of a leaf's, else those of the first block (whose values are in the slab)
-    const int c_end = leaf ? f : min(32, f);
-    auto u_of = [&](int j) { return j < c_end && lane < k ? __ldcg(F + (int64_t)j * ld + lane) : 0.0; };
+    auto u_of = [&](int j) { return j < f && lane < k ? __ldcg(F + (int64_t)j * ld + lane) : 0.0; };
     double bn = u_of(k + warp);
-    for (int j = k + warp; j < c_end; j += kBodyThreads / 32) {
+    for (int j = k + warp; j < f; j += kBodyThreads / 32) {
         const double b = bn;
         bn = u_of(j + kBodyThreads / 32);
         constexpr int U = 4;  // rows a lane carries together
@@ -1159,31 +1133,11 @@ __global__ void __launch_bounds__(kBodyThreads, 3) k_thin_fronts(DevPlan P, DevV
 #pragma unroll
             for (int u = 0; u < U; u++) {
                 if (i0 + 32 * u >= f) continue;
-                if (leaf) {
-                    // 0 - acc without an FP64 instruction (0 - 0 is +0)
-                    const long long bits = dbits(acc[u]);
-                    e[32 * u] = (bits & kAbsMask) ? __longlong_as_double(bits ^ kSignBit) : 0.0;
-                } else {
-                    e[32 * u] = e[32 * u] - acc[u];
-                }
+                // 0 - acc without an FP64 instruction (0 - 0 is +0)
+                const long long bits = dbits(acc[u]);
+                e[32 * u] = (bits & kAbsMask) ? __longlong_as_double(bits ^ kSignBit) : 0.0;
             }
         }
-    }
-    if (leaf) return;
-    for (int a = nr, na = asm_tiles(f); a < na; a++) {
-        const AsmItem ai = A.items[a0 + a];
-        __syncthreads();
-        for (int t = tid; t < 32 * 32; t += kBodyThreads) {
-            const int q = t & 31, c = ai.c_lo + (t >> 5);
-            if (q < k) Bt[t >> 5][q] = c < f ? __ldcg(F + (int64_t)c * ld + q) : 0.0;
-        }
-        assemble_block(P, V, fronts, A, ai, pool, [&](int r, int c, double v) {
-            if (r < c) return;
-            const double *b = Bt[c - ai.c_lo];
-            double acc = 0.0;
-            for (int q = 0; q < k; q++) acc += Lp[q * ls + r] * b[q];
-            F[(int64_t)c * ld + r] = v - acc;
-        });
     }
 }
 
@@ -1683,14 +1637,14 @@ void launch_rank_one(const DevPlan &P, const DevVals &V, double *fronts, double 
 }
 
 void launch_thin_fronts(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
-                        DevCtl *ctl, const int32_t *list, const int32_t *first_asm, const int32_t *slots,
-                        const AsmLists &A, double *pws, int32_t count, int32_t nb, cudaStream_t st) {
+                        DevCtl *ctl, const int32_t *list, const int32_t *slots, double *pws, int32_t count, int32_t nb,
+                        cudaStream_t st) {
     if (count <= 0) return;
     static uint64_t attr = 0;
     constexpr int smem = kThinPanel * (int)sizeof(double);
     if (first_on_device(attr))
         cudaFuncSetAttribute(k_thin_fronts, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    k_thin_fronts<<<count, kBodyThreads, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, first_asm, slots, A, pws, nb);
+    k_thin_fronts<<<count, kBodyThreads, smem, st>>>(P, V, fronts, D, Dinv, dyn, ctl, list, slots, pws, nb);
 }
 
 void launch_large_level(const DevPlan &P, const DevVals &V, double *fronts, double *D, double *Dinv, double *dyn,
