@@ -16,6 +16,7 @@
 #include "../../include/ipm_mf.h"
 #include "ipm_dev.h"
 #include "ipm_plan.h"
+#include "point_lists.h"
 
 using namespace ipm;
 
@@ -282,14 +283,18 @@ int dalloc(ipm_ctx *c, T **p, size_t count) {
 }
 
 template <typename T>
-int dupload(ipm_ctx *c, T **p, const std::vector<T> &h) {
-    int rc = dalloc(c, p, h.size());
+int dupload(ipm_ctx *c, T **p, const T *h, size_t count) {
+    int rc = dalloc(c, p, count);
     if (rc) return rc;
-    if (!h.empty()) {
-        cudaError_t e = cudaMemcpy(*p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
+    if (count > 0) {
+        cudaError_t e = cudaMemcpy(*p, h, count * sizeof(T), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) return to_err(e);
     }
     return IPM_OK;
+}
+template <typename T>
+int dupload(ipm_ctx *c, T **p, const std::vector<T> &h) {
+    return dupload(c, p, h.data(), h.size());
 }
 
 // The rows of a CSR pointer summed by a CTA each (more than kLongColumn
@@ -776,8 +781,7 @@ int setup_device(ipm_ctx *c) {
     std::vector<PanelItem> panel_items, trsm_items;
     std::vector<AsmItem> asm_items;
     std::vector<AsmChild> asm_child;
-    std::vector<int32_t> seg_dst, asm_rt;
-    std::vector<int64_t> seg_ptr(1, 0), seg_src;
+    std::vector<int32_t> asm_rt;
     std::vector<int64_t> first_item(P.nsuper, -1);  // a front's assembly items in asm_items
     std::vector<int32_t> trsm_slots, trsm_sbase, slot_of(P.nsuper, -1);
     std::vector<int32_t> thin_list, thin_slot;
@@ -824,27 +828,12 @@ int setup_device(ipm_ctx *c) {
         }
         return fr;
     };
+    // the lists of small children's entries (the pivoting mode has no use for them)
+    PointLists points;
+    if (!c->opt.pivoting) build_point_lists(P, points);
     // The assembly items of large front s, one per 32 columns x kAsmRows rows of
-    // its lower part, appended to asm_items (the terms' lists are built once
+    // its lower part, appended to asm_items (the children's ranges are found once
     // per front; a front's items may be appended again).
-    using Points = std::vector<std::pair<int32_t, int64_t>>;  // destination, arena position; children ascending
-    auto add_segments = [&](Points &pt, int64_t &seg0, int64_t &seg1) {
-        std::stable_sort(pt.begin(), pt.end(),
-                         [](const std::pair<int32_t, int64_t> &x, const std::pair<int32_t, int64_t> &y) {
-                             return x.first < y.first;
-                         });
-        seg0 = (int64_t)seg_dst.size();
-        for (size_t u = 0; u < pt.size(); u++) {
-            if (u == 0 || pt[u].first != pt[u - 1].first) {
-                if (u > 0) seg_ptr.push_back((int64_t)seg_src.size());
-                seg_dst.push_back(pt[u].first);
-            }
-            seg_src.push_back(pt[u].second);
-        }
-        if (!pt.empty()) seg_ptr.push_back((int64_t)seg_src.size());
-        seg1 = (int64_t)seg_dst.size();
-    };
-    std::vector<Points> points;                                    // per item
     std::vector<std::vector<AsmChild>> block_child, block_rank1;   // per column block
     auto add_asm = [&](int32_t s) {
         const int32_t ld = P.sn_ld[s], f = P.sn_f[s], ntile = asm_tiles(f), nblk = (f + 31) / 32;
@@ -856,27 +845,13 @@ int setup_device(ipm_ctx *c) {
             return;
         }
         first_item[s] = (int64_t)asm_items.size();
-        if ((int32_t)points.size() < ntile) points.resize(ntile);
         if ((int32_t)block_child.size() < nblk) block_child.resize(nblk), block_rank1.resize(nblk);
-        std::vector<int32_t> first_tile(nblk);  // item of the block's first rows
-        for (int32_t cb = 0, t = 0; cb < nblk; cb++) {
-            first_tile[cb] = t;
-            t += (f + kAsmRows - 1) / kAsmRows - 32 * cb / kAsmRows;
-        }
-        for (int32_t t = 0; t < ntile; t++) points[t].clear();
         for (int32_t cb = 0; cb < nblk; cb++) block_child[cb].clear(), block_rank1[cb].clear();
         for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
             const int32_t ch = P.child_list[q], kc = P.sn_k[ch], cc = P.sn_f[ch] - kc, ldc = P.sn_ld[ch];
             const int32_t *m = P.relmap.data() + P.map_off[ch];
             const int64_t cb0 = P.sn_off[ch] + (int64_t)kc * ldc + kc;
-            if (cc <= kPointRows) {
-                for (int32_t jj = 0; jj < cc; jj++)
-                    for (int32_t ii = jj; ii < cc; ii++) {
-                        const int32_t cb = m[jj] / 32, t = first_tile[cb] + m[ii] / kAsmRows - 32 * cb / kAsmRows;
-                        points[t].push_back({kAsmRows * (m[jj] % 32) + m[ii] % kAsmRows, cb0 + (int64_t)jj * ldc + ii});
-                    }
-                continue;
-            }
+            if (cc <= kPointRows) continue;
             const int32_t rt = (int32_t)asm_rt.size();
             for (int32_t r = 0; r < f + kAsmRows; r += kAsmRows)
                 asm_rt.push_back((int32_t)(std::lower_bound(m, m + cc, r) - m));
@@ -903,7 +878,8 @@ int setup_device(ipm_ctx *c) {
             for (int32_t rb = 32 * cb / kAsmRows; rb * kAsmRows < f; rb++, t++) {
                 ai.r_lo = std::max(rb * kAsmRows, ai.c_lo);
                 ai.r_hi = std::min((rb + 1) * kAsmRows, f);
-                add_segments(points[t], ai.seg0, ai.seg1);
+                ai.seg0 = points.seg.empty() ? 0 : points.seg[points.first[s] + t];
+                ai.seg1 = points.seg.empty() ? 0 : points.seg[points.first[s] + t + 1];
                 asm_items.push_back(ai);
             }
         }
@@ -911,24 +887,13 @@ int setup_device(ipm_ctx *c) {
     // the small fronts' lists
     std::vector<int64_t> small_seg(2 * (size_t)P.nsuper, 0);
     std::vector<int32_t> small_big(P.nsuper, 0);
-    if (!c->opt.pivoting) {
-        Points pt;
-        for (int32_t s = 0; s < P.nsuper; s++) {
-            if (P.sn_large[s]) continue;
-            pt.clear();
-            small_big[s] = P.child_ptr[s];
-            for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++) {
-                const int32_t ch = P.child_list[q], kc = P.sn_k[ch], cc = P.sn_f[ch] - kc, ldc = P.sn_ld[ch];
-                if (cc > kPointRows) continue;
-                small_big[s]++;
-                const int32_t *m = P.relmap.data() + P.map_off[ch];
-                const int64_t cb0 = P.sn_off[ch] + (int64_t)kc * ldc + kc;
-                for (int32_t jj = 0; jj < cc; jj++)
-                    for (int32_t ii = jj; ii < cc; ii++)
-                        pt.push_back({m[jj] * P.sn_ld[s] + m[ii], cb0 + (int64_t)jj * ldc + ii});
-            }
-            add_segments(pt, small_seg[2 * (size_t)s], small_seg[2 * (size_t)s + 1]);
-        }
+    for (int32_t s = 0; s < P.nsuper && !c->opt.pivoting; s++) {
+        if (P.sn_large[s]) continue;
+        small_seg[2 * (size_t)s] = points.seg[points.first[s]];
+        small_seg[2 * (size_t)s + 1] = points.seg[points.first[s] + 1];
+        small_big[s] = P.child_ptr[s];
+        for (int32_t q = P.child_ptr[s]; q < P.child_ptr[s + 1]; q++)
+            small_big[s] += P.sn_f[P.child_list[q]] - P.sn_k[P.child_list[q]] <= kPointRows;
     }
     // One step of the large-front path: for each (front s, panel start p0)
     // of fp, the diagonal block of the panel, the triangular solve of the rows
@@ -1325,8 +1290,9 @@ int setup_device(ipm_ctx *c) {
         (rc = dupload(c, &d_perm, P.perm)) || (rc = dupload(c, &d_uoff, upd_off)) || (rc = dupload(c, &d_kp, kp)) ||
         (rc = dupload(c, &d_kj, kj)) || (rc = dupload(c, &d_ksrc, ksrc)) ||
         (rc = dupload(c, &c->lvl_small, small_lists)) || (rc = dupload(c, &c->lvl_all, lvl_all)) ||
-        (rc = dupload(c, (AsmItem **)&c->al.items, asm_items)) || (rc = dupload(c, (int32_t **)&c->al.seg_dst, seg_dst)) ||
-        (rc = dupload(c, (int64_t **)&c->al.seg_ptr, seg_ptr)) || (rc = dupload(c, (int64_t **)&c->al.src, seg_src)) ||
+        (rc = dupload(c, (AsmItem **)&c->al.items, asm_items)) || (rc = dupload(c, (int32_t **)&c->al.seg_dst, points.dst.get(), points.ndst)) ||
+        (rc = dupload(c, (int64_t **)&c->al.seg_ptr, points.ptr.get(), points.ptr ? points.ndst + 1 : 0)) ||
+        (rc = dupload(c, (int64_t **)&c->al.src, points.src.get(), points.nsrc)) ||
         (rc = dupload(c, (AsmChild **)&c->al.child, asm_child)) || (rc = dupload(c, (int32_t **)&c->al.rt, asm_rt)) ||
         (rc = dupload(c, (int64_t **)&c->al.small, small_seg)) || (rc = dupload(c, (int32_t **)&c->al.small_big, small_big)) ||
         (rc = dupload(c, &c->panel_items, panel_items)) ||

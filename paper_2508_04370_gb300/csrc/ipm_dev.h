@@ -5,6 +5,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "point_lists.h"
+
 namespace ipm {
 
 // Status bits written by kernels (never traps): OR-ed into DevCtl::status.
@@ -210,16 +212,10 @@ struct PanelItem {
 // of arena positions per destination, [seg0, seg1) of AsmLists; the large
 // children [ch0, ch1); the rank-one leaves [ch1, ch2).  Device child lists hold the small children before the
 // large ones, so every path adds in this order.
-constexpr int kAsmRows = 64;
-constexpr int kPointRows = 64;
 struct AsmItem {
     int64_t o0, o1, seg0, seg1;
     int32_t ch0, ch1, ch2, s, c_lo, c_hi, r_lo, r_hi;
 };
-__host__ __device__ inline int32_t asm_tiles(int32_t f) {  // items of a front of f rows
-    const int32_t nc = (f + 31) / 32, nr = (f + kAsmRows - 1) / kAsmRows;
-    return nc * nr - (nc - 1) * (nc - 1) / 4;  // block column i starts at block row i / 2
-}
 // A large child's part in a block of columns: its columns [a, b) land there;
 // rt + i is where its rows of the front's i-th block of kAsmRows rows begin.
 // (Of a rank-one leaf cb is its column of L, row 1 first, and cb + ldc the
