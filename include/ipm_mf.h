@@ -378,7 +378,8 @@ int ipm_solve_noalloc(ipm_ctx *ctx, const double *r7_dev, const double *r1_dev, 
  *   - the level-kernel threshold: a tree level runs its large fronts in one
  *     persistent launch when their FP64 work at 1 TFLOP/s is below ratio x
  *     (35 us per 32-column panel of its widest front); candidates 0 (never),
- *     0.25, 0.5, 1 (default), 2, 1e30 (always);
+ *     0.25, 0.5, 1 (default; 0.65 on levels with sliced updates in use), 2,
+ *     1e30 (always); a set or tuned ratio holds on every level;
  *   - the threads per small-front CTA of each size class present: by each
  *     launch's number of fronts (default, see ipm_set_launch_shapes), or one
  *     width for the class (f <= 32: 32 or 64; f <= 64: 64 or 128; f <= 128:

@@ -53,6 +53,7 @@ struct SmallClass {
     int32_t cls;  // size class: f <= 32, <= 64, <= 128
     Work w;
 };
+constexpr double kSlicedLevelRatio = 0.65;
 struct LevelWork {
     std::vector<SmallClass> small;  // small fronts of the level by size class
     int64_t all_off;
@@ -72,10 +73,14 @@ struct LevelWork {
     bool has_tc = false;   // some front of the level has tensor-core update tiles
     // The level kernel pays off where a level's large fronts are bound by
     // their pivot chains (about 35 us per 32-column panel): a level takes it
-    // when its FP64 front work at ~1 TFLOP/s is below tune_ratio times its
-    // longest chain (1 unless ipm_autotune chose otherwise: a random 1537 x 3843
-    // LP's root level of 0.73 GFLOP and 41 panels takes 1.92 ms with it and 2.42
-    // by steps).  Levels with more work run one launch per step at full occupancy.
+    // when its FP64 front work at ~1 TFLOP/s is below a ratio times its longest
+    // chain.  Levels with more work run one launch per step at full occupancy.
+    // The ratio is 1 unless tuned or set (factorisations of random LPs, level kernel
+    // against steps: m = 1537 1.85 ms against 2.05, 1800 2.45 / 2.65, 2100 3.28 / 3.40;
+    // 2300 stays with the steps' 3.97, with 3xTF32 updates m = 1537 1.84 / 3.4 and 2100
+    // 3.3 / 4.7), and kSlicedLevelRatio on levels with sliced updates in use, where
+    // the steps have the tensor cores (m = 1537 1.84 / 2.00, 1650 2.03 / 2.07, 1700
+    // 2.21 / 2.19, 1750 2.29 / 2.22, 2100 3.27 / 2.82).
     int32_t lvl_chain = 0;  // 32-column panels of the level's widest large front
     Work lvl_w;             // algorithmic work of the level's large fronts (assembly and factorisation)
 };
@@ -149,7 +154,7 @@ struct ipm_ctx {
     // sub-partition's FP64 pipe to one CTA's pivot chain; two keep more
     // trailing tiles in flight.
     int32_t tune_threads[3] = {0, 0, 0};
-    double tune_ratio = 1.0;
+    double tune_ratio = -1.0;  // < 0: the default (see LevelWork::lvl_chain)
     int32_t tune_lvl_per_sm = 0;
     double tune_ms = 0.0;
     bool mixed_active = false;  // tensor-core updates in use (mixed precision, no fallback yet)
@@ -306,6 +311,12 @@ void long_rows(const V &ptr, std::vector<int32_t> &lng, std::vector<int32_t> &mi
         if (len > kLongColumn) lng.push_back((int32_t)i);
         else if (len > kWarpRow) mid.push_back((int32_t)i);
     }
+}
+
+// The default level-kernel ratio of levels with tensor-core updates.
+double default_level_ratio(const ipm_ctx *c) {
+    const bool sliced = c->opt.precision == IPM_PREC_SLICED && (c->mixed_active || !c->dev_ready);
+    return sliced ? kSlicedLevelRatio : 1.0;
 }
 
 // Items of the persistent level kernel for the large fronts of a level, in
@@ -1761,10 +1772,10 @@ int factorise_enqueue(ipm_ctx *c, const double *theta, double rho, double delta,
             }
             if (W.asm_cnt == 0 && W.steps.empty() && W.thin_cnt == 0) continue;
             if (small_before) cudaStreamWaitEvent(sd, small_before, 0);
-            const bool latency_bound = W.lvl_w.flops / 1.0e12 < c->tune_ratio * W.lvl_chain * 35e-6;
             // (a latency-bound level keeps the FP64 level kernel in the tensor-core
             // modes too: its work is too small for the tensor cores to matter)
-            if (c->opt.level_kernel && W.lvl_cnt > 0 && latency_bound) {
+            const double ratio = c->tune_ratio >= 0.0 ? c->tune_ratio : W.has_tc ? default_level_ratio(c) : 1.0;
+            if (c->opt.level_kernel && W.lvl_cnt > 0 && W.lvl_w.flops / 1.0e12 < ratio * W.lvl_chain * 35e-6) {
                 // FP64: all large-front work of the level in one dependency-driven launch
                 {
                     Prof pr(c, IPM_K_LARGE_PANEL, W.lvl_w, sd);
@@ -2314,7 +2325,7 @@ int ipm_autotune(ipm_ctx *c, const double *theta_dev, double rho, double delta, 
         const double r0 = c->tune_ratio;
         double pick = r0;
         for (double r : ratios) {
-            if (r == r0) continue;
+            if (r == (r0 >= 0.0 ? r0 : default_level_ratio(c))) continue;
             c->tune_ratio = r;
             double ms;
             if ((rc = measure(ms))) goto done;
@@ -2672,7 +2683,7 @@ int ipm_get_info(ipm_ctx *c, ipm_info *out) {
         out->tune_small_by_count[b] = c->tune_threads[b] == 0;
         out->tune_small_threads[b] = c->tune_threads[b] > 0 ? c->tune_threads[b] : kSmallBaseWidth[b];
     }
-    out->tune_level_ratio = c->tune_ratio;
+    out->tune_level_ratio = c->tune_ratio >= 0.0 ? c->tune_ratio : default_level_ratio(c);
     out->tune_level_ctas_per_sm = c->dev_ready ? level_grid(c) / c->sms : 0;
     out->graph_kernels = c->graph_kernels;
     out->schedule = c->dep_sched ? IPM_SCHED_DEPENDENCY : IPM_SCHED_LEVELS;
