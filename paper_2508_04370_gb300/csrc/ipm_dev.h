@@ -53,7 +53,6 @@ struct DevCtl {
     double dinf;           // ||d||_inf of the current iterate (as ordered bits >= 0)
     int32_t done;          // refinement finished
     int32_t steps;
-    int32_t improved;      // the last step improved omega_best
     double omega_hist[16];
     int32_t gmres_iters;   // GMRES iterations of a graph-resident refinement
     int32_t best;          // graph-resident refinement: which of its two iterates is the best

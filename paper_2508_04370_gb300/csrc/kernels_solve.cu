@@ -1181,14 +1181,12 @@ __global__ void k_refine_init(DevCtl *ctl, double target, int max_steps) {
     ctl->omega_hist[0] = w;
     ctl->steps = 0;
     ctl->gmres_iters = 0;
-    ctl->improved = 1;
     ctl->best = 0;
     ctl->done = (w <= target || max_steps <= 0) ? 1 : 0;
 }
 
 __global__ void k_refine_step(DevCtl *ctl, double target, int step, int max_steps, unsigned long long handle) {
     if (ctl->done) {
-        ctl->improved = 0;
         if (handle) cudaGraphSetConditional((cudaGraphConditionalHandle)handle, 0);
         return;
     }
@@ -1196,8 +1194,7 @@ __global__ void k_refine_step(DevCtl *ctl, double target, int step, int max_step
     ctl->steps = step;
     if (step < 16) ctl->omega_hist[step] = w;
     const bool halved = w <= 0.5 * ctl->omega_best;
-    ctl->improved = w < ctl->omega_best ? 1 : 0;
-    if (ctl->improved) {
+    if (w < ctl->omega_best) {
         ctl->omega_best = w;
         ctl->best = step & 1;
     }
