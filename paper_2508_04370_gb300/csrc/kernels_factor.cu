@@ -5,10 +5,17 @@
 // ld) in one device arena.  After its factorisation the first k columns hold
 // L (strictly lower part; D on the diagonal) and the trailing (f-k) x (f-k)
 // lower block holds the contribution block (Schur complement) that the
-// parent pulls during its own assembly (the strict upper part of a small
-// front's slab holds scratch and is never read).  Children are always summed
-// in ascending order, original entries first, so results do not depend on
-// scheduling (Sec. 4.3, determinism).
+// parent pulls during its own assembly.  The strict upper part of a small
+// front's slab holds scratch and is never read; that of a large front holds, for
+// each row i below a panel, u_iq = l_iq d_q at (row q, column i), the FP64 updates'
+// second operand (written by the triangular solve, read by no one after the
+// panel's update).  A rank-one leaf holds -u in its second column instead of a
+// contribution block.
+//
+// A front's entries are summed in one order whatever the schedule: the original
+// entry, the children of up to kPointRows contribution rows ascending, the
+// larger ones ascending, the rank-one leaves ascending (Sec. 4.3, determinism).
+// The pivoting mode's fronts take all children ascending.
 //
 // Kernels: k_small_fronts (a whole front of f <= 128 in shared memory, one
 // CTA per front); the large-front bodies (assembly, diagonal block,

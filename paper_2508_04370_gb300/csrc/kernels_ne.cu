@@ -3,8 +3,10 @@
 //   Theta~ = (Theta^-1 + rho I)^-1
 //   M      = A Theta~ A^T            (formed every iteration; delta enters at the pivot)
 //   r8     = r1 + A Theta~ r7,   M_reg dy = r8,   dx = Theta~ (A^T dy - r7).
-// Formation is deterministic: every lower entry (r, i) of M sums its own
-// contributor pairs a_rj Theta~_j a_ij in ascending column j (no atomics).
+// Formation is deterministic (no atomics): every lower entry (r, i) of M sums its
+// own contributor pairs a_rj Theta~_j a_ij, up to kWarpRow of them in ascending
+// column j, more of them strided over the lanes of a warp or a CTA and the lanes'
+// sums in a fixed tree (rows_common.cuh).
 #include <cuda_runtime.h>
 
 #include <cstdint>

@@ -27,8 +27,8 @@
 //     (|x_0| <= 128), each exactly a bf16.  The digits go to a work space in
 //     the 128-byte-swizzled K-major image the tensor cores read, one image
 //     set per chunk.
-//  2. k_update_sliced: a CTA takes a run of 128 x 32 output tiles of one row
-//     block; the row block's digit images arrive once by bulk copies (TMA) and
+//  2. k_update_sliced: a CTA takes runs of 128 x 32 output tiles, each run in one
+//     row block, whose digit images arrive once by bulk copies (TMA), and
 //     the column tiles' images through two stages; one thread issues, per
 //     slice t of the rows, one tcgen05.mma.kind::f16 (K = 16) against the
 //     column slices u = 0 .. 7 - t side by side (N = 32 (8 - t)), which adds the
@@ -37,14 +37,15 @@
 //     given d at most two products involve x_0 or y_0 (up to 128 x 64) and
 //     the others are at most 64 x 64, so |S_d| <= 40960 K <= 2^21.4 for
 //     K <= 64 and FP32 accumulation is exact.  The epilogue forms
-//     hi = sum_{d<4} S_d 2^(7 (3 - d)) and lo = sum_{d>=4} S_d 2^(7 (7 - d))
-//     exactly in integers, the product
-//     sum_q a_iq b_jq ~= 2^(E_i + E_j - 63) (hi 2^28 + lo)
+//     T = sum_d S_d 2^(7 (7 - d)) in 64-bit integers without its low 8 bits
+//     (digit_sum.h), the product
+//     sum_q a_iq b_jq ~= 2^(E_i + E_j - 63) T
 //     as a double built from the integer's bits (one rounding), and
 //     subtracts it from the FP64 entry: one FP64 instruction per entry.
 // Error per entry: operand rounding 2^-57 and the dropped digit products
 // (t + u >= 8) below 2^-55, relative to 2^(E_i + E_j) per column of the
-// chunks, that is about 2^-52 sqrt(max_q L_iq^2 |d_q| max_q L_jq^2 |d_q|);
+// chunks, and the low bits of T, below 2^-55 once: about
+// 2^-52 sqrt(max_q L_iq^2 |d_q| max_q L_jq^2 |d_q|) together;
 // FP64 GEMM's is 2^-53 of each |L_iq d_q L_jq|, summed.  Without the
 // balancing a panel mixing pivots of size delta and of size 1/delta pairs
 // the largest a of one column with the largest b of another, and the
