@@ -863,14 +863,14 @@ int setup_device(ipm_ctx *c) {
             const int32_t *m = P.relmap.data() + P.map_off[ch];
             const int64_t cb0 = P.sn_off[ch] + (int64_t)kc * ldc + kc;
             if (cc <= kPointRows) continue;
-            const int32_t rt = (int32_t)asm_rt.size();
+            const int64_t rt = (int64_t)asm_rt.size();
             for (int32_t r = 0; r < f + kAsmRows; r += kAsmRows)
                 asm_rt.push_back((int32_t)(std::lower_bound(m, m + cc, r) - m));
             for (int32_t a = 0, b; a < cc; a = b) {
                 const int32_t cb = m[a] / 32;
                 for (b = a; b < cc && m[b] / 32 == cb; b++) {}
-                if (rank1[ch]) block_rank1[cb].push_back({P.sn_off[ch] + 1, P.map_off[ch], ldc, a, b, rt});
-                else block_child[cb].push_back({cb0, P.map_off[ch], ldc, a, b, rt});
+                if (rank1[ch]) block_rank1[cb].push_back(asm_child_of(P.sn_off[ch] + 1, P.map_off[ch], ldc, a, b - a, rt));
+                else block_child[cb].push_back(asm_child_of(cb0, P.map_off[ch], ldc, a, b - a, rt));
             }
         }
         const int32_t *d0 = P.orig_dst.data() + P.orig_ptr[s], *d1 = P.orig_dst.data() + P.orig_ptr[s + 1];

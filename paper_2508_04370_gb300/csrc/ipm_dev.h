@@ -215,14 +215,6 @@ struct AsmItem {
     int64_t o0, o1, seg0, seg1;
     int32_t ch0, ch1, ch2, s, c_lo, c_hi, r_lo, r_hi;
 };
-// A large child's part in a block of columns: its columns [a, b) land there;
-// rt + i is where its rows of the front's i-th block of kAsmRows rows begin.
-// (Of a rank-one leaf cb is its column of L, row 1 first, and cb + ldc the
-// column -u, u = L d: entry (i, j) of its contribution is l_i (-u_j).)
-struct AsmChild {
-    int64_t cb, map;  // its contribution block in the arena, its row map
-    int32_t ldc, a, b, rt;
-};
 struct AsmLists {
     const AsmItem *items;
     const int32_t *seg_dst;  // destination within the item: 64 (column - c_lo) + row % 64

@@ -379,8 +379,9 @@ __device__ __forceinline__ void body_assemble(const DevPlan &P, const DevVals &V
         m.cb = C.cb;
         m.ldc = C.ldc;
         m.a = C.a;
-        m.col = C.a + lane < C.b ? __ldg(P.relmap + C.map + C.a + lane) - c_lo : -1;
-        const int ilo = A.rt[C.rt + rbase / R], ihi = A.rt[C.rt + rbase / R + 1];
+        m.col = lane < C.n() ? __ldg(P.relmap + C.map + C.a + lane) - c_lo : -1;
+        const int32_t *rt = A.rt + C.rt() + rbase / R;
+        const int ilo = rt[0], ihi = rt[1];
         m.i0 = ilo + lane;
         m.r0 = m.i0 < ihi ? __ldg(P.relmap + C.map + m.i0) - rbase : -1;
         m.r1 = m.i0 + 32 < ihi ? __ldg(P.relmap + C.map + m.i0 + 32) - rbase : -1;
@@ -424,11 +425,12 @@ __device__ __forceinline__ void body_assemble(const DevPlan &P, const DevVals &V
     auto leaf = [&](int q) {
         const AsmChild C = A.child[min(q, ai.ch2 - 1)];
         Rank1 m;
-        const int ilo = A.rt[C.rt + rbase / R], ihi = A.rt[C.rt + rbase / R + 1];
+        const int32_t *rt = A.rt + C.rt() + rbase / R;
+        const int ilo = rt[0], ihi = rt[1];
         const int32_t *map = P.relmap + C.map;
         const double *L = fronts + C.cb;
         m.a = C.a;
-        const bool in = C.a + lane < C.b;
+        const bool in = lane < C.n();
         m.col = in ? __ldg(map + C.a + lane) - c_lo : -1;
         m.nu = in ? __ldcg(L + C.ldc + C.a + lane) : 0.0;
         m.i0 = ilo + lane;

@@ -88,6 +88,12 @@ static int check(const Plan &P, const PointLists &L) {
 }
 
 int main() {
+    // a child's place in a list of row blocks beyond 2^31
+    for (int64_t rt : {int64_t(0), int64_t(1) << 31, (int64_t(1) << 40) + 5})
+        for (int n : {1, 31, 32}) {
+            const AsmChild c = asm_child_of(int64_t(1) << 35, int64_t(1) << 34, 200000, 100000, n, rt);
+            if (c.rt() != rt || c.n() != n || c.a != 100000 || c.ldc != 200000) return 3;
+        }
     std::mt19937 g(1);
     for (int round = 0; round < 20; round++) {
         std::vector<std::pair<int, bool>> parents;
